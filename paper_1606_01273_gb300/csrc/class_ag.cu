@@ -489,14 +489,15 @@ __global__ void k_sector(const double* __restrict__ in, int m, int n, double sgn
 }
 
 // Eigenvalues ascending: the kept overlap directions are the last nk columns.
-// X[i][c] = Q[i][m - nk + c] / sqrt(s[m - nk + c])   (m x nk, row-major)
-__global__ void k_range_basis(const double* __restrict__ Q, const double* __restrict__ s, int m,
-                              int nk, double* __restrict__ X) {
+// X[i][c] = Q[i * ldq + qoff + c] / sqrt(s[m - nk + c])   (m x nk, row-major)
+__global__ void k_range_basis(const double* __restrict__ Q, int ldq, int qoff,
+                              const double* __restrict__ s, int m, int nk,
+                              double* __restrict__ X) {
   const long total = (long)m * nk;
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
-    const int i = e / nk, c = e % nk, k = m - nk + c;
-    X[e] = Q[(long)i * m + k] / sqrt(s[k]);
+    const int i = e / nk, c = e % nk;
+    X[e] = Q[(long)i * ldq + qoff + c] / sqrt(s[m - nk + c]);
   }
 }
 
@@ -1297,19 +1298,16 @@ int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double 
       SectorKeep& K = w.keep[sec * nsel + is];
       K.nk = 0;
       OzWork* ozn = (oz && oz->on && oz->S >= kOzMaxSlices) ? oz : nullptr;
-      int st = sym_eig(sw.Ssec, msec, sw.s, sw.Qs, sw.jac, s, tm, ozn);
+      // eigenvalues of the overlap and the eigenvectors of those at or above the threshold
+      int nk = 0, ldq = 0, qoff = 0;
+      int st = sym_eig_above(sw.Ssec, msec, thresh, sw.s, sw.Qs, &nk, &ldq, &qoff, sw.jac, s, tm,
+                             ozn);
       if (st != CASPT2_OK) return st;
-      // number of overlap eigenvalues at or above the threshold (ascending order)
-      std::vector<double> hs(msec);
-      CASPT2_CUDA_TRY(cudaMemcpyAsync(hs.data(), sw.s, sizeof(double) * msec,
-                                      cudaMemcpyDeviceToHost, s));
-      CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
-      int nk = 0;
-      for (int k = 0; k < msec; ++k) nk += hs[k] >= thresh ? 1 : 0;
       if (nk == 0) continue;
       K.nk = nk;
       ++launch_counter();
-      k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, sw.s, msec, nk, sw.X);
+      k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, ldq, qoff, sw.s, msec,
+                                                                   nk, sw.X);
       CASPT2_CUDA_TRY(cudaGetLastError());
       const bool ozx = oz && oz->on && oz->S >= kOzMaxSlices && msec >= kOzTransformMin;
       if (ozx) {

@@ -716,10 +716,10 @@ __device__ __forceinline__ double hash_unit(unsigned a, unsigned b) {
   return (double)(h & 0xFFFFFF) / 16777216.0 + 0.5;   // in [0.5, 1.5)
 }
 
-// Inverse iteration for eigenvalue j (thread j).  Scratch arrays are laid out
-// [i][j] so that threads access consecutive addresses.  Z[i][j] = component i of vector j.
+// Inverse iteration for the nc eigenvalues w[0..nc) (thread j).  Scratch arrays are laid
+// out [i][j] so that threads access consecutive addresses.  Z[i][j] = component i of vector j.
 __global__ void k_inviter(const double* __restrict__ dg, const double* __restrict__ eg,
-                          const double* __restrict__ w, int m, double tnorm,
+                          const double* __restrict__ w, int m, int nc, double tnorm,
                           double* __restrict__ u0, double* __restrict__ u1,
                           double* __restrict__ u2, double* __restrict__ lm,
                           double* __restrict__ pv, double* __restrict__ Z) {
@@ -732,10 +732,10 @@ __global__ void k_inviter(const double* __restrict__ dg, const double* __restric
   const double* d = sde;
   const double* e = sde + m;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m) return;
+  if (j >= nc) return;
   const double lam = w[j];
   const double tiny = 2.2e-16 * (tnorm > 0 ? tnorm : 1.0);
-#define IX(i) ((long)(i) * m + j)
+#define IX(i) ((long)(i) * nc + j)
   // Factor T - lam I = P L U (U with two superdiagonals), the current row carried in
   // registers; rows are final once passed, so their pivots are stored as reciprocals
   // (|pivot| raised to tiny) and the solves below multiply.
@@ -851,14 +851,12 @@ __global__ void k_inviter(const double* __restrict__ dg, const double* __restric
 #undef IX
 }
 
-// Modified Gram-Schmidt inside each cluster of (numerically) equal eigenvalues.
-// One block per eigenvalue index; only cluster starts do work.
 // Orthonormalise each cluster of close eigenvalues (w sorted): the block of the cluster's
 // first index takes the cluster's columns, in shared memory when they fit (else in place
 // in Z), and applies classical Gram-Schmidt twice per vector (each pass projects the
-// vector on all earlier cluster vectors at once), then normalises it.
+// vector on all earlier cluster vectors at once), then normalises it.  Z is m x nc.
 __global__ void __launch_bounds__(256)
-k_cluster_cgs2(const double* __restrict__ w, int m, double tol, int smem_bytes,
+k_cluster_cgs2(const double* __restrict__ w, int m, int nc, double tol, int smem_bytes,
                double* __restrict__ Z) {
   extern __shared__ double cs[];
   __shared__ double part[8][33];
@@ -866,18 +864,18 @@ k_cluster_cgs2(const double* __restrict__ w, int m, double tol, int smem_bytes,
   __shared__ double sc;
   const int j0 = blockIdx.x;
   if (j0 > 0 && w[j0] - w[j0 - 1] <= tol) return;            // not a start
-  if (j0 + 1 >= m || w[j0 + 1] - w[j0] > tol) return;         // singleton
+  if (j0 + 1 >= nc || w[j0 + 1] - w[j0] > tol) return;         // singleton
   int j1 = j0 + 1;
-  while (j1 + 1 < m && w[j1 + 1] - w[j1] <= tol) ++j1;
+  while (j1 + 1 < nc && w[j1 + 1] - w[j1] <= tol) ++j1;
   const int c = j1 - j0 + 1;
   const bool in_smem = ((long)m * c + c) * 8 <= smem_bytes;
   double* Zb = in_smem ? cs : Z + j0;          // column q of the cluster: Zb[i * ld + q]
-  const long ld = in_smem ? c : m;
+  const long ld = in_smem ? c : nc;
   double* pk = in_smem ? cs + (long)m * c : cs;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   if (in_smem) {
     for (long t = threadIdx.x; t < (long)m * c; t += blockDim.x)
-      cs[t] = Z[(t / c) * m + j0 + t % c];
+      cs[t] = Z[(t / c) * nc + j0 + t % c];
     __syncthreads();
   }
   for (int q = 0; q < c; ++q) {
@@ -934,7 +932,7 @@ k_cluster_cgs2(const double* __restrict__ w, int m, double tol, int smem_bytes,
   }
   if (in_smem)
     for (long t = threadIdx.x; t < (long)m * c; t += blockDim.x)
-      Z[(t / c) * m + j0 + t % c] = cs[t];
+      Z[(t / c) * nc + j0 + t % c] = cs[t];
 }
 
 // G[i][i] -= x
@@ -975,13 +973,13 @@ __device__ __forceinline__ double probe_sign(int k, int which) {
 }
 // u[q][i] = sum_k Z[i][k] r_q[k]: a warp per row
 __global__ void __launch_bounds__(256)
-k_ortho_probe1(const double* __restrict__ Z, int m, double* __restrict__ u) {
+k_ortho_probe1(const double* __restrict__ Z, int m, int nc, double* __restrict__ u) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int i = warp; i < m; i += nw) {
-    const double* row = Z + (long)i * m;
+    const double* row = Z + (long)i * nc;
     double s1 = 0.0, s2 = 0.0;
-    for (int k = lane; k < m; k += 32) {
+    for (int k = lane; k < nc; k += 32) {
       const double z = row[k];
       s1 = fma(z, probe_sign(k, 0), s1);
       s2 = fma(z, probe_sign(k, 1), s2);
@@ -1000,22 +998,22 @@ k_ortho_probe1(const double* __restrict__ Z, int m, double* __restrict__ u) {
 // w_q[c] = sum_i Z[i][c] u_q[i] (32 columns x 8 row groups per block, fixed-order sum over
 // the groups) and dev = max |w_q[c] - r_q[c]| (integer maximum of the bit patterns)
 __global__ void __launch_bounds__(256)
-k_ortho_probe2(const double* __restrict__ Z, int m, const double* __restrict__ u,
+k_ortho_probe2(const double* __restrict__ Z, int m, int nc, const double* __restrict__ u,
                unsigned long long* __restrict__ dev) {
   __shared__ double part[2][8][33];
   const int cx = threadIdx.x & 31, rg = threadIdx.x >> 5;
   const int c = blockIdx.x * 32 + cx;
   double s1 = 0.0, s2 = 0.0;
-  if (c < m)
+  if (c < nc)
     for (int i = rg; i < m; i += 8) {
-      const double z = Z[(long)i * m + c];
+      const double z = Z[(long)i * nc + c];
       s1 = fma(z, u[i], s1);
       s2 = fma(z, u[m + i], s2);
     }
   part[0][rg][cx] = s1;
   part[1][rg][cx] = s2;
   __syncthreads();
-  if (rg == 0 && c < m) {
+  if (rg == 0 && c < nc) {
     double w1 = 0.0, w2 = 0.0;
     for (int g = 0; g < 8; ++g) {
       w1 += part[0][g][cx];
@@ -1028,38 +1026,13 @@ k_ortho_probe2(const double* __restrict__ Z, int m, const double* __restrict__ u
   }
 }
 
-// r[c] = sum_i v[i] Z[k+1+i][c]: 32 columns x 8 row groups per block (coalesced rows),
-// fixed-order reduction over the row groups in shared memory.
-__global__ void __launch_bounds__(256)
-k_vtz(const double* __restrict__ vbuf, int m, int k, const double* __restrict__ Z,
-      double* __restrict__ r) {
-  __shared__ double part[8][33];
-  const int n1 = m - k - 1;
-  const double* v = vbuf + (long)k * m + k + 1;
-  const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-  const int c = blockIdx.x * 32 + cx;
-  double s = 0.0;
-  if (c < m) {
-#pragma unroll 4
-    for (int i = ry; i < n1; i += 8) s += v[i] * Z[(long)(k + 1 + i) * m + c];
-  }
-  part[ry][cx] = s;
-  __syncthreads();
-  if (ry == 0 && c < m) {
-    double t = 0.0;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) t += part[q][cx];
-    r[c] = t;
-  }
-}
-
 // Back-transformation V = H_0 ... H_{m-3} Z with each block owning cb consecutive columns
 // (cb = 8 with 32 row groups of 256 threads): for every reflector (in reverse order) the block
 // forms r_c = v . Z[k+1.., c] for its columns over rg = blockDim / cb row groups and
 // applies Z[k+1+i][c] -= tau v_i r_c.  Columns are independent, so no grid-wide
 // synchronisation is needed.
 __global__ void __launch_bounds__(256)
-k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau, int m, int cb,
+k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau, int m, int nc, int cb,
                 double* __restrict__ Z) {
   __shared__ double part[256];
   __shared__ double rc[32];
@@ -1071,8 +1044,8 @@ k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau,
     const int n1 = m - k - 1;
     const double* v = vbuf + (long)k * m + k + 1;
     double s = 0.0;
-    if (act && c < m)
-      for (int i = ry; i < n1; i += rg) s += v[i] * Z[(long)(k + 1 + i) * m + c];
+    if (act && c < nc)
+      for (int i = ry; i < n1; i += rg) s += v[i] * Z[(long)(k + 1 + i) * nc + c];
     part[threadIdx.x] = s;
     __syncthreads();
     if (threadIdx.x < cb) {
@@ -1081,9 +1054,9 @@ k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau,
       rc[threadIdx.x] = t * tau[k];
     }
     __syncthreads();
-    if (act && c < m) {
+    if (act && c < nc) {
       const double r = rc[cx];
-      for (int i = ry; i < n1; i += rg) Z[(long)(k + 1 + i) * m + c] -= v[i] * r;
+      for (int i = ry; i < n1; i += rg) Z[(long)(k + 1 + i) * nc + c] -= v[i] * r;
     }
     __syncthreads();
   }
@@ -1096,16 +1069,16 @@ k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau,
 // 8-byte cp.async copies) has landed.  Z is read and written once.
 __global__ void __launch_bounds__(512)
 k_backtransform_smem(const double* __restrict__ vbuf, const double* __restrict__ tau, int m,
-                     int cb, double* __restrict__ Z) {
+                     int nc, int cb, double* __restrict__ Z) {
   extern __shared__ double zs[];                 // zs[cb][m], then vs[2][m]
   double* vs = zs + (long)cb * m;
   const int c0 = blockIdx.x * cb;
-  const int ncol = min(cb, m - c0);
+  const int ncol = min(cb, nc - c0);
   const int lane = threadIdx.x & 31, wc = threadIdx.x >> 5;
   const int nth = blockDim.x;
   for (long q = threadIdx.x; q < (long)m * cb; q += nth) {
     const int i = q / cb, c = q % cb;            // row-major walk of Z (coalesced per row)
-    zs[(long)c * m + i] = c < ncol ? Z[(long)i * m + c0 + c] : 0.0;
+    zs[(long)c * m + i] = c < ncol ? Z[(long)i * nc + c0 + c] : 0.0;
   }
   auto prefetch = [&](int k) {                   // v_k -> vs[k & 1]
     const int n1 = m - k - 1;
@@ -1147,22 +1120,7 @@ k_backtransform_smem(const double* __restrict__ vbuf, const double* __restrict__
   __syncthreads();
   for (long q = threadIdx.x; q < (long)m * cb; q += nth) {
     const int i = q / cb, c = q % cb;
-    if (c < ncol) Z[(long)i * m + c0 + c] = zs[(long)c * m + i];
-  }
-}
-
-// Z[k+1+i][c] -= tau v[i] r[c]
-__global__ void k_zupd(const double* __restrict__ vbuf, int m, int k,
-                       const double* __restrict__ tau, const double* __restrict__ r,
-                       double* __restrict__ Z) {
-  const int n1 = m - k - 1;
-  const double* v = vbuf + (long)k * m + k + 1;
-  const double t = tau[k];
-  const long total = (long)n1 * m;
-  for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < total;
-       q += (long)gridDim.x * blockDim.x) {
-    const int i = q / m, c = q % m;
-    Z[(long)(k + 1 + i) * m + c] -= t * v[i] * r[c];
+    if (c < ncol) Z[(long)i * nc + c0 + c] = zs[(long)c * m + i];
   }
 }
 
@@ -1195,13 +1153,13 @@ constexpr int kWyMinSize = 1024;    // blocked back-transformation from this siz
 // W = Vp^T V (rows below the panel start), W <- T W, V -= Vp W, three FP64 GEMMs per
 // panel.  vbuf rows hold the reflectors with zeros left of their first entry, so a panel's
 // rows of vbuf are Vp^T as it stands.  scratch >= 2 b m + 2 b^2 + part doubles.
-int backtransform_wy(const double* vbuf, const double* tau, int m, double* V, double* scratch,
-                     long scratch_size, cudaStream_t s, OzWork* oz) {
+int backtransform_wy(const double* vbuf, const double* tau, int m, int nc, double* V,
+                     double* scratch, long scratch_size, cudaStream_t s, OzWork* oz) {
   const int nref = m - 2;
   const int nb = kWyPanel;
   double* W = scratch;
-  double* W2 = W + (long)nb * m;
-  double* Gp = W2 + (long)nb * m;
+  double* W2 = W + (long)nb * nc;
+  double* Gp = W2 + (long)nb * nc;
   double* T = Gp + (long)nb * nb;
   double* part = T + (long)nb * nb;
   const long partmax = scratch_size - (part - scratch);
@@ -1219,19 +1177,19 @@ int backtransform_wy(const double* vbuf, const double* tau, int m, double* V, do
       // precision form: the two large products as FP64-accurate split products (the
       // eigenvalues are fixed before this step; only the vectors pass through it)
       const OzView va{Vt + k0 + 1, m, 1, r, 0};                  // rows l, K = row i
-      const OzView vb{V + (long)(k0 + 1) * m, 1, m, r, 0};       // rows col, K = row i
-      CASPT2_CUDA_TRY(oz_matmul(*oz, va, vb, false, b, m, r, 1.0, 0.0, W, m, s));
-      CASPT2_CUDA_TRY(dgemm(b, m, b, 1.0, T, b, false, W, m, false, 0.0, W2, m, s));
+      const OzView vb{V + (long)(k0 + 1) * nc, 1, nc, r, 0};     // rows col, K = row i
+      CASPT2_CUDA_TRY(oz_matmul(*oz, va, vb, false, b, nc, r, 1.0, 0.0, W, nc, s));
+      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, T, b, false, W, nc, false, 0.0, W2, nc, s));
       const OzView vp{Vt + k0 + 1, 1, m, b, 0};                  // rows i, K = l
-      const OzView vw{W2, 1, m, b, 0};                           // rows col, K = l
-      CASPT2_CUDA_TRY(oz_matmul(*oz, vp, vw, false, r, m, b, -1.0, 1.0, V + (long)(k0 + 1) * m,
-                                m, s));
+      const OzView vw{W2, 1, nc, b, 0};                          // rows col, K = l
+      CASPT2_CUDA_TRY(oz_matmul(*oz, vp, vw, false, r, nc, b, -1.0, 1.0, V + (long)(k0 + 1) * nc,
+                                nc, s));
     } else {
-      CASPT2_CUDA_TRY(dgemm(b, m, r, 1.0, Vt + k0 + 1, m, false, V + (long)(k0 + 1) * m, m,
-                            false, 0.0, W, m, s));
-      CASPT2_CUDA_TRY(dgemm(b, m, b, 1.0, T, b, false, W, m, false, 0.0, W2, m, s));
-      CASPT2_CUDA_TRY(dgemm(r, m, b, -1.0, Vt + k0 + 1, m, true, W2, m, false, 1.0,
-                            V + (long)(k0 + 1) * m, m, s));
+      CASPT2_CUDA_TRY(dgemm(b, nc, r, 1.0, Vt + k0 + 1, m, false, V + (long)(k0 + 1) * nc, nc,
+                            false, 0.0, W, nc, s));
+      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, T, b, false, W, nc, false, 0.0, W2, nc, s));
+      CASPT2_CUDA_TRY(dgemm(r, nc, b, -1.0, Vt + k0 + 1, m, true, W2, nc, false, 1.0,
+                            V + (long)(k0 + 1) * nc, nc, s));
     }
   }
   return CASPT2_OK;
@@ -1239,7 +1197,8 @@ int backtransform_wy(const double* vbuf, const double* tau, int m, double* V, do
 }  // namespace
 
 int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
-                    KernelTimer* tm, OzWork* oz) {
+                    KernelTimer* tm, OzWork* oz, double wmin, int* nkept) {
+  if (nkept) *nkept = 0;
   if (m <= 0) return CASPT2_OK;
   const long mm = (long)m * m;
   double* vbuf = work;            // m*m reflectors
@@ -1442,19 +1401,32 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   const int bis_t = (int)std::min<long>(1024, std::max<long>(32, ((8L * m + nsm - 1) / nsm + 31) / 32 * 32));
   k_bisect<<<(unsigned)((8L * m + bis_t - 1) / bis_t), bis_t, 3 * sizeof(double) * m, s>>>(
       d, e, e2, m, glo, ghi, 4.0 * 2.2e-16 * std::max(1.0, tnorm), w);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  // the vectors to form: all, or those of the eigenvalues at or above wmin (the last nc of
+  // the ascending list)
+  int j0 = 0;
+  if (nkept) {
+    CASPT2_CUDA_TRY(cudaMemcpyAsync(hd.data(), w, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
+    CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
+    while (j0 < m && hd[j0] < wmin) ++j0;
+    *nkept = m - j0;
+    if (j0 == m) return CASPT2_OK;
+  }
+  const int nc = m - j0;
+  const double* wk = w + j0;
   // 3. eigenvectors of T
   ++launch_counter();
   // one warp per block so that the m independent LU chains spread over the SMs
   CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_inviter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kBisectSmemMax));
-  k_inviter<<<(m + 31) / 32, 32, 2 * sizeof(double) * m, s>>>(d, e, w, m, tnorm, u0, u1, u2, lm,
-                                                               pv, Z);
+  k_inviter<<<(nc + 31) / 32, 32, 2 * sizeof(double) * m, s>>>(d, e, wk, m, nc, tnorm, u0, u1, u2,
+                                                                lm, pv, Z);
   ++launch_counter();
   CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_cluster_cgs2, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kBisectSmemMax));
   {
-    const int cbytes = (int)std::min<size_t>(kBisectSmemMax, 8ull * ((size_t)m * m + m));
-    k_cluster_cgs2<<<m, 256, cbytes, s>>>(w, m, 1e-12 * std::max(1.0, tnorm), cbytes, Z);
+    const int cbytes = (int)std::min<size_t>(kBisectSmemMax, 8ull * ((size_t)m * nc + nc));
+    k_cluster_cgs2<<<nc, 256, cbytes, s>>>(wk, m, nc, 1e-12 * std::max(1.0, tnorm), cbytes, Z);
   }
   CASPT2_CUDA_TRY(cudaGetLastError());
   // 4. Newton-Schulz: Z <- Z (1.5 I - 0.5 Z^T Z), skipped when Z is already orthonormal to
@@ -1464,9 +1436,9 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   unsigned long long* ns_dev = reinterpret_cast<unsigned long long*>(r + m);
   CASPT2_CUDA_TRY(cudaMemsetAsync(ns_dev, 0, sizeof(unsigned long long), s));
   ++launch_counter();
-  k_ortho_probe1<<<nblocks(32L * m), kT, 0, s>>>(Z, m, G);
+  k_ortho_probe1<<<nblocks(32L * m), kT, 0, s>>>(Z, m, nc, G);
   ++launch_counter();
-  k_ortho_probe2<<<(m + 31) / 32, 256, 0, s>>>(Z, m, G, ns_dev);
+  k_ortho_probe2<<<(nc + 31) / 32, 256, 0, s>>>(Z, m, nc, G, ns_dev);
   CASPT2_CUDA_TRY(cudaGetLastError());
   unsigned long long hdev = 0;
   CASPT2_CUDA_TRY(cudaMemcpyAsync(&hdev, ns_dev, sizeof(hdev), cudaMemcpyDeviceToHost, s));
@@ -1475,12 +1447,12 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   std::memcpy(&dev_probe, &hdev, sizeof(double));
   if (!(dev_probe == dev_probe)) return CASPT2_ENAN;
   if (dev_probe <= 1e-13) {
-    CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * mm, cudaMemcpyDeviceToDevice, s));
+    CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
   } else {
     CASPT2_CUDA_TRY(cudaMemsetAsync(ns_dev, 0, sizeof(unsigned long long), s));
-    CASPT2_CUDA_TRY(dgemm_sym(m, m, 1.0, Z, m, true, Z, m, false, 0.0, G, m, s));
+    CASPT2_CUDA_TRY(dgemm_sym(nc, m, 1.0, Z, nc, true, Z, nc, false, 0.0, G, nc, s));
     ++launch_counter();
-    k_ns_coef<<<nblocks(mm), kT, 0, s>>>(G, m, ns_dev);
+    k_ns_coef<<<nblocks((long)nc * nc), kT, 0, s>>>(G, nc, ns_dev);
     CASPT2_CUDA_TRY(cudaGetLastError());
     CASPT2_CUDA_TRY(cudaMemcpyAsync(&hdev, ns_dev, sizeof(hdev), cudaMemcpyDeviceToHost, s));
     CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1488,48 +1460,49 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
     std::memcpy(&dev_ortho, &hdev, sizeof(double));
     if (!(dev_ortho == dev_ortho)) return CASPT2_ENAN;
     if (dev_ortho <= 1e-13) {
-      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * mm, cudaMemcpyDeviceToDevice, s));
+      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
     } else if (oz && oz->on) {
       // V = Z + Z Ec, Ec = (1/2)(I - Z^T Z) (G - I): the correction is of the size of the
       // orthogonality error, so a split product with S slices (error below about
       // 2^(1-7S) m max|Z| max|Ec|) is kept under 1e-17 with S = ceil((57 + log2(m dev/2)) / 7)
       ++launch_counter();
-      k_sub_diag<<<(m + 255) / 256, 256, 0, s>>>(G, m, 1.0);
+      k_sub_diag<<<(nc + 255) / 256, 256, 0, s>>>(G, nc, 1.0);
       CASPT2_CUDA_TRY(cudaGetLastError());
-      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * mm, cudaMemcpyDeviceToDevice, s));
+      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
       const double lg = std::log2(std::max(1e-300, 0.5 * (double)m * dev_ortho));
       const int S = std::max(2, std::min(kOzMaxSlices, (int)std::ceil((57.0 + lg) / 7.0)));
       const int S0 = oz->S;
       oz->S = S;
-      const OzView vz{Z, m, 1, m, 0}, vg{G, m, 1, m, 0};   // G symmetric: B(j, k) = G[j][k]
-      const cudaError_t e = oz_matmul(*oz, vz, vg, false, m, m, m, 1.0, 1.0, V, m, s);
+      const OzView vz{Z, nc, 1, nc, 0}, vg{G, nc, 1, nc, 0};   // G symmetric: B(j, k) = G[j][k]
+      const cudaError_t e = oz_matmul(*oz, vz, vg, false, m, nc, nc, 1.0, 1.0, V, nc, s);
       oz->S = S0;
       CASPT2_CUDA_TRY(e);
     } else {
-      CASPT2_CUDA_TRY(dgemm(m, m, m, 1.0, Z, m, false, G, m, false, 0.0, V, m, s));
+      CASPT2_CUDA_TRY(dgemm(m, nc, nc, 1.0, Z, nc, false, G, nc, false, 0.0, V, nc, s));
     }
   }
   // 5. back-transformation V = H_0 ... H_{m-3} Z: blocked (compact WY panels as FP64
   //    GEMMs) for large matrices, else column-owned in one launch.  Z, G and the
   //    inverse-iteration scratch are free here.
   if (m >= kWyMinSize) {
-    const int st = backtransform_wy(vbuf, tau, m, V, Z, 7 * mm, s, oz);
+    const int st = backtransform_wy(vbuf, tau, m, nc, V, Z, 7 * mm, s, oz);
     if (st != CASPT2_OK) return st;
   } else if (m >= 3) {
     ++launch_counter();
     // columns resident in shared memory: ceil(m / SMs) per block (one block per SM, the
     // FP64 work spread evenly, one warp per column), fewer per block when they do not fit
     const long fit = (long)(kBackSmemMax / (8ull * m)) - 2;      // minus the v buffers
-    const int cbs = (int)std::min<long>(std::min<long>(16, (m + nsm - 1) / nsm), fit);
+    const int cbs = (int)std::min<long>(std::min<long>(16, (nc + nsm - 1) / nsm), fit);
     if (cbs >= 1) {
       CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_backtransform_smem,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)kBackSmemMax));
-      k_backtransform_smem<<<(m + cbs - 1) / cbs, 32 * cbs, sizeof(double) * (size_t)m * (cbs + 2),
-                             s>>>(vbuf, tau, m, cbs, V);
+      k_backtransform_smem<<<(nc + cbs - 1) / cbs, 32 * cbs,
+                             sizeof(double) * (size_t)m * (cbs + 2), s>>>(vbuf, tau, m, nc, cbs,
+                                                                          V);
     } else {
       const int cb = 8;     // 8 columns x 32 row groups per block
-      k_backtransform<<<(m + cb - 1) / cb, 256, 0, s>>>(vbuf, tau, m, cb, V);
+      k_backtransform<<<(nc + cb - 1) / cb, 256, 0, s>>>(vbuf, tau, m, nc, cb, V);
     }
   }
   CASPT2_CUDA_TRY(cudaGetLastError());

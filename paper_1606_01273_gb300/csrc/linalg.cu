@@ -514,4 +514,24 @@ int sym_eig_jacobi(double* A, int m, double* w, double* V, double* work, cudaStr
   return conv ? CASPT2_OK : CASPT2_ENOTCONV;
 }
 
+int sym_eig_above(double* A, int m, double wmin, double* w, double* V, int* nkept, int* ldv,
+                  int* voff, double* work, cudaStream_t s, KernelTimer* tm, OzWork* oz) {
+  *nkept = 0;
+  *voff = 0;
+  if (m > 32) {
+    const int st = sym_eig_tridiag(A, m, w, V, work, s, tm, oz, wmin, nkept);
+    *ldv = *nkept;
+    return st;
+  }
+  *ldv = m;
+  const int st = sym_eig_jacobi(A, m, w, V, work, s);
+  if (st != CASPT2_OK) return st;
+  std::vector<double> hw(m);
+  CASPT2_CUDA_TRY(cudaMemcpyAsync(hw.data(), w, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
+  CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
+  while (*voff < m && hw[*voff] < wmin) ++*voff;
+  *nkept = m - *voff;
+  return CASPT2_OK;
+}
+
 }  // namespace caspt2

@@ -62,8 +62,11 @@ size_t sym_eig_tridiag_work(int m);
 // oz (optional, on): the Newton-Schulz correction Z (1/2)(I - Z^T Z), a term of the size of
 // the orthogonality error, runs as a split-BF16 product with just enough slices.
 struct OzWork;
+// nkept (optional): only the vectors of the eigenvalues >= wmin are formed, V is m x *nkept
+// (ascending), and *nkept is known on the host when the call returns.
 int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
-                    KernelTimer* tm = nullptr, OzWork* oz = nullptr);
+                    KernelTimer* tm = nullptr, OzWork* oz = nullptr, double wmin = 0.0,
+                    int* nkept = nullptr);
 
 // Dispatch: Jacobi for small matrices, tridiagonal method otherwise.
 inline int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
@@ -71,6 +74,15 @@ inline int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStr
   return m <= 32 ? sym_eig_jacobi(A, m, w, V, work, s)
                  : sym_eig_tridiag(A, m, w, V, work, s, tm, oz);
 }
+// Eigenvalues w[m] (all) and the eigenvectors of those >= wmin: *nkept vectors, V[i * ldv +
+// voff + c] component i of the c-th (ascending).  The vectors below the cut are not formed
+// where the tridiagonal method runs: an overlap matrix of rank r spends its inverse
+// iteration, cluster orthogonalisation and back-transformation on r columns, and its null
+// space (one cluster of equal eigenvalues, serial in the Gram-Schmidt: 0.9 s of the 1.3 s of
+// a c42 a6 v350 n4 solve) costs nothing.
+int sym_eig_above(double* A, int m, double wmin, double* w, double* V, int* nkept, int* ldv,
+                  int* voff, double* work, cudaStream_t s, KernelTimer* tm = nullptr,
+                  OzWork* oz = nullptr);
 inline size_t sym_eig_work(int m) {
   return std::max<size_t>((size_t)2 * m * m + 2, sym_eig_tridiag_work(m));
 }
