@@ -61,6 +61,7 @@ struct caspt2_ctx {
   ClassWork cw[7];
   bool cw_on[7] = {};
   SectorWork sw{};
+  SectorBatch sb{};
   double *rdm3r = nullptr, *rdm4r = nullptr, *h = nullptr, *fact = nullptr, *eps = nullptr;
   double* hk = nullptr;               // precision form: core exchange block for h
   double *pack0 = nullptr, *pack1 = nullptr;
@@ -359,6 +360,38 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       for (int k = 0; k < 7; ++k)
         if (c->cw_on[k]) c->cw[k].V = vb;
     }
+    // the small sectors as jobs of one launch, and the denominator minima of every sector
+    {
+      SectorBatch& sb = c->sb;
+      long nmdn = 0;
+      for (int k = 0; k < 7; ++k) {
+        sb.first[k] = (int)sb.jobs.size();
+        if (!c->cw_on[k]) continue;
+        ClassWork& w = c->cw[k];
+        for (SectorKeep& K : w.keep) {
+          if (K.ntup == 0) continue;
+          K.mdn = nmdn;
+          nmdn += K.msec;
+          if (K.msec > kSectorBlockMax) continue;
+          SectorJob J{w.Sact, w.Fact, w.m, d.n, K.Lsel, K.msec, sector_sign(w, K.sec),
+                      o.ovl_thresh, nullptr, nullptr, K.Y, K.omega};
+          ALLOC(J.X, (size_t)K.msec * K.msec);
+          ALLOC(J.scr, sector_block_scratch(K.msec));
+          K.job = (int)sb.jobs.size();
+          sb.jobs.push_back(J);
+        }
+      }
+      sb.first[7] = (int)sb.jobs.size();
+      sb.hinfo.assign(2 * sb.jobs.size(), 0);
+      sb.hmdn.assign((size_t)nmdn, 0.0);
+      ALLOC(sb.mdn, (size_t)nmdn);
+      ALLOC(sb.info, 2 * sb.jobs.size());
+      ALLOC(sb.dev, sb.jobs.size());
+      if (st == CASPT2_OK && !sb.jobs.empty() &&
+          cudaMemcpy(sb.dev, sb.jobs.data(), sizeof(SectorJob) * sb.jobs.size(),
+                     cudaMemcpyHostToDevice) != cudaSuccess)
+        st = CASPT2_ECUDA;
+    }
     if (m2max > 0) {
       SectorWork& q = c->sw;
       const long mx = (long)std::sqrt((double)m2max) + 1;
@@ -611,13 +644,60 @@ int solve_impl(caspt2_ctx* c, void* stream) {
         CASPT2_CUDA_TRY(presum_block(d, sp, c->eri_blk.at(key), c->presum_blk[k], s));
       }
       RdmPtrs g{{nullptr, c->rdm1r, c->rdm2r, c->rdm3r, c->rdm4r}};
+      // partial solves: classes A-F belong to the partition that starts at closed 0
+      auto on = [&](int k) {
+        return c->cw_on[k] && (k == CASPT2_CLASS_G || o.closed_begin == 0);
+      };
+      // the sectors' eigenbases: the small ones of all classes in one launch, the others one
+      // by one; then the denominator minima of all of them
+      SectorBatch& sb = c->sb;
       for (int k = 0; k < 7; ++k) {
-        if (!c->cw_on[k]) continue;
-        // partial solves: classes A-F belong to the partition that starts at closed 0
-        if (k != CASPT2_CLASS_G && o.closed_begin > 0) continue;
-        int st = class_solve(c->cw[k], c->sw, d, o.scheme, o.shift, o.ovl_thresh, g, c->fact, c->h,
-                             c->eri_tab, c->presum_tab, c->E0, c->eps, c->mom + (long)k * msz,
-                             c->mindenom, s, &c->tri, &c->oz, o.closed_begin, o.closed_end);
+        if (!on(k)) continue;
+        const int st = class_matrices(c->cw[k], d, g, c->fact, s);
+        if (st != CASPT2_OK) return st;
+      }
+      const int j0 = o.closed_begin == 0 ? 0 : sb.first[CASPT2_CLASS_G];
+      const int nj = sb.first[7] - j0;
+      if (nj > 0) {
+        int mmax = 0;
+        for (int j = j0; j < j0 + nj; ++j) mmax = std::max(mmax, sb.jobs[j].msec);
+        CASPT2_CUDA_TRY(sector_block_launch(sb.dev + j0, nj, mmax, sb.info + 2 * j0, s));
+        CASPT2_CUDA_TRY(cudaMemcpyAsync(sb.hinfo.data() + 2 * j0, sb.info + 2 * j0,
+                                        2 * sizeof(int) * nj, cudaMemcpyDeviceToHost, s));
+      }
+      for (int k = 0; k < 7; ++k) {
+        if (!on(k)) continue;
+        for (SectorKeep& K : c->cw[k].keep) {
+          if (K.ntup == 0 || K.job >= 0) continue;
+          const int st = class_sector_basis(c->cw[k], K, c->sw, d, o.ovl_thresh, s, &c->tri,
+                                            &c->oz);
+          if (st != CASPT2_OK) return st;
+        }
+      }
+      CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
+      CASPT2_CUDA_TRY(launch_fill(sb.mdn, (long)sb.hmdn.size(), 1e300, s));
+      for (int k = 0; k < 7; ++k) {
+        if (!on(k)) continue;
+        for (SectorKeep& K : c->cw[k].keep) {
+          if (K.job >= 0) {
+            if (sb.hinfo[2 * K.job + 1] != 0) return CASPT2_ENAN;
+            K.nk = sb.hinfo[2 * K.job];
+          }
+          const int st = class_sector_mindenom(c->cw[k], K, c->sw, d, o.shift, c->E0, c->eps,
+                                               sb.mdn, s);
+          if (st != CASPT2_OK) return st;
+        }
+      }
+      if (!sb.hmdn.empty())
+        CASPT2_CUDA_TRY(cudaMemcpyAsync(sb.hmdn.data(), sb.mdn, sizeof(double) * sb.hmdn.size(),
+                                        cudaMemcpyDeviceToHost, s));
+      CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
+      for (int k = 0; k < 7; ++k) {
+        if (!on(k)) continue;
+        const int st = class_solve(c->cw[k], c->sw, d, o.scheme, o.shift, g, c->h, c->eri_tab,
+                                   c->presum_tab, c->E0, c->eps, sb.hmdn.data(),
+                                   c->mom + (long)k * msz, c->mindenom, s, &c->oz,
+                                   o.closed_begin, o.closed_end);
         if (st != CASPT2_OK) return st;
         CASPT2_CUDA_TRY(launch_moments_to_e(c->mom + (long)k * msz, n, c->ecls + (long)k * n * n,
                                             c->ncls + (long)k * n, s));

@@ -1221,19 +1221,109 @@ cudaError_t class_upload_plans(ClassWork& w, const std::vector<ActPlan>& S,
   return cudaSuccess;
 }
 
-int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double shift,
-                double thresh, RdmPtrs rdm, const double* f_act, const double* h,
-                const EriBlocks& eri, const PresumBlocks& pb, const double* E0,
-                const double* eps_cv, double* mom, double* mindenom, cudaStream_t s,
-                KernelTimer* tm, OzWork* oz, int ci0, int ci1) {
+int class_matrices(ClassWork& w, const Dims& d, RdmPtrs rdm, const double* f_act,
+                   cudaStream_t s) {
   const int m = w.m, n = d.n;
   if (w.vsize == 0 || m == 0) return CASPT2_OK;
   const long mm = (long)m * m;
-  // overlap, active Fock, sources
   ++launch_counter();
   k_act_eval<<<launch_blocks(mm), 256, 0, s>>>(w.dS, w.nS, w.dc, d.a, n, rdm, f_act, w.Sact, m);
   ++launch_counter();
   k_act_eval<<<launch_blocks(mm), 256, 0, s>>>(w.dF, w.nF, w.dc, d.a, n, rdm, f_act, w.Fact, m);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  return CASPT2_OK;
+}
+
+double sector_sign(const ClassWork& w, int sec) {
+  return w.dc.pair0 < 0 ? 0.0 : (sec == 0 ? 1.0 : -1.0);
+}
+
+int class_sector_basis(ClassWork& w, SectorKeep& K, SectorWork& sw, const Dims& d, double thresh,
+                       cudaStream_t s, KernelTimer* tm, OzWork* oz) {
+  const int m = w.m, n = d.n, msec = K.msec;
+  const long ms2 = (long)msec * msec;
+  const double sgn = sector_sign(w, K.sec);
+  ++launch_counter();
+  k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Sact, m, n, sgn, K.Lsel, sw.Ssec, msec);
+  ++launch_counter();
+  k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Fact, m, n, sgn, K.Lsel, sw.Fsec, msec);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  K.nk = 0;
+  OzWork* ozn = (oz && oz->on && oz->S >= kOzMaxSlices) ? oz : nullptr;
+  // eigenvalues of the overlap and the eigenvectors of those at or above the threshold
+  int nk = 0, ldq = 0, qoff = 0;
+  int st = sym_eig_above(sw.Ssec, msec, thresh, sw.s, sw.Qs, &nk, &ldq, &qoff, sw.jac, s, tm,
+                         ozn);
+  if (st != CASPT2_OK) return st;
+  if (nk == 0) return CASPT2_OK;
+  K.nk = nk;
+  ++launch_counter();
+  k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, ldq, qoff, sw.s, msec,
+                                                               nk, sw.X);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  const bool ozx = oz && oz->on && oz->S >= kOzMaxSlices && msec >= kOzTransformMin;
+  if (ozx) {
+    // precision form, FP64-accurate split products (7 slices) for the sector
+    // transforms F X, X^T (F X) and X Q of the large sectors
+    const OzView vf{sw.Fsec, msec, 1, msec, 0}, vxt{sw.X, 1, nk, msec, 0};
+    CASPT2_CUDA_TRY(oz_matmul(*oz, vf, vxt, false, msec, nk, msec, 1.0, 0.0, sw.FX, nk, s));
+    const OzView vfx{sw.FX, 1, nk, msec, 0};
+    CASPT2_CUDA_TRY(oz_matmul(*oz, vxt, vfx, false, nk, nk, msec, 1.0, 0.0, sw.Ft, nk, s));
+    CASPT2_CUDA_TRY(launch_symmetrize(sw.Ft, nk, 1, s));
+  } else {
+    CASPT2_CUDA_TRY(dgemm(msec, nk, msec, 1.0, sw.Fsec, msec, false, sw.X, nk, false, 0.0,
+                          sw.FX, nk, s));
+    CASPT2_CUDA_TRY(dgemm_sym(nk, msec, 1.0, sw.X, nk, true, sw.FX, nk, false, 0.0, sw.Ft, nk,
+                              s));
+  }
+  st = sym_eig(sw.Ft, nk, K.omega, sw.Qf, sw.jac, s, tm, ozn);
+  if (st != CASPT2_OK) return st;
+  if (ozx) {
+    const OzView vx{sw.X, nk, 1, nk, 0}, vq{sw.Qf, 1, nk, nk, 0};
+    CASPT2_CUDA_TRY(oz_matmul(*oz, vx, vq, false, msec, nk, nk, 1.0, 0.0, K.Y, nk, s));
+  } else {
+    CASPT2_CUDA_TRY(dgemm(msec, nk, nk, 1.0, sw.X, nk, false, sw.Qf, nk, false, 0.0, K.Y, nk,
+                          s));
+  }
+  return CASPT2_OK;
+}
+
+int class_sector_mindenom(const ClassWork& w, const SectorKeep& K, SectorWork& sw, const Dims& d,
+                          double shift, const double* E0, const double* eps_cv, double* mdn,
+                          cudaStream_t s) {
+  const long ntup = K.ntup;
+  const int nk = K.nk, n = d.n;
+  if (nk == 0 || ntup == 0) return CASPT2_OK;
+  const dim3 grid((unsigned)std::min<long>((ntup + 255) / 256, 64), nk);
+  if (ntup <= sw.wcap) {
+    // the tuples' external energies once into W (free until the sector sources)
+    ++launch_counter();
+    k_sector_eext<<<launch_blocks(ntup), 256, 0, s>>>(eps_cv, w.dc, w.ed, d.c, K.sec, ntup, sw.W);
+    ++launch_counter();
+    k_mu_mindenom_ee<<<grid, 256, 0, s>>>(K.omega, E0, sw.W, n, K.Lsel, ntup, shift, mdn + K.mdn);
+  } else {
+    ++launch_counter();
+    k_mu_mindenom<<<grid, 256, 0, s>>>(K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, K.sec, K.Lsel,
+                                       ntup, nk, shift, mdn + K.mdn);
+  }
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  return CASPT2_OK;
+}
+
+cudaError_t launch_fill(double* x, long n, double v, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  ++launch_counter();
+  k_fill<<<launch_blocks(n), 256, 0, s>>>(x, n, v);
+  return cudaGetLastError();
+}
+
+int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double shift,
+                RdmPtrs rdm, const double* h, const EriBlocks& eri, const PresumBlocks& pb,
+                const double* E0, const double* eps_cv, const double* hmdn, double* mom,
+                double* mindenom, cudaStream_t s, OzWork* oz, int ci0, int ci1) {
+  const int m = w.m, n = d.n;
+  if (w.vsize == 0 || m == 0) return CASPT2_OK;
+  // sources
   ++launch_counter();
   if (n <= 4) {
     const long total2 = w.vsize / ((long)n * n);
@@ -1280,182 +1370,111 @@ int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double 
     }
   }
 
-  const int nsec = w.dc.pair0 < 0 ? 1 : 2;
-  for (int sec = 0; sec < nsec; ++sec) {
-    const long ntup = sector_tuples(w, sec);
-    if (ntup == 0) continue;
-    const double sgn = w.dc.pair0 < 0 ? 0.0 : (sec == 0 ? 1.0 : -1.0);
-    const int nsel = scheme == CASPT2_SSSR ? n : 1;
-    for (int is = 0; is < nsel; ++is) {
-      const int Lsel = scheme == CASPT2_SSSR ? is : -1;
-      const int msec = scheme == CASPT2_SSSR ? m / n : m;
-      const long ms2 = (long)msec * msec;
+  for (SectorKeep& K : w.keep) {
+    const int sec = K.sec, Lsel = K.Lsel, msec = K.msec, nk = K.nk;
+    const long ntup = K.ntup, ms2 = (long)msec * msec;
+    if (ntup == 0 || nk == 0) continue;
+    // eigenvalues next to small denominators: Rayleigh quotients in double-double
+    // against the sector's S and F (rebuilt into Qs and Fsec)
+    const double* hm = hmdn + K.mdn;
+    std::vector<int> list;
+    for (int k = 0; k < nk; ++k)
+      if (hm[k] < kRefineDenom) list.push_back(k);
+    if (!list.empty()) {
+      // list (ints) at the start of part2, the stage-1 partials in W (free here)
+      const int nl = (int)list.size();
+      const int nrb = (int)std::max<long>(1, std::min<long>(
+          {(long)(msec + 63) / 64, 1216L / nl + 1, sw.wcap / (4L * nl)}));
+      if ((long)nl > sw.p2size || 4L * nl * nrb > sw.wcap) return CASPT2_EINVAL;
+      int* dlist = reinterpret_cast<int*>(sw.part2);
+      CASPT2_CUDA_TRY(cudaMemcpyAsync(dlist, list.data(), sizeof(int) * nl,
+                                      cudaMemcpyHostToDevice, s));
+      const double sgn = sector_sign(w, sec);
       ++launch_counter();
-      k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Sact, m, n, sgn, Lsel, sw.Ssec, msec);
+      k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Sact, m, n, sgn, Lsel, sw.Qs, msec);
       ++launch_counter();
       k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Fact, m, n, sgn, Lsel, sw.Fsec, msec);
-      CASPT2_CUDA_TRY(cudaGetLastError());
-      SectorKeep& K = w.keep[sec * nsel + is];
-      K.nk = 0;
-      OzWork* ozn = (oz && oz->on && oz->S >= kOzMaxSlices) ? oz : nullptr;
-      // eigenvalues of the overlap and the eigenvectors of those at or above the threshold
-      int nk = 0, ldq = 0, qoff = 0;
-      int st = sym_eig_above(sw.Ssec, msec, thresh, sw.s, sw.Qs, &nk, &ldq, &qoff, sw.jac, s, tm,
-                             ozn);
-      if (st != CASPT2_OK) return st;
-      if (nk == 0) continue;
-      K.nk = nk;
       ++launch_counter();
-      k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, ldq, qoff, sw.s, msec,
-                                                                   nk, sw.X);
+      k_rq_partial<<<dim3(nrb, nl), kRqThreads, 0, s>>>(sw.Qs, sw.Fsec, msec, K.Y, nk, dlist,
+                                                       sw.W);
+      ++launch_counter();
+      k_rq_finish<<<(nl + 127) / 128, 128, 0, s>>>(sw.W, nrb, dlist, nl, K.omega);
       CASPT2_CUDA_TRY(cudaGetLastError());
-      const bool ozx = oz && oz->on && oz->S >= kOzMaxSlices && msec >= kOzTransformMin;
-      if (ozx) {
-        // precision form, FP64-accurate split products (7 slices) for the sector
-        // transforms F X, X^T (F X) and X Q of the large sectors
-        const OzView vf{sw.Fsec, msec, 1, msec, 0}, vxt{sw.X, 1, nk, msec, 0};
-        CASPT2_CUDA_TRY(oz_matmul(*oz, vf, vxt, false, msec, nk, msec, 1.0, 0.0, sw.FX, nk, s));
-        const OzView vfx{sw.FX, 1, nk, msec, 0};
-        CASPT2_CUDA_TRY(oz_matmul(*oz, vxt, vfx, false, nk, nk, msec, 1.0, 0.0, sw.Ft, nk, s));
-        CASPT2_CUDA_TRY(launch_symmetrize(sw.Ft, nk, 1, s));
+      // eigenvectors: y_k += sum_j c_j y_j with the double-double residual of (F, S)
+      double* R = sw.W;                                  // [msec][nl]
+      double* Cm = R + (long)msec * nl;                  // [nk][nl]
+      double* Dl = Cm + (long)nk * nl;                   // [msec][nl]
+      if ((long)(2 * msec + nk) * nl > sw.wcap) return CASPT2_EINVAL;
+      ++launch_counter();
+      k_rq_resid<<<dim3(nrb, nl), kRqThreads, 0, s>>>(sw.Qs, sw.Fsec, msec, K.Y, nk, dlist, nl,
+                                                     K.omega, R);
+      CASPT2_CUDA_TRY(cudaGetLastError());
+      CASPT2_CUDA_TRY(dgemm(nk, nl, msec, 1.0, K.Y, nk, true, R, nl, false, 0.0, Cm, nl, s));
+      ++launch_counter();
+      k_rq_coef<<<launch_blocks((long)nk * nl), 256, 0, s>>>(Cm, nk, dlist, nl, K.omega);
+      CASPT2_CUDA_TRY(cudaGetLastError());
+      CASPT2_CUDA_TRY(dgemm(msec, nl, nk, 1.0, K.Y, nk, false, Cm, nl, false, 0.0, Dl, nl, s));
+      ++launch_counter();
+      k_rq_apply<<<launch_blocks((long)msec * nl), 256, 0, s>>>(K.Y, msec, nk, dlist, nl, Dl);
+      CASPT2_CUDA_TRY(cudaGetLastError());
+      CASPT2_CUDA_TRY(cudaStreamSynchronize(s));   // the host list is released below
+    }
+    const long ncol = ntup * n;
+    const int nL = Lsel < 0 ? n : 1;
+    const int pcol = nL * n * (n + 2);
+    // tuples in chunks so that the sector sources W (msec x chunk n) and the moment
+    // partials (chunk x pcol) stay within the work arrays the context holds
+    long chunk = std::min<long>(ntup, sw.wcap / ((long)msec * n));
+    chunk = std::min<long>(chunk, sw.pcap / pcol);
+    if (chunk < 1 || (long)nk * ncol > (1L << 62)) return CASPT2_EINVAL;
+    // class G under a closed-orbital range: the sector tuples are ordered with the
+    // closed index slowest, so the range is a contiguous run of them
+    long tb = 0, te = ntup;
+    if (w.cls == CASPT2_CLASS_G && (ci0 > 0 || (ci1 >= 0 && ci1 < d.c))) {
+      const long per_i = ntup / d.c;
+      tb = (long)ci0 * per_i;
+      te = (long)(ci1 < 0 || ci1 > d.c ? d.c : ci1) * per_i;
+    }
+    for (long t0 = tb; t0 < te; t0 += chunk) {
+      const long nt = std::min(chunk, te - t0);
+      ++launch_counter();
+      k_sector_src<<<launch_blocks((long)(scheme == CASPT2_SSSR ? msec : msec / n) * nt), 256, 0, s>>>(
+          w.V, w.dc, w.ed, d.a, n, sec, Lsel, t0, nt, msec, sw.W);
+      CASPT2_CUDA_TRY(cudaGetLastError());
+      if (oz && oz->on && oz->S >= kOzMaxSlices) {
+        // precision form with every product FP64-accurate (7 slices): the sector
+        // transform as a split-BF16 tensor-core product (fewer slices keep it in FP64:
+        // the energies are first order in its rounding)
+        const OzView vy{K.Y, 1, nk, msec, 0};               // rows mu, K = sector row
+        const OzView vw{sw.W, 1, nt * n, msec, 0};           // rows (t, L'), K = sector row
+        CASPT2_CUDA_TRY(oz_matmul(*oz, vy, vw, false, nk, (int)(nt * n), msec, 1.0, 0.0,
+                                  K.Vt + t0 * n, ncol, s));
       } else {
-        CASPT2_CUDA_TRY(dgemm(msec, nk, msec, 1.0, sw.Fsec, msec, false, sw.X, nk, false, 0.0,
-                              sw.FX, nk, s));
-        CASPT2_CUDA_TRY(dgemm_sym(nk, msec, 1.0, sw.X, nk, true, sw.FX, nk, false, 0.0, sw.Ft, nk,
-                                  s));
+        CASPT2_CUDA_TRY(dgemm(nk, (int)(nt * n), msec, 1.0, K.Y, nk, true, sw.W,
+                              (int)(nt * n), false, 0.0, K.Vt + t0 * n, (int)ncol, s));
       }
-      st = sym_eig(sw.Ft, nk, K.omega, sw.Qf, sw.jac, s, tm, ozn);
-      if (st != CASPT2_OK) return st;
-      if (ozx) {
-        const OzView vx{sw.X, nk, 1, nk, 0}, vq{sw.Qf, 1, nk, nk, 0};
-        CASPT2_CUDA_TRY(oz_matmul(*oz, vx, vq, false, msec, nk, nk, 1.0, 0.0, K.Y, nk, s));
+      ++launch_counter();
+      if (n <= 4) {
+        k_sector_energy_ml<4><<<launch_blocks(nt * nL), 256, 0, s>>>(
+            K.Vt, K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, sec, Lsel, ntup, t0, nt, nk, shift,
+            sw.part, mindenom);
+      } else if (n <= 6) {
+        k_sector_energy_ml<6><<<launch_blocks(nt * nL), 256, 0, s>>>(
+            K.Vt, K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, sec, Lsel, ntup, t0, nt, nk, shift,
+            sw.part, mindenom);
       } else {
-        CASPT2_CUDA_TRY(dgemm(msec, nk, nk, 1.0, sw.X, nk, false, sw.Qf, nk, false, 0.0, K.Y, nk,
-                              s));
+        const long ne = nt * nL * n;
+        k_sector_energy<<<launch_blocks(ne), 256, 0, s>>>(K.Vt, K.omega, E0, eps_cv, w.dc, w.ed,
+                                                          d.c, n, sec, Lsel, ntup, t0, nt, nk,
+                                                          shift, sw.part, mindenom);
       }
-      {
-        // eigenvalues next to small denominators: Rayleigh quotients in double-double
-        // against the sector's S (rebuilt into Qs, free once X is formed) and F
-        double* mdn = sw.part2;      // nk minima (free until the column sums below)
-        if (nk > sw.p2size) return CASPT2_EINVAL;
-        const double big = 1e300;
-        ++launch_counter();
-        k_fill<<<launch_blocks(nk), 256, 0, s>>>(mdn, nk, big);
-        if (ntup <= sw.wcap) {
-          // the tuples' external energies once into W (free until the sector sources)
-          ++launch_counter();
-          k_sector_eext<<<launch_blocks(ntup), 256, 0, s>>>(eps_cv, w.dc, w.ed, d.c, sec, ntup,
-                                                            sw.W);
-          ++launch_counter();
-          k_mu_mindenom_ee<<<dim3((unsigned)std::min<long>((ntup + 255) / 256, 64), nk), 256, 0,
-                             s>>>(K.omega, E0, sw.W, n, Lsel, ntup, shift, mdn);
-        } else {
-          ++launch_counter();
-          k_mu_mindenom<<<dim3((unsigned)std::min<long>((ntup + 255) / 256, 64), nk), 256, 0,
-                          s>>>(K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, sec, Lsel, ntup, nk,
-                               shift, mdn);
-        }
-        CASPT2_CUDA_TRY(cudaGetLastError());
-        std::vector<double> hm(nk);
-        CASPT2_CUDA_TRY(cudaMemcpyAsync(hm.data(), mdn, sizeof(double) * nk, cudaMemcpyDeviceToHost, s));
-        CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
-        std::vector<int> list;
-        for (int k = 0; k < nk; ++k)
-          if (hm[k] < kRefineDenom) list.push_back(k);
-        if (!list.empty()) {
-          // list (ints) at the start of part2, the stage-1 partials in W (free here)
-          const int nl = (int)list.size();
-          const int nrb = (int)std::max<long>(1, std::min<long>(
-              {(long)(msec + 63) / 64, 1216L / nl + 1, sw.wcap / (4L * nl)}));
-          if ((long)nl > sw.p2size || 4L * nl * nrb > sw.wcap) return CASPT2_EINVAL;
-          int* dlist = reinterpret_cast<int*>(sw.part2);
-          CASPT2_CUDA_TRY(cudaMemcpyAsync(dlist, list.data(), sizeof(int) * nl,
-                                          cudaMemcpyHostToDevice, s));
-          ++launch_counter();
-          k_sector<<<launch_blocks(ms2), 256, 0, s>>>(w.Sact, m, n, sgn, Lsel, sw.Qs, msec);
-          ++launch_counter();
-          k_rq_partial<<<dim3(nrb, nl), kRqThreads, 0, s>>>(sw.Qs, sw.Fsec, msec, K.Y, nk, dlist,
-                                                           sw.W);
-          ++launch_counter();
-          k_rq_finish<<<(nl + 127) / 128, 128, 0, s>>>(sw.W, nrb, dlist, nl, K.omega);
-          CASPT2_CUDA_TRY(cudaGetLastError());
-          // eigenvectors: y_k += sum_j c_j y_j with the double-double residual of (F, S)
-          double* R = sw.W;                                  // [msec][nl]
-          double* Cm = R + (long)msec * nl;                  // [nk][nl]
-          double* Dl = Cm + (long)nk * nl;                   // [msec][nl]
-          if ((long)(2 * msec + nk) * nl > sw.wcap) return CASPT2_EINVAL;
-          ++launch_counter();
-          k_rq_resid<<<dim3(nrb, nl), kRqThreads, 0, s>>>(sw.Qs, sw.Fsec, msec, K.Y, nk, dlist, nl,
-                                                         K.omega, R);
-          CASPT2_CUDA_TRY(cudaGetLastError());
-          CASPT2_CUDA_TRY(dgemm(nk, nl, msec, 1.0, K.Y, nk, true, R, nl, false, 0.0, Cm, nl, s));
-          ++launch_counter();
-          k_rq_coef<<<launch_blocks((long)nk * nl), 256, 0, s>>>(Cm, nk, dlist, nl, K.omega);
-          CASPT2_CUDA_TRY(cudaGetLastError());
-          CASPT2_CUDA_TRY(dgemm(msec, nl, nk, 1.0, K.Y, nk, false, Cm, nl, false, 0.0, Dl, nl, s));
-          ++launch_counter();
-          k_rq_apply<<<launch_blocks((long)msec * nl), 256, 0, s>>>(K.Y, msec, nk, dlist, nl, Dl);
-          CASPT2_CUDA_TRY(cudaGetLastError());
-          CASPT2_CUDA_TRY(cudaStreamSynchronize(s));   // the host list is released below
-        }
-      }
-      const long ncol = ntup * n;
-      const int nL = Lsel < 0 ? n : 1;
-      const int pcol = nL * n * (n + 2);
-      // tuples in chunks so that the sector sources W (msec x chunk n) and the moment
-      // partials (chunk x pcol) stay within the work arrays the context holds
-      long chunk = std::min<long>(ntup, sw.wcap / ((long)msec * n));
-      chunk = std::min<long>(chunk, sw.pcap / pcol);
-      if (chunk < 1 || (long)nk * ncol > (1L << 62)) return CASPT2_EINVAL;
-      // class G under a closed-orbital range: the sector tuples are ordered with the
-      // closed index slowest, so the range is a contiguous run of them
-      long tb = 0, te = ntup;
-      if (w.cls == CASPT2_CLASS_G && (ci0 > 0 || (ci1 >= 0 && ci1 < d.c))) {
-        const long per_i = ntup / d.c;
-        tb = (long)ci0 * per_i;
-        te = (long)(ci1 < 0 || ci1 > d.c ? d.c : ci1) * per_i;
-      }
-      for (long t0 = tb; t0 < te; t0 += chunk) {
-        const long nt = std::min(chunk, te - t0);
-        ++launch_counter();
-        k_sector_src<<<launch_blocks((long)(scheme == CASPT2_SSSR ? msec : msec / n) * nt), 256, 0, s>>>(
-            w.V, w.dc, w.ed, d.a, n, sec, Lsel, t0, nt, msec, sw.W);
-        CASPT2_CUDA_TRY(cudaGetLastError());
-        if (oz && oz->on && oz->S >= kOzMaxSlices) {
-          // precision form with every product FP64-accurate (7 slices): the sector
-          // transform as a split-BF16 tensor-core product (fewer slices keep it in FP64:
-          // the energies are first order in its rounding)
-          const OzView vy{K.Y, 1, nk, msec, 0};               // rows mu, K = sector row
-          const OzView vw{sw.W, 1, nt * n, msec, 0};           // rows (t, L'), K = sector row
-          CASPT2_CUDA_TRY(oz_matmul(*oz, vy, vw, false, nk, (int)(nt * n), msec, 1.0, 0.0,
-                                    K.Vt + t0 * n, ncol, s));
-        } else {
-          CASPT2_CUDA_TRY(dgemm(nk, (int)(nt * n), msec, 1.0, K.Y, nk, true, sw.W,
-                                (int)(nt * n), false, 0.0, K.Vt + t0 * n, (int)ncol, s));
-        }
-        ++launch_counter();
-        if (n <= 4) {
-          k_sector_energy_ml<4><<<launch_blocks(nt * nL), 256, 0, s>>>(
-              K.Vt, K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, sec, Lsel, ntup, t0, nt, nk, shift,
-              sw.part, mindenom);
-        } else if (n <= 6) {
-          k_sector_energy_ml<6><<<launch_blocks(nt * nL), 256, 0, s>>>(
-              K.Vt, K.omega, E0, eps_cv, w.dc, w.ed, d.c, n, sec, Lsel, ntup, t0, nt, nk, shift,
-              sw.part, mindenom);
-        } else {
-          const long ne = nt * nL * n;
-          k_sector_energy<<<launch_blocks(ne), 256, 0, s>>>(K.Vt, K.omega, E0, eps_cv, w.dc, w.ed,
-                                                            d.c, n, sec, Lsel, ntup, t0, nt, nk,
-                                                            shift, sw.part, mindenom);
-        }
-        // fixed-order column sums: row blocks, then the block partials in order
-        const long nb = std::min<long>(sw.nb2, std::max<long>(1, nt / 64));
-        ++launch_counter();
-        k_colsum_rows<<<(unsigned)nb, 256, 0, s>>>(sw.part, nt, pcol, sw.part2);
-        ++launch_counter();
-        k_moment_colsum<<<pcol, 256, 0, s>>>(sw.part2, nb, n, nL, Lsel, mom);
-        CASPT2_CUDA_TRY(cudaGetLastError());
-      }
+      // fixed-order column sums: row blocks, then the block partials in order
+      const long nb = std::min<long>(sw.nb2, std::max<long>(1, nt / 64));
+      ++launch_counter();
+      k_colsum_rows<<<(unsigned)nb, 256, 0, s>>>(sw.part, nt, pcol, sw.part2);
+      ++launch_counter();
+      k_moment_colsum<<<pcol, 256, 0, s>>>(sw.part2, nb, n, nL, Lsel, mom);
+      CASPT2_CUDA_TRY(cudaGetLastError());
     }
   }
   return CASPT2_OK;

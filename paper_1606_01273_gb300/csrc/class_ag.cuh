@@ -5,6 +5,7 @@
 #include "kernels.cuh"
 #include "linalg.cuh"
 #include "ozaki.cuh"
+#include "sector_block.cuh"
 #include "terms.h"
 
 namespace caspt2 {
@@ -33,6 +34,8 @@ __device__ __forceinline__ void atomicMin_double(double* addr, double v) {
 struct SectorKeep {
   int sec = 0, Lsel = -1, msec = 0, nk = 0;
   long ntup = 0;
+  int job = -1;          // index in the one-launch sector batch (SectorBatch); -1: solved alone
+  long mdn = 0;          // offset of the sector's denominator minima
   double *Y = nullptr, *omega = nullptr, *Vt = nullptr;
 };
 
@@ -109,13 +112,39 @@ long class_sector_wsize(const ClassWork& w, const Dims& d, int scheme, long* par
 cudaError_t class_upload_plans(ClassWork& w, const std::vector<ActPlan>& S,
                                const std::vector<ActPlan>& F, const std::vector<SrcPlan>& V);
 
-// Evaluate S, F_act, V of a class and solve it; accumulates the moment sums
-// mom = [M1: n^3][M2: n^2][M3: n] (see k_sector_energy).
+// The small sectors of all classes, solved in one launch (sector_block.cuh): jobs in class
+// order, class k's at [first[k], first[k + 1]).
+struct SectorBatch {
+  std::vector<SectorJob> jobs;
+  SectorJob* dev = nullptr;
+  int* info = nullptr;               // device, 2 per job
+  std::vector<int> hinfo;
+  int first[8] = {};
+  double* mdn = nullptr;             // denominator minima of every kept eigenvector
+  std::vector<double> hmdn;
+};
+
+// Overlap and active Fock matrices of a class from the rotated RDMs.
+int class_matrices(ClassWork& w, const Dims& d, RdmPtrs rdm, const double* f_act,
+                   cudaStream_t s);
+// Sign of the pair-swap part in a sector's matrices (0: the class has no pair).
+double sector_sign(const ClassWork& w, int sec);
+// Eigenbasis (K.Y, K.omega, K.nk) of a sector that is not in the batch.
+int class_sector_basis(ClassWork& w, SectorKeep& K, SectorWork& sw, const Dims& d, double thresh,
+                       cudaStream_t s, KernelTimer* tm = nullptr, OzWork* oz = nullptr);
+// Smallest |e_ext + omega_mu - E0_L + E_s| of every kept eigenvector of a sector into
+// mdn[K.mdn ..] (filled with 1e300 by the caller).
+int class_sector_mindenom(const ClassWork& w, const SectorKeep& K, SectorWork& sw, const Dims& d,
+                          double shift, const double* E0, const double* eps_cv, double* mdn,
+                          cudaStream_t s);
+cudaError_t launch_fill(double* x, long n, double v, cudaStream_t s);
+// Sources of a class and its moment sums mom = [M1: n^3][M2: n^2][M3: n] (see
+// k_sector_energy) from the sectors' eigenbases; hmdn: host copy of the denominator minima.
 int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double shift,
-                double thresh, RdmPtrs rdm, const double* f, const double* h, const EriBlocks& eri,
-                const PresumBlocks& pb, const double* E0, const double* eps_cv, double* mom,
-                double* mindenom, cudaStream_t s, KernelTimer* tm = nullptr,
-                OzWork* oz = nullptr, int ci0 = 0, int ci1 = -1);
+                RdmPtrs rdm, const double* h, const EriBlocks& eri, const PresumBlocks& pb,
+                const double* E0, const double* eps_cv, const double* hmdn, double* mom,
+                double* mindenom, cudaStream_t s, OzWork* oz = nullptr, int ci0 = 0,
+                int ci1 = -1);
 // Doubles of a pre-summed block, and its evaluation from the (pq|rt) block of its spaces.
 long presum_size(const Dims& d, const PresumSpec& sp);
 cudaError_t presum_block(const Dims& d, const PresumSpec& sp, const double* src, double* out,
