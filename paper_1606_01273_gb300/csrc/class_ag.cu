@@ -489,15 +489,14 @@ __global__ void k_sector(const double* __restrict__ in, int m, int n, double sgn
 }
 
 // Eigenvalues ascending: the kept overlap directions are the last nk columns.
-// X[i][c] = Q[i * ldq + qoff + c] / sqrt(s[m - nk + c])   (m x nk, row-major)
-__global__ void k_range_basis(const double* __restrict__ Q, int ldq, int qoff,
-                              const double* __restrict__ s, int m, int nk,
-                              double* __restrict__ X) {
+// X[i][c] = Q[i][c] / sqrt(s[m - nk + c])   (m x nk, row-major)
+__global__ void k_range_basis(const double* __restrict__ Q, const double* __restrict__ s, int m,
+                              int nk, double* __restrict__ X) {
   const long total = (long)m * nk;
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
-    const int i = e / nk, c = e % nk;
-    X[e] = Q[(long)i * ldq + qoff + c] / sqrt(s[m - nk + c]);
+    const int c = e % nk;
+    X[e] = Q[e] / sqrt(s[m - nk + c]);
   }
 }
 
@@ -1251,15 +1250,13 @@ int class_sector_basis(ClassWork& w, SectorKeep& K, SectorWork& sw, const Dims& 
   K.nk = 0;
   OzWork* ozn = (oz && oz->on && oz->S >= kOzMaxSlices) ? oz : nullptr;
   // eigenvalues of the overlap and the eigenvectors of those at or above the threshold
-  int nk = 0, ldq = 0, qoff = 0;
-  int st = sym_eig_above(sw.Ssec, msec, thresh, sw.s, sw.Qs, &nk, &ldq, &qoff, sw.jac, s, tm,
-                         ozn);
+  int nk = 0;
+  int st = sym_eig_above(sw.Ssec, msec, thresh, sw.s, sw.Qs, &nk, sw.jac, s, tm, ozn);
   if (st != CASPT2_OK) return st;
   if (nk == 0) return CASPT2_OK;
   K.nk = nk;
   ++launch_counter();
-  k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, ldq, qoff, sw.s, msec,
-                                                               nk, sw.X);
+  k_range_basis<<<launch_blocks((long)msec * nk), 256, 0, s>>>(sw.Qs, sw.s, msec, nk, sw.X);
   CASPT2_CUDA_TRY(cudaGetLastError());
   const bool ozx = oz && oz->on && oz->S >= kOzMaxSlices && msec >= kOzTransformMin;
   if (ozx) {

@@ -5,6 +5,21 @@
 
 namespace caspt2 {
 
+// Where only the eigenvectors at or above a cut wmin are returned, those of the eigenvalues
+// down to this bound are formed and orthogonalised with them: vectors from inverse iteration
+// overlap by about eps ||T|| / gap, so a kept vector would carry 1e-9 of a dropped one a gap
+// of 1e-6 below it.  What lies below 1e-4 of the cut has an overlap norm smaller by as much;
+// what lies within the rounding of zero is the null space, which enters nothing.
+__host__ __device__ inline double eig_guard(double wmin, double tnorm) {
+  const double g = fmax(1e-4 * wmin, 1e-14 * tnorm);
+  return g < wmin ? g : wmin;
+}
+
+// Bracket width at which an eigenvalue is taken (times max(1, ||T||)): half an FP64 rounding,
+// so that the search adds nothing to the rounding of T.  The overlap's small eigenvalues
+// normalise the range basis, s^(-1/2): at s = 1e-6 one rounding of ||T|| = 10 is 2e-9 of s.
+constexpr double kEigTol = 1.1e-16;
+
 __device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
 __device__ __forceinline__ unsigned long long abits(double v) {   // |v| as an ordered integer
   return (unsigned long long)dbits(v) & 0x7FFFFFFFFFFFFFFFull;
@@ -125,19 +140,24 @@ __device__ __forceinline__ double eigenvalue_f64(const double* __restrict__ d,
       --todo;
       if (!(x > lo && x < hi)) continue;
     } else {
-      if (hi - lo <= tol || hi < wmin) break;
+      // least distance of a point from the ends: a rounding of theirs where tol is below it
+      const double ulp = 2.3e-16 * fmax(fabs(lo), fabs(hi)), step = fmax(0.75 * tol, ulp);
+      if (hi - lo <= fmax(tol, ulp) || hi < wmin) break;
       x = 0.5 * (lo + hi);
-      if (klo && khi && ch - cl == 1) {
+      if (klo && khi && ch - cl == 1 && it < 60) {
         if ((sec & 3) == 0) {
           if (sec > 0 && hi - lo > 0.125 * wide) sec = -1;     // this step halves
           wide = hi - lo;
         }
         if (sec >= 0) {
-          double t;                              // vlo / (vlo - vhi), exponents apart
-          if (xlo == xhi) t = vlo / (vlo - vhi);
-          else t = xlo > xhi ? 1.0 : 0.0;
+          // vlo / (vlo - vhi); the ends' exponents may differ by a rescaling step
+          double a = vlo, b = vhi;
+          if (xlo > xhi) { a *= 0x1p250; b *= 0x1p-250; }
+          else if (xlo < xhi) { a *= 0x1p-250; b *= 0x1p250; }
+          const double t = abs(xlo - xhi) <= 1 ? a / (a - b) : (xlo > xhi ? 1.0 : 0.0);
           x = fma(t, hi - lo, lo);
-          x = fmin(fmax(x, lo + 0.75 * tol), hi - 0.75 * tol);
+          x = fmin(fmax(x, lo + step), hi - step);
+          if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
         }
         ++sec;
       }
@@ -155,6 +175,72 @@ __device__ __forceinline__ double eigenvalue_f64(const double* __restrict__ d,
       kept = kept < 0 ? kept - 1 : -1;
       if (kept < -1) vhi *= 0.5;
     }
+  }
+  return 0.5 * (lo + hi);
+}
+
+// The same by an aligned group of eight lanes, for matrices whose eigenvalues leave the FP64
+// units of other sub-partitions idle: every pass evaluates seven points at the latency of
+// one.  While the bracket holds several eigenvalues they are its eighth points; once it
+// holds one they lie around the secant point, at the least step and at the two geometric means
+// between that and the width, with the midpoint: about three passes after the isolation.
+// Every lane of the group calls it with the same j; the result is the group's.
+__device__ __forceinline__ double eigenvalue_f64_group(const double* __restrict__ d,
+                                                       const double* __restrict__ e2, int m,
+                                                       int j, double glo, double ghi, double flo,
+                                                       double fhi, double tol, double wmin) {
+  const unsigned grp = 0xFFu << (threadIdx.x & 24);
+  const int q = threadIdx.x & 7;
+  double lo = glo, hi = ghi, vlo = 0.0, vhi = 0.0;
+  int cl = 0, ch = m, xlo = 0, xhi = 0;
+  bool klo = false, khi = false;
+  const bool f32 = f32_usable(glo, ghi);
+  const double gap = f32_gap(glo, ghi);
+  for (int it = f32 ? -1 : 0; it < 60; ++it) {
+    double x;
+    bool use;
+    if (it < 0) {                                // the single-precision bracket, widened
+      x = q == 0 ? flo - gap : fhi + gap;
+      use = q < 2;
+    } else {
+      const double ulp = 2.3e-16 * fmax(fabs(lo), fabs(hi)), step = fmax(0.75 * tol, ulp);
+      const double width = hi - lo;
+      if (width <= fmax(tol, ulp) || hi < wmin) break;
+      if (klo && khi && ch - cl == 1 && it < 40) {
+        double a = vlo, b = vhi;                 // exponents may differ by a rescaling step
+        if (xlo > xhi) { a *= 0x1p250; b *= 0x1p-250; }
+        else if (xlo < xhi) { a *= 0x1p-250; b *= 0x1p250; }
+        const double t = abs(xlo - xhi) <= 1 ? a / (a - b) : (xlo > xhi ? 1.0 : 0.0);
+        const double xs = fma(t, width, lo);
+        const float l0 = log2f((float)step), l1 = log2f((float)width);
+        const int lev = q >> 1;                  // 0, 1, 2 (two lanes each), 3: midpoint
+        const double off = lev == 0 ? step
+                                    : (double)exp2f(l0 + (l1 - l0) * (float)lev * (1.f / 3.f));
+        x = lev == 3 ? lo + 0.5 * width : (q & 1 ? xs + off : xs - off);
+      } else {
+        x = lo + 0.125 * width * (q + 1);
+      }
+      use = q < 7;
+    }
+    use = use && x > lo && x < hi;
+    double v = 0.0;
+    int ex = 0, c = 0;
+    if (use) c = sturm_value(d, e2, m, x, v, ex);
+    __syncwarp(grp);
+    bool moved = false;
+#pragma unroll
+    for (int r = 0; r < 7; ++r) {
+      const double xr = __shfl_sync(grp, x, r, 8), vr = __shfl_sync(grp, v, r, 8);
+      const int cr = __shfl_sync(grp, c, r, 8), er = __shfl_sync(grp, ex, r, 8);
+      const bool ur = __shfl_sync(grp, use ? 1 : 0, r, 8) != 0;
+      if (!ur) continue;
+      if (cr > j) {
+        if (xr < hi) { hi = xr; ch = cr; vhi = vr; xhi = er; khi = true; moved = true; }
+      } else if (xr > lo) {
+        lo = xr; cl = cr; vlo = vr; xlo = er; klo = true; moved = true;
+      }
+    }
+    if (!moved && it >= 0) break;                // no representable point left inside
   }
   return 0.5 * (lo + hi);
 }

@@ -1,11 +1,12 @@
 // FP64 symmetric eigensolver for the per-class overlap and Fock matrices
-// (Sec. II.B: eigenvalues of the overlap below the threshold are truncated):
+// (Sec. II.B: eigenvalues of the overlap below the threshold are truncated) above the size
+// that one block solves (sector_block.cu):
 //   1. Householder reduction to tridiagonal form, T = Q^T A Q (one reflector per step:
 //      p = tau A22 v, w = p - (tau/2)(p.v) v, A22 -= v w^T + w v^T);
-//   2. every eigenvalue of T by bisection on Sturm counts (one thread per eigenvalue,
-//      absolute accuracy ~ eps ||T||);
-//   3. every eigenvector of T by inverse iteration on the pivoted tridiagonal LU
-//      (one thread per eigenvalue), Gram-Schmidt inside clusters of equal eigenvalues;
+//   2. every eigenvalue of T from Sturm counts and minors (eig_dev.cuh, absolute accuracy
+//      ~ eps ||T||);
+//   3. eigenvectors of T by inverse iteration on the pivoted tridiagonal LU (one thread per
+//      eigenvalue), Gram-Schmidt inside clusters of equal eigenvalues;
 //   4. one Newton-Schulz step Z <- Z (3 - Z^T Z) / 2 to restore orthogonality to
 //      rounding level (skipped when Z^T Z is already within 1e-13 of the identity);
 //   5. back-transformation V = Q Z by applying the reflectors in reverse order.
@@ -13,6 +14,7 @@
 #include <vector>
 
 #include "class_ag.cuh"
+#include "eig_dev.cuh"
 #include "ozaki.cuh"
 #include "linalg.cuh"
 
@@ -28,81 +30,6 @@ int nblocks(long total, int threads = kT) {
 }
 
 }  // namespace
-
-// Reflector for column k: x = A[k][k+1..m-1] (row k, symmetric storage).
-// v is stored in vbuf[k*m + k+1 ..] with v[k+1] = 1; tau[k]; d[k] = A[k][k]; e[k] = beta.
-__global__ void k_house(double* __restrict__ A, int m, int k, double* __restrict__ vbuf,
-                        double* __restrict__ tau, double* __restrict__ d, double* __restrict__ e) {
-  __shared__ double red[32];
-  __shared__ double sh[2];
-  const double* x = A + (long)k * m + k + 1;
-  const int n1 = m - k - 1;
-  double s = 0.0;
-  for (int i = 1 + threadIdx.x; i < n1; i += blockDim.x) s += x[i] * x[i];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) {
-    const double alpha = x[0];
-    double beta, t, scale;
-    if (s == 0.0) {
-      beta = alpha;
-      t = 0.0;
-      scale = 0.0;
-    } else {
-      beta = -copysign(sqrt(alpha * alpha + s), alpha);
-      t = (beta - alpha) / beta;
-      scale = 1.0 / (alpha - beta);
-    }
-    sh[0] = t;
-    sh[1] = scale;
-    tau[k] = t;
-    d[k] = A[(long)k * m + k];
-    e[k] = beta;
-  }
-  __syncthreads();
-  const double scale = sh[1];
-  double* v = vbuf + (long)k * m + k + 1;
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) v[i] = (i == 0) ? 1.0 : x[i] * scale;
-}
-
-// p[i] = tau * sum_j A22[i][j] v[j], one warp per row of the trailing block
-__global__ void k_symv(const double* __restrict__ A, int m, int k, const double* __restrict__ vbuf,
-                       const double* __restrict__ tau, double* __restrict__ p) {
-  const int n1 = m - k - 1;
-  const double* v = vbuf + (long)k * m + k + 1;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  const double t = tau[k];
-  for (int i = warp; i < n1; i += nw) {
-    const double* row = A + (long)(k + 1 + i) * m + k + 1;
-    double s = 0.0;
-    for (int j = lane; j < n1; j += 32) s += row[j] * v[j];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) p[i] = t * s;
-  }
-}
-
-// A22 -= v w^T + w v^T with w = p - (tau/2)(p.v) v  (each block recomputes p.v)
-__global__ void k_rank2(double* __restrict__ A, int m, int k, const double* __restrict__ vbuf,
-                        const double* __restrict__ tau, const double* __restrict__ p) {
-  __shared__ double red[32];
-  __shared__ double sg;
-  const int n1 = m - k - 1;
-  const double* v = vbuf + (long)k * m + k + 1;
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) s += p[i] * v[i];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) sg = 0.5 * tau[k] * s;
-  __syncthreads();
-  const double g = sg;
-  const long total = (long)n1 * n1;
-  for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < total;
-       t += (long)gridDim.x * blockDim.x) {
-    const int i = t / n1, j = t % n1;
-    const double wi = p[i] - g * v[i], wj = p[j] - g * v[j];
-    A[(long)(k + 1 + i) * m + k + 1 + j] -= v[i] * wj + wi * v[j];
-  }
-}
 
 // Grid-wide barrier for a cooperative launch, bounded: after kSpinLimit polls it sets
 // *err and returns false so that every block can leave the kernel.
@@ -139,87 +66,6 @@ __device__ bool grid_sync_bounded(unsigned* count, volatile unsigned* gen, int* 
   }
   __syncthreads();
   return ok != 0;
-}
-
-// Reflector of row k from its trailing part (one block): tau, d[k], e[k] = beta, v.
-__device__ void house_row(double* __restrict__ A, int m, int k, double* __restrict__ vbuf,
-                          double* __restrict__ tau, double* __restrict__ d,
-                          double* __restrict__ e, double* red, double* sh) {
-  const int n1 = m - k - 1;
-  const double* x = A + (long)k * m + k + 1;
-  double s = 0.0;
-  for (int i = 1 + threadIdx.x; i < n1; i += blockDim.x) s += __ldcg(x + i) * __ldcg(x + i);
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) {
-    const double alpha = __ldcg(x);
-    double beta, t, scale;
-    if (s == 0.0) { beta = alpha; t = 0.0; scale = 0.0; }
-    else {
-      beta = -copysign(sqrt(alpha * alpha + s), alpha);
-      t = (beta - alpha) / beta;
-      scale = 1.0 / (alpha - beta);
-    }
-    sh[1] = scale;
-    tau[k] = t;
-    d[k] = __ldcg(A + (long)k * m + k);
-    e[k] = beta;
-  }
-  __syncthreads();
-  const double scale = sh[1];
-  double* v = vbuf + (long)k * m + k + 1;
-  for (int i = threadIdx.x; i < n1; i += blockDim.x) v[i] = (i == 0) ? 1.0 : __ldcg(x + i) * scale;
-  __syncthreads();
-}
-
-// Householder reduction in one cooperative launch, two bounded grid barriers per step:
-//   p = tau A22 v (warps over rows)                              | barrier
-//   A22 -= v w^T + w v^T; block 0 then forms the next reflector   | barrier
-// from row k+1, which its warp 0 has just finished updating.
-// sync[0..1] barrier state (zeroed by the host), sync[2] error flag.
-__global__ void __launch_bounds__(512)
-k_tridiag(double* __restrict__ A, int m, double* __restrict__ vbuf, double* __restrict__ tau,
-          double* __restrict__ d, double* __restrict__ e, double* __restrict__ p,
-          unsigned* sync) {
-  __shared__ double red[32];
-  __shared__ double sh[2];
-  int* err = reinterpret_cast<int*>(sync + 2);
-  if (blockIdx.x == 0) house_row(A, m, 0, vbuf, tau, d, e, red, sh);
-  if (!grid_sync_bounded(sync, sync + 1, err)) return;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int k = 0; k + 2 < m; ++k) {
-    const int n1 = m - k - 1;
-    const double* v = vbuf + (long)k * m + k + 1;
-    const double t = __ldcg(tau + k);
-    for (int i = warp; i < n1; i += nw) {
-      const double* row = A + (long)(k + 1 + i) * m + k + 1;
-      double s = 0.0;
-      for (int j = lane; j < n1; j += 32) s += __ldcg(row + j) * __ldcg(v + j);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) p[i] = t * s;
-    }
-    if (!grid_sync_bounded(sync, sync + 1, err)) return;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n1; i += blockDim.x) s += __ldcg(p + i) * __ldcg(v + i);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) sh[0] = 0.5 * t * s;
-    __syncthreads();
-    const double g = sh[0];
-    for (int i = warp; i < n1; i += nw) {
-      const double vi = __ldcg(v + i), wi = __ldcg(p + i) - g * vi;
-      double* row = A + (long)(k + 1 + i) * m + k + 1;
-      for (int j = lane; j < n1; j += 32) {
-        const double vj = __ldcg(v + j), wj = __ldcg(p + j) - g * vj;
-        row[j] = __ldcg(row + j) - (vi * wj + wi * vj);
-      }
-    }
-    if (blockIdx.x == 0 && k + 3 < m) {
-      __syncthreads();
-      house_row(A, m, k + 1, vbuf, tau, d, e, red, sh);
-    }
-    if (!grid_sync_bounded(sync, sync + 1, err)) return;
-  }
 }
 
 // Blocked Householder reduction, one cooperative launch per panel of b columns
@@ -565,80 +411,19 @@ __global__ void k_tail(const double* __restrict__ A, int m, double* d, double* e
   e[m - 1] = 0.0;
 }
 
-// Sturm count: number of eigenvalues of T below x
-__device__ int sturm(const double* __restrict__ d, const double* __restrict__ e2, int m, double x,
-                     double pivmin) {
-  int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  if (q < 0.0) ++cnt;
-  for (int i = 1; i < m; ++i) {
-    q = d[i] - x - e2[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0.0) ++cnt;
-  }
-  return cnt;
-}
-
 __global__ void k_e2(const double* __restrict__ e, int m, double* __restrict__ e2) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < m) e2[i] = (i < m - 1) ? e[i] * e[i] : 0.0;
 }
 
-// Number of eigenvalues of T below x from the sign changes of the leading principal
-// minors p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (p_{-1} = 1): three FP64 operations
-// per step and no division.  Signs, exact zeros (which take the sign opposite to their
-// predecessor) and the range check are integer operations on the bit patterns; the pair
-// (p_i, p_{i-1}) is rescaled by 2^(-+500) when |p_i| leaves [2^-600, 2^600], checked every
-// 4 steps (|p| grows by at most (2||T|| + ||T||^2) per step, far inside the FP64 range).
-__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
-
-__device__ int sturm_nodiv(const double* __restrict__ d, const double* __restrict__ e2, int m,
-                           double x) {
-  double pm = 1.0, pc = d[0] - x;
-  if ((dbits(pc) << 1) == 0) pc = -1e-300;
-  int cnt = (int)((unsigned long long)dbits(pc) >> 63);
-  for (int i = 1; i < m; ++i) {
-    double pn = fma(d[i] - x, pc, -e2[i - 1] * pm);
-    const long long bn = dbits(pn), bc = dbits(pc);
-    if ((bn << 1) == 0) pn = bc < 0 ? 1e-300 : -1e-300;
-    cnt += (int)((unsigned long long)(dbits(pn) ^ bc) >> 63);
-    pm = pc;
-    pc = pn;
-    if ((i & 3) == 0) {
-      const int ex = (int)((dbits(pc) >> 52) & 0x7FF);
-      const int exm = (int)((dbits(pm) >> 52) & 0x7FF);
-      if (ex > 1023 + 600) { pc *= 0x1p-500; pm *= 0x1p-500; }
-      else if (ex < 1023 - 600 && exm < 1023 - 600) { pc *= 0x1p500; pm *= 0x1p500; }
-    }
-  }
-  return cnt;
-}
-
-// Sturm count in single precision by the ratio recurrence q_i = d_i - x - e_(i-1)^2 / q_(i-1)
-// (q raised to -pivmin where it vanishes): the count is exact for a tridiagonal matrix whose
-// elements carry relative errors of a few float roundings, so it brackets every eigenvalue
-// to within a few 2^-24 tnorm.
-__device__ int sturm_f32(const float* __restrict__ d, const float* __restrict__ e2, int m, float x,
-                         float pivmin) {
-  float q = d[0] - x;
-  if (fabsf(q) < pivmin) q = -pivmin;
-  int cnt = q < 0.f ? 1 : 0;
-  for (int i = 1; i < m; ++i) {
-    q = (d[i] - x) - __fdividef(e2[i - 1], q);
-    if (fabsf(q) < pivmin) q = -pivmin;
-    cnt += q < 0.f ? 1 : 0;
-  }
-  return cnt;
-}
-
-// j-th smallest eigenvalue by 4-way multisection inside the Gershgorin interval: four
-// lanes per eigenvalue evaluate the Sturm count at the three interior quarter points
-// (lane 3 idles), so each step removes two bits; stop at an absolute width of tol.
-__global__ void k_bisect(const double* __restrict__ dg, const double* __restrict__ e,
-                         const double* __restrict__ e2g, int m, double glo, double ghi, double tol,
-                         double* __restrict__ w) {
-  extern __shared__ double sde[];      // d[m], e2[m] staged per block (and float copies)
+// Eigenvalues of T, eight lanes each: single-precision brackets, then FP64 (eig_dev.cuh).
+// A warp's FP64 instruction occupies its sub-partition for 64 clocks, so the number of
+// Sturm evaluations one after the other decides: 4 to 7 in place of the 12 passes of an FP64
+// octasection.  Dynamic shared memory: d, e^2 and their float copies.
+__global__ void k_eigenvalues(const double* __restrict__ dg, const double* __restrict__ e2g,
+                              int m, double glo, double ghi, double tol, double wmin,
+                              double* __restrict__ w) {
+  extern __shared__ double sde[];
   float* sdf = reinterpret_cast<float*>(sde + 2 * m);
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     sde[i] = dg[i];
@@ -647,208 +432,26 @@ __global__ void k_bisect(const double* __restrict__ dg, const double* __restrict
     sdf[m + i] = (float)e2g[i];
   }
   __syncthreads();
-  const double* d = sde;
-  const double* e2 = sde + m;
-  // eight lanes per eigenvalue: lanes 0..6 count at the seven interior eighth points of
-  // the bracket (three bits per pass); one Sturm chain per lane, many warps, so that every
-  // SM sub-partition's FP64 unit has work
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = gid >> 3, q = gid & 7;
-  const unsigned sh = threadIdx.x & 24;
-  const unsigned grp = 0xFFu << sh;
-  if ((gid & ~7) >= (m << 3)) return;          // whole group beyond m
-  const bool live = j < m;
-  double lo = glo, hi = ghi;
-  // single-precision phase (the float units run many times the FP64 rate): octasection to
-  // a width of 64 float roundings of the norm, then the bracket widened by as much and
-  // checked with two FP64 counts (the full interval again if it fails)
-  const double span = fmax(fabs(glo), fabs(ghi));
-  const double fgap = 64.0 * 0x1p-24 * span;
-  if (span > 0.0 && span < 1e30 && ghi - glo > 4.0 * fgap) {
-    const float pivmin = (float)fmax(1e-30, 0x1p-24 * 1e-8 * span);
-    float flo = (float)glo, fhi = (float)ghi;
-    for (int it = 0; it < 40; ++it) {
-      if ((double)fhi - (double)flo <= fgap) break;
-      const float h = 0.125f * (fhi - flo);
-      const float x = flo + h * (float)(q + 1);
-      const bool above = live && q < 7 && x > flo && x < fhi &&
-                         sturm_f32(sdf, sdf + m, m, x, pivmin) > j;
-      const unsigned b = (__ballot_sync(grp, above) >> sh) & 0x7Fu;
-      const int first = b ? (__ffs(b) - 1) : 7;
-      const float nhi = first < 7 ? flo + h * (float)(first + 1) : fhi;
-      const float nlo = first > 0 ? flo + h * (float)first : flo;
-      if (!(nhi < fhi || nlo > flo)) break;
-      flo = nlo;
-      fhi = nhi;
-    }
-    const double clo = fmax(glo, (double)flo - fgap), chi = fmin(ghi, (double)fhi + fgap);
-    // lane 0 checks count(clo) <= j, lane 1 count(chi) > j
-    bool good = true;
-    if (live && q < 2) {
-      const int cnt = sturm_nodiv(d, e2, m, q == 0 ? clo : chi);
-      good = q == 0 ? (clo <= glo || cnt <= j) : (chi >= ghi || cnt > j);
-    }
-    const unsigned bad = (__ballot_sync(grp, !good) >> sh) & 0x3u;
-    if (!bad) {
-      lo = clo;
-      hi = chi;
-    }
-  }
-  for (int it = 0; it < 60; ++it) {
-    if (hi - lo <= tol) break;
-    const double h = 0.125 * (hi - lo);
-    const double x = lo + h * (q + 1);
-    const bool above = live && q < 7 && x > lo && x < hi && sturm_nodiv(d, e2, m, x) > j;
-    const unsigned b = (__ballot_sync(grp, above) >> sh) & 0x7Fu;
-    const int first = b ? (__ffs(b) - 1) : 7;           // first eighth point above j
-    const double nhi = first < 7 ? lo + h * (first + 1) : hi;
-    const double nlo = first > 0 ? lo + h * first : lo;
-    if (!(nhi < hi || nlo > lo)) break;
-    lo = nlo;
-    hi = nhi;
-  }
-  if (live && q == 0) w[j] = 0.5 * (lo + hi);
+  const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+  const int j = min(g, m - 1);
+  float flo, fhi;
+  bisect_f32(sdf, sdf + m, m, j, glo, ghi, flo, fhi);
+  const double x = eigenvalue_f64_group(sde, sde + m, m, j, glo, ghi, flo, fhi, tol, wmin);
+  if (g < m && (threadIdx.x & 7) == 0) w[g] = x;
 }
 
-__device__ __forceinline__ double hash_unit(unsigned a, unsigned b) {
-  unsigned h = a * 0x9E3779B1u ^ (b + 0x7F4A7C15u) * 0x85EBCA77u;
-  h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
-  return (double)(h & 0xFFFFFF) / 16777216.0 + 0.5;   // in [0.5, 1.5)
-}
-
-// Inverse iteration for the nc eigenvalues w[0..nc) (thread j).  Scratch arrays are laid
-// out [i][j] so that threads access consecutive addresses.  Z[i][j] = component i of vector j.
+// Inverse iteration for the nc eigenvalues w[0..nc) (thread j, eig_dev.cuh); scr as there.
 __global__ void k_inviter(const double* __restrict__ dg, const double* __restrict__ eg,
                           const double* __restrict__ w, int m, int nc, double tnorm,
-                          double* __restrict__ u0, double* __restrict__ u1,
-                          double* __restrict__ u2, double* __restrict__ lm,
-                          double* __restrict__ pv, double* __restrict__ Z) {
+                          double* __restrict__ scr, double* __restrict__ Z) {
   extern __shared__ double sde[];      // d[m], e[m] staged per block
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
     sde[i] = dg[i];
     sde[m + i] = eg[i];
   }
   __syncthreads();
-  const double* d = sde;
-  const double* e = sde + m;
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= nc) return;
-  const double lam = w[j];
-  const double tiny = 2.2e-16 * (tnorm > 0 ? tnorm : 1.0);
-#define IX(i) ((long)(i) * nc + j)
-  // Factor T - lam I = P L U (U with two superdiagonals), the current row carried in
-  // registers; rows are final once passed, so their pivots are stored as reciprocals
-  // (|pivot| raised to tiny) and the solves below multiply.
-  auto raise = [&](double piv, double rp) {   // reciprocal of the pivot raised to tiny
-    return fabs(piv) < tiny ? 1.0 / copysign(tiny, piv == 0.0 ? 1.0 : piv) : rp;
-  };
-  double a = d[0] - lam, b = m > 1 ? e[0] : 0.0;
-  for (int i = 0; i < m - 1; ++i) {
-    const double c = e[i];          // subdiagonal element of row i+1
-    const double an = d[i + 1] - lam, bn = (i + 1 < m - 1) ? e[i + 1] : 0.0;
-    if (fabs(a) >= fabs(c)) {
-      const double piv = (a == 0.0) ? tiny : a;
-      const double rp = 1.0 / piv;
-      const double l = c * rp;
-      u0[IX(i)] = raise(piv, rp);
-      u1[IX(i)] = b;
-      u2[IX(i)] = 0.0;
-      lm[IX(i)] = l;
-      pv[IX(i)] = 0.0;
-      a = an - l * b;
-      b = bn;
-    } else {
-      const double rp = 1.0 / c;
-      const double l = a * rp;
-      u0[IX(i)] = raise(c, rp);
-      u1[IX(i)] = an;
-      u2[IX(i)] = bn;
-      lm[IX(i)] = l;
-      pv[IX(i)] = 1.0;
-      a = b - l * an;
-      b = -l * bn;
-    }
-  }
-  {
-    const double piv = a == 0.0 ? tiny : a;
-    u0[IX(m - 1)] = raise(piv, 1.0 / piv);
-  }
-  u1[IX(m - 1)] = 0.0;
-  u2[IX(m - 1)] = 0.0;
-  // three inverse iterations from a fixed start vector; the normalisation of each
-  // iterate is folded into the next forward pass.  Both passes go in chunks of eight
-  // rows whose operands are loaded before the dependent chain runs through them.
-  constexpr int CH = 8;
-  double scale = 1.0;
-  for (int iter = 0; iter < 3; ++iter) {
-    // apply L^-1 with the row interchanges
-    double cur = iter == 0 ? hash_unit(0, j) : Z[IX(0)] * scale;
-    for (int i0 = 0; i0 < m - 1; i0 += CH) {
-      const int cnt = min(CH, m - 1 - i0);
-      double yv[CH], lv[CH], pq[CH];
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        if (u < cnt) {
-          const int i = i0 + u;
-          yv[u] = iter == 0 ? hash_unit(i + 1, j) : Z[IX(i + 1)] * scale;
-          lv[u] = lm[IX(i)];
-          pq[u] = pv[IX(i)];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        if (u < cnt) {
-          double yn = yv[u];
-          if (pq[u] != 0.0) {
-            const double t = cur; cur = yn; yn = t;
-          }
-          Z[IX(i0 + u)] = cur;
-          cur = yn - lv[u] * cur;
-        }
-      }
-    }
-    // U^-1 with overflow guard (x1 = x_{i+1}, x2 = x_{i+2})
-    double big = 0.0, nrm = 0.0, x1 = 0.0, x2 = 0.0;
-    for (int i0 = m - 1; i0 >= 0; i0 -= CH) {
-      const int cnt = min(CH, i0 + 1);
-      double zv[CH], a0[CH], a1[CH], a2[CH];
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        if (u < cnt) {
-          const int i = i0 - u;
-          zv[u] = i == m - 1 ? cur : Z[IX(i)];
-          a0[u] = u0[IX(i)];
-          a1[u] = u1[IX(i)];
-          a2[u] = u2[IX(i)];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < CH; ++u) {
-        if (u < cnt) {
-          const int i = i0 - u;
-          double x = zv[u];
-          x -= a1[u] * x1;
-          x -= a2[u] * x2;
-          x *= a0[u];
-          Z[IX(i)] = x;
-          nrm += x * x;
-          x2 = x1;
-          x1 = x;
-          big = fmax(big, fabs(x));
-          if (big > 1e100) {  // rescale the partial solution
-            for (int k2 = i; k2 < m; ++k2) Z[IX(k2)] *= 1e-100;
-            big *= 1e-100;
-            nrm *= 1e-200;
-            x1 *= 1e-100;
-            x2 *= 1e-100;
-          }
-        }
-      }
-    }
-    scale = 1.0 / sqrt(nrm);
-  }
-  for (int i = 0; i < m; ++i) Z[IX(i)] *= scale;
-#undef IX
+  if (j < nc) inverse_iteration(sde, sde + m, m, w[j], tnorm, nc, j, scr, Z);
 }
 
 // Orthonormalise each cluster of close eigenvalues (w sorted): the block of the cluster's
@@ -1124,62 +727,102 @@ k_backtransform_smem(const double* __restrict__ vbuf, const double* __restrict__
   }
 }
 
-// Compact WY form of a panel of reflectors (Schreiber and Van Loan): H_k0 ... H_k0+b-1 =
+// Compact WY form of the panels of reflectors (Schreiber and Van Loan): H_k0 ... H_k0+b-1 =
 // I - Vp T Vp^T with T upper triangular, T_ii = tau_i and
-// T_{j,i} = -tau_i sum_{l = j..i-1} T_{j,l} (v_l . v_i) (j < i).  One block of b threads;
-// Gp[l][i] = v_{k0+l} . v_{k0+i}.
-__global__ void k_wy_T(const double* __restrict__ Gp, const double* __restrict__ tau, int k0,
-                       int b, double* __restrict__ T) {
-  const int j = threadIdx.x;
+// T_{j,i} = -tau_i sum_{l = j..i-1} T_{j,l} (v_l . v_i) (j < i).  One block per panel of nb
+// reflectors (the last one shorter), all panels at once; G[panel][l][i] = v_l . v_i is
+// overwritten by T.  Column i of G is needed at step i only, so T takes its place in shared
+// memory; eight lanes a row.  (One block of b threads a panel, each with a serial sum over
+// global memory, took 0.51 ms a panel, one panel after the other.)
+constexpr int kWyPanel = 128;       // reflectors per compact-WY panel
+__global__ void __launch_bounds__(256)
+k_wy_T(double* __restrict__ G, const double* __restrict__ tau, int nref) {
+  extern __shared__ double t[];
+  constexpr int nb = kWyPanel, ld = nb + 1;
+  const int k0 = blockIdx.x * nb, b = min(nb, nref - k0);
+  double* Gp = G + (long)blockIdx.x * nb * nb;
+  for (int q = threadIdx.x; q < b * b; q += blockDim.x) t[(q / b) * ld + q % b] = Gp[(q / b) * nb + q % b];
+  __syncthreads();
+  const int sub = threadIdx.x & 7;
   for (int i = 0; i < b; ++i) {
-    double acc = 0.0;
-    if (j < i)
-      for (int l = j; l < i; ++l) acc = fma(T[j * b + l], Gp[l * b + i], acc);
+    const double ti = tau[k0 + i];
+    double res[nb / 32];
+#pragma unroll
+    for (int r = 0; r < nb / 32; ++r) {
+      const int j = r * 32 + (threadIdx.x >> 3);
+      double s0 = 0.0, s1 = 0.0;
+      if (j < i) {
+        int l = j + sub;
+        for (; l + 8 < i; l += 16) {
+          s0 = fma(t[j * ld + l], t[l * ld + i], s0);
+          s1 = fma(t[j * ld + l + 8], t[(l + 8) * ld + i], s1);
+        }
+        if (l < i) s0 = fma(t[j * ld + l], t[l * ld + i], s0);
+      }
+      res[r] = 0.0;
+      if (r * 32 + (threadIdx.x >> 5) * 4 < i) {        // whole warps
+        double s = s0 + s1;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        res[r] = -ti * s;
+      }
+    }
     __syncthreads();
-    if (j < i) T[j * b + i] = -tau[k0 + i] * acc;
-    else if (j == i) T[j * b + i] = tau[k0 + i];
-    else if (j < b) T[j * b + i] = 0.0;
+#pragma unroll
+    for (int r = 0; r < nb / 32; ++r) {
+      const int j = r * 32 + (threadIdx.x >> 3);
+      if (sub == 0 && j < b) t[j * ld + i] = j < i ? res[r] : (j == i ? ti : 0.0);
+    }
     __syncthreads();
   }
+  for (int q = threadIdx.x; q < b * b; q += blockDim.x) Gp[(q / b) * nb + q % b] = t[(q / b) * ld + q % b];
 }
 
 size_t sym_eig_tridiag_work(int m) { return (size_t)m * m * 9 + (size_t)m * 8 + 64; }
 
 namespace {
-constexpr int kWyPanel = 128;       // reflectors per compact-WY panel
 constexpr int kWyMinSize = 1024;    // blocked back-transformation from this size up
 
 // V <- H_0 H_1 ... H_{m-3} V as panels P_j = I - Vp T Vp^T applied last panel first:
 // W = Vp^T V (rows below the panel start), W <- T W, V -= Vp W, three FP64 GEMMs per
 // panel.  vbuf rows hold the reflectors with zeros left of their first entry, so a panel's
-// rows of vbuf are Vp^T as it stands.  scratch >= 2 b m + 2 b^2 + part doubles.
+// rows of vbuf are Vp^T as it stands.  scratch >= 2 b nc + b (m + b) doubles.
 int backtransform_wy(const double* vbuf, const double* tau, int m, int nc, double* V,
                      double* scratch, long scratch_size, cudaStream_t s, OzWork* oz) {
   const int nref = m - 2;
   const int nb = kWyPanel;
+  const int npanel = (nref + nb - 1) / nb;
   double* W = scratch;
   double* W2 = W + (long)nb * nc;
-  double* Gp = W2 + (long)nb * nc;
-  double* T = Gp + (long)nb * nb;
-  double* part = T + (long)nb * nb;
-  const long partmax = scratch_size - (part - scratch);
-  if (partmax < (long)nb * nb) return CASPT2_EINVAL;
+  double* T = W2 + (long)nb * nc;                        // [panel][nb][nb]
+  if ((T - scratch) + (long)npanel * nb * nb > scratch_size) return CASPT2_EINVAL;
+  // every panel's T at once: Gram matrices (the last, shorter panel apart), then k_wy_T
+  const int full = nref / nb, last = nref - full * nb;
+  CASPT2_CUDA_TRY(dgemm(nb, nb, m, 1.0, vbuf, m, false, vbuf, m, true, 0.0, T, nb, s, full,
+                        (long)nb * m, (long)nb * m, (long)nb * nb));
+  if (last > 0) {
+    const double* vl = vbuf + (long)full * nb * m;
+    CASPT2_CUDA_TRY(dgemm(last, last, m, 1.0, vl, m, false, vl, m, true, 0.0,
+                          T + (long)full * nb * nb, nb, s));
+  }
+  constexpr size_t tsm = sizeof(double) * kWyPanel * (kWyPanel + 1);
+  CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_wy_T, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)tsm));
+  ++launch_counter();
+  k_wy_T<<<npanel, 256, tsm, s>>>(T, tau, nref);
+  CASPT2_CUDA_TRY(cudaGetLastError());
   for (int k0 = ((nref - 1) / nb) * nb; k0 >= 0; k0 -= nb) {
     const int b = std::min(nb, nref - k0);
     const int r = m - k0 - 1;                            // rows k0+1 .. m-1
     const double* Vt = vbuf + (long)k0 * m;              // b x m, zeros left of each v
-    int st = gram_product(Vt, Vt, 1, b, m, 0, Gp, b, 0, part, partmax, s, nullptr);
-    if (st != CASPT2_OK) return st;
-    ++launch_counter();
-    k_wy_T<<<1, b, 0, s>>>(Gp, tau, k0, b, T);
-    CASPT2_CUDA_TRY(cudaGetLastError());
+    const double* Tp = T + (long)(k0 / nb) * nb * nb;
     if (oz && oz->on) {
       // precision form: the two large products as FP64-accurate split products (the
       // eigenvalues are fixed before this step; only the vectors pass through it)
       const OzView va{Vt + k0 + 1, m, 1, r, 0};                  // rows l, K = row i
       const OzView vb{V + (long)(k0 + 1) * nc, 1, nc, r, 0};     // rows col, K = row i
       CASPT2_CUDA_TRY(oz_matmul(*oz, va, vb, false, b, nc, r, 1.0, 0.0, W, nc, s));
-      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, T, b, false, W, nc, false, 0.0, W2, nc, s));
+      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, Tp, nb, false, W, nc, false, 0.0, W2, nc, s));
       const OzView vp{Vt + k0 + 1, 1, m, b, 0};                  // rows i, K = l
       const OzView vw{W2, 1, nc, b, 0};                          // rows col, K = l
       CASPT2_CUDA_TRY(oz_matmul(*oz, vp, vw, false, r, nc, b, -1.0, 1.0, V + (long)(k0 + 1) * nc,
@@ -1187,7 +830,7 @@ int backtransform_wy(const double* vbuf, const double* tau, int m, int nc, doubl
     } else {
       CASPT2_CUDA_TRY(dgemm(b, nc, r, 1.0, Vt + k0 + 1, m, false, V + (long)(k0 + 1) * nc, nc,
                             false, 0.0, W, nc, s));
-      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, T, b, false, W, nc, false, 0.0, W2, nc, s));
+      CASPT2_CUDA_TRY(dgemm(b, nc, b, 1.0, Tp, nb, false, W, nc, false, 0.0, W2, nc, s));
       CASPT2_CUDA_TRY(dgemm(r, nc, b, -1.0, Vt + k0 + 1, m, true, W2, nc, false, 1.0,
                             V + (long)(k0 + 1) * nc, nc, s));
     }
@@ -1207,9 +850,7 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   double* u0 = G + mm;            // 5*m*m inverse-iteration scratch
   double* u1 = u0 + mm;
   double* u2 = u1 + mm;
-  double* lm = u2 + mm;
-  double* pv = lm + mm;
-  double* d = pv + mm;
+  double* d = u2 + 3 * mm;
   double* e = d + m;
   double* e2 = e + m;
   double* tau = e2 + m;
@@ -1223,7 +864,7 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   CASPT2_CUDA_TRY(cudaGetDevice(&dev));
   CASPT2_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   const int Gs = std::max(1, std::min(nsm, m));
-  const size_t smem_b = m > 64 ? tridiag_smem_bytes(m, Gs) : 0;
+  const size_t smem_b = tridiag_smem_bytes(m, Gs);
   if (smem_b > 0) {
     unsigned* sync = reinterpret_cast<unsigned*>(r);   // r is free until the back-transform
     double* pbuf = u0;                                 // u0.. are free until inverse iteration
@@ -1253,7 +894,7 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
       tm->bytes += 8.0 * m * m + 4.0 * m * (m - 1.0);
       ++tm->launches;
     }
-  } else if (m > 64 && m >= kLatrdMin) {
+  } else {
     // blocked reduction: panels of kLatrdPanel columns (one cooperative launch each) and
     // the trailing update as two FP64 GEMMs per panel
     unsigned* sync = reinterpret_cast<unsigned*>(r);   // r is free until the back-transform
@@ -1331,40 +972,6 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
       }
       ++tm->launches;
     }
-  } else if (m > 64) {
-    int per = 0;
-    CASPT2_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_tridiag, 512, 0));
-    const int grid = std::max(1, std::min(nsm * std::max(per, 1), nsm));
-    unsigned* sync = reinterpret_cast<unsigned*>(r);   // r is free until the back-transform
-    CASPT2_CUDA_TRY(cudaMemsetAsync(sync, 0, 4 * sizeof(unsigned), s));
-    void* args[] = {&A, (void*)&m, &vbuf, &tau, &d, &e, &p, &sync};
-    ++launch_counter();
-    if (tm && tm->e0) CASPT2_CUDA_TRY(cudaEventRecord(tm->e0, s));
-    CASPT2_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_tridiag, grid, 512, args, 0, s));
-    if (tm && tm->e1) CASPT2_CUDA_TRY(cudaEventRecord(tm->e1, s));
-    int herr = 0;
-    CASPT2_CUDA_TRY(cudaMemcpyAsync(&herr, sync + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
-    CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
-    if (herr != 0) return CASPT2_ETIMEOUT;
-    if (tm && tm->e0) {
-      float ms = 0.f;
-      CASPT2_CUDA_TRY(cudaEventElapsedTime(&ms, tm->e0, tm->e1));
-      tm->ms += ms;
-      tm->flops += 4.0 / 3.0 * (double)m * m * m;   // Householder tridiagonalisation
-      // the matrix read once and the reflectors (lower triangle) written once
-      tm->bytes += 8.0 * m * m + 4.0 * m * (m - 1.0);
-      ++tm->launches;
-    }
-  } else {
-    for (int k = 0; k + 2 < m; ++k) {
-      const int n1 = m - k - 1;
-      ++launch_counter();
-      k_house<<<1, 256, 0, s>>>(A, m, k, vbuf, tau, d, e);
-      ++launch_counter();
-      k_symv<<<std::max(1, std::min((n1 + 7) / 8, 152 * 8)), 256, 0, s>>>(A, m, k, vbuf, tau, p);
-      ++launch_counter();
-      k_rank2<<<nblocks((long)n1 * n1), kT, 0, s>>>(A, m, k, vbuf, tau, p);
-    }
   }
   if (smem_b == 0) {
     ++launch_counter();
@@ -1376,41 +983,40 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   CASPT2_CUDA_TRY(cudaMemcpyAsync(hd.data(), d, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
   CASPT2_CUDA_TRY(cudaMemcpyAsync(he.data(), e, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
   CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
-  double glo = 1e300, ghi = -1e300, emax2 = 0.0, tnorm = 0.0;
+  double glo = 1e300, ghi = -1e300, tnorm = 0.0;
   for (int i = 0; i < m; ++i) {
     const double r0 = (i > 0 ? fabs(he[i - 1]) : 0.0) + (i < m - 1 ? fabs(he[i]) : 0.0);
     glo = std::min(glo, hd[i] - r0);
     ghi = std::max(ghi, hd[i] + r0);
-    if (i < m - 1) emax2 = std::max(emax2, he[i] * he[i]);
     tnorm = std::max(tnorm, fabs(hd[i]) + r0);
     if (!(hd[i] == hd[i]) || !(he[i] == he[i])) return CASPT2_ENAN;
   }
   const double pad = 2.2e-16 * std::max(1.0, tnorm) * 4.0 + 1e-300;
   glo -= pad;
   ghi += pad;
-  const double pivmin = std::max(1e-300, 1e-290 * std::max(1.0, emax2));
   // 2. eigenvalues
   ++launch_counter();
   k_e2<<<(m + 255) / 256, 256, 0, s>>>(e, m, e2);
   ++launch_counter();
   if (3 * sizeof(double) * (size_t)m > kBisectSmemMax) return CASPT2_EINVAL;
-  CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_bisect, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_eigenvalues, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kBisectSmemMax));
   // blocks sized so that one wave covers all 8m lanes (the staged copy of the tridiagonal
   // matrix limits residency to one block per SM at the largest sizes)
-  const int bis_t = (int)std::min<long>(1024, std::max<long>(32, ((8L * m + nsm - 1) / nsm + 31) / 32 * 32));
-  k_bisect<<<(unsigned)((8L * m + bis_t - 1) / bis_t), bis_t, 3 * sizeof(double) * m, s>>>(
-      d, e, e2, m, glo, ghi, 4.0 * 2.2e-16 * std::max(1.0, tnorm), w);
+  const int ev_t = (int)std::min<long>(1024, std::max<long>(32, ((8L * m + nsm - 1) / nsm + 31) / 32 * 32));
+  k_eigenvalues<<<(unsigned)((8L * m + ev_t - 1) / ev_t), ev_t, 3 * sizeof(double) * m, s>>>(
+      d, e2, m, glo, ghi, kEigTol * std::max(1.0, tnorm), nkept ? eig_guard(wmin, tnorm) : -1e300, w);
   CASPT2_CUDA_TRY(cudaGetLastError());
-  // the vectors to form: all, or those of the eigenvalues at or above wmin (the last nc of
-  // the ascending list)
-  int j0 = 0;
+  // the vectors to return: all, or those of the eigenvalues at or above wmin (the last nk of
+  // the ascending list); nc >= nk are formed (eig_guard)
+  int j0 = 0, nk = m;
   if (nkept) {
     CASPT2_CUDA_TRY(cudaMemcpyAsync(hd.data(), w, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
     while (j0 < m && hd[j0] < wmin) ++j0;
-    *nkept = m - j0;
-    if (j0 == m) return CASPT2_OK;
+    *nkept = nk = m - j0;
+    if (nk == 0) return CASPT2_OK;
+    while (j0 > 0 && hd[j0 - 1] >= eig_guard(wmin, tnorm)) --j0;
   }
   const int nc = m - j0;
   const double* wk = w + j0;
@@ -1419,8 +1025,7 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   // one warp per block so that the m independent LU chains spread over the SMs
   CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_inviter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kBisectSmemMax));
-  k_inviter<<<(nc + 31) / 32, 32, 2 * sizeof(double) * m, s>>>(d, e, wk, m, nc, tnorm, u0, u1, u2,
-                                                                lm, pv, Z);
+  k_inviter<<<(nc + 31) / 32, 32, 2 * sizeof(double) * m, s>>>(d, e, wk, m, nc, tnorm, u0, Z);
   ++launch_counter();
   CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_cluster_cgs2, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kBisectSmemMax));
@@ -1446,8 +1051,13 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
   double dev_probe;
   std::memcpy(&dev_probe, &hdev, sizeof(double));
   if (!(dev_probe == dev_probe)) return CASPT2_ENAN;
+  // V = the last nk columns of Z
+  auto take_columns = [&]() {
+    return cudaMemcpy2DAsync(V, sizeof(double) * nk, Z + (nc - nk), sizeof(double) * nc,
+                             sizeof(double) * nk, m, cudaMemcpyDeviceToDevice, s);
+  };
   if (dev_probe <= 1e-13) {
-    CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
+    CASPT2_CUDA_TRY(take_columns());
   } else {
     CASPT2_CUDA_TRY(cudaMemsetAsync(ns_dev, 0, sizeof(unsigned long long), s));
     CASPT2_CUDA_TRY(dgemm_sym(nc, m, 1.0, Z, nc, true, Z, nc, false, 0.0, G, nc, s));
@@ -1460,7 +1070,7 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
     std::memcpy(&dev_ortho, &hdev, sizeof(double));
     if (!(dev_ortho == dev_ortho)) return CASPT2_ENAN;
     if (dev_ortho <= 1e-13) {
-      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
+      CASPT2_CUDA_TRY(take_columns());
     } else if (oz && oz->on) {
       // V = Z + Z Ec, Ec = (1/2)(I - Z^T Z) (G - I): the correction is of the size of the
       // orthogonality error, so a split product with S slices (error below about
@@ -1468,41 +1078,42 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
       ++launch_counter();
       k_sub_diag<<<(nc + 255) / 256, 256, 0, s>>>(G, nc, 1.0);
       CASPT2_CUDA_TRY(cudaGetLastError());
-      CASPT2_CUDA_TRY(cudaMemcpyAsync(V, Z, sizeof(double) * m * nc, cudaMemcpyDeviceToDevice, s));
+      CASPT2_CUDA_TRY(take_columns());
       const double lg = std::log2(std::max(1e-300, 0.5 * (double)m * dev_ortho));
       const int S = std::max(2, std::min(kOzMaxSlices, (int)std::ceil((57.0 + lg) / 7.0)));
       const int S0 = oz->S;
       oz->S = S;
-      const OzView vz{Z, nc, 1, nc, 0}, vg{G, nc, 1, nc, 0};   // G symmetric: B(j, k) = G[j][k]
-      const cudaError_t e = oz_matmul(*oz, vz, vg, false, m, nc, nc, 1.0, 1.0, V, nc, s);
+      // G symmetric: B(j, k) = G[nc - nk + j][k]
+      const OzView vz{Z, nc, 1, nc, 0}, vg{G + (long)(nc - nk) * nc, nc, 1, nc, 0};
+      const cudaError_t e = oz_matmul(*oz, vz, vg, false, m, nk, nc, 1.0, 1.0, V, nk, s);
       oz->S = S0;
       CASPT2_CUDA_TRY(e);
     } else {
-      CASPT2_CUDA_TRY(dgemm(m, nc, nc, 1.0, Z, nc, false, G, nc, false, 0.0, V, nc, s));
+      CASPT2_CUDA_TRY(dgemm(m, nk, nc, 1.0, Z, nc, false, G + (nc - nk), nc, false, 0.0, V, nk, s));
     }
   }
   // 5. back-transformation V = H_0 ... H_{m-3} Z: blocked (compact WY panels as FP64
   //    GEMMs) for large matrices, else column-owned in one launch.  Z, G and the
   //    inverse-iteration scratch are free here.
   if (m >= kWyMinSize) {
-    const int st = backtransform_wy(vbuf, tau, m, nc, V, Z, 7 * mm, s, oz);
+    const int st = backtransform_wy(vbuf, tau, m, nk, V, Z, 7 * mm, s, oz);
     if (st != CASPT2_OK) return st;
   } else if (m >= 3) {
     ++launch_counter();
     // columns resident in shared memory: ceil(m / SMs) per block (one block per SM, the
     // FP64 work spread evenly, one warp per column), fewer per block when they do not fit
     const long fit = (long)(kBackSmemMax / (8ull * m)) - 2;      // minus the v buffers
-    const int cbs = (int)std::min<long>(std::min<long>(16, (nc + nsm - 1) / nsm), fit);
+    const int cbs = (int)std::min<long>(std::min<long>(16, (nk + nsm - 1) / nsm), fit);
     if (cbs >= 1) {
       CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_backtransform_smem,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)kBackSmemMax));
-      k_backtransform_smem<<<(nc + cbs - 1) / cbs, 32 * cbs,
-                             sizeof(double) * (size_t)m * (cbs + 2), s>>>(vbuf, tau, m, nc, cbs,
+      k_backtransform_smem<<<(nk + cbs - 1) / cbs, 32 * cbs,
+                             sizeof(double) * (size_t)m * (cbs + 2), s>>>(vbuf, tau, m, nk, cbs,
                                                                           V);
     } else {
       const int cb = 8;     // 8 columns x 32 row groups per block
-      k_backtransform<<<(nc + cb - 1) / cb, 256, 0, s>>>(vbuf, tau, m, nc, cb, V);
+      k_backtransform<<<(nk + cb - 1) / cb, 256, 0, s>>>(vbuf, tau, m, nk, cb, V);
     }
   }
   CASPT2_CUDA_TRY(cudaGetLastError());

@@ -49,12 +49,6 @@ cudaError_t dgemm_sym(int N, int K, double alpha, const double* A, int lda, bool
                       const double* B, int ldb, bool tb, double beta, double* C, int ldc,
                       cudaStream_t s);
 
-// Eigenpairs of a symmetric m x m matrix by parallel cyclic Jacobi.  A is destroyed
-// (left holding the diagonalised matrix); w[m] eigenvalues (ascending), V[m][m] with
-// eigenvectors as columns; work >= 2*m*m + 2 doubles.  Returns CASPT2_OK, ENOTCONV,
-// ENAN or ECUDA.  Synchronises the stream once per sweep.
-int sym_eig_jacobi(double* A, int m, double* w, double* V, double* work, cudaStream_t s);
-
 // Eigenpairs of a symmetric m x m matrix by Householder tridiagonalisation, bisection,
 // inverse iteration and back-transformation (eig_tridiag.cu).  A is destroyed; w[m]
 // ascending; V[m][m] eigenvectors as columns.  work >= sym_eig_tridiag_work(m) doubles.
@@ -68,23 +62,27 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
                     KernelTimer* tm = nullptr, OzWork* oz = nullptr, double wmin = 0.0,
                     int* nkept = nullptr);
 
-// Dispatch: Jacobi for small matrices, tridiagonal method otherwise.
-inline int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
-                   KernelTimer* tm = nullptr, OzWork* oz = nullptr) {
-  return m <= 32 ? sym_eig_jacobi(A, m, w, V, work, s)
-                 : sym_eig_tridiag(A, m, w, V, work, s, tm, oz);
+// The same in one block in shared memory, m <= kSectorBlockMax (sector_block.cu): V is m x m,
+// or m x *nkept with nkept.  work >= sym_eig_work(m).  Synchronises the stream.
+int sym_eig_block(const double* A, int m, double* w, double* V, double* work, cudaStream_t s,
+                  double wmin = -1e300, int* nkept = nullptr);
+
+// Eigenpairs of A (destroyed): w[m] ascending, V[m][m] eigenvectors as columns.  One block for
+// up to kSectorBlockMax rows, where the whole solve is a chain of FP64 latencies and its
+// launches and host round trips would cost more (m = 96: 0.8 ms against 1.9 ms for the
+// stages as launches); the whole GPU above.
+int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
+            KernelTimer* tm = nullptr, OzWork* oz = nullptr);
+inline size_t sym_eig_work(int m) {
+  return std::max<size_t>((size_t)5 * m * m + 2 * m + 64, sym_eig_tridiag_work(m));
 }
-// Eigenvalues w[m] (all) and the eigenvectors of those >= wmin: *nkept vectors, V[i * ldv +
-// voff + c] component i of the c-th (ascending).  The vectors below the cut are not formed
-// where the tridiagonal method runs: an overlap matrix of rank r spends its inverse
+
+// Eigenvalues w[m] (all) and the eigenvectors of those >= wmin: V is m x *nkept (ascending).
+// The vectors below the cut are not formed: an overlap matrix of rank r spends its inverse
 // iteration, cluster orthogonalisation and back-transformation on r columns, and its null
 // space (one cluster of equal eigenvalues, serial in the Gram-Schmidt: 0.9 s of the 1.3 s of
 // a c42 a6 v350 n4 solve) costs nothing.
-int sym_eig_above(double* A, int m, double wmin, double* w, double* V, int* nkept, int* ldv,
-                  int* voff, double* work, cudaStream_t s, KernelTimer* tm = nullptr,
-                  OzWork* oz = nullptr);
-inline size_t sym_eig_work(int m) {
-  return std::max<size_t>((size_t)2 * m * m + 2, sym_eig_tridiag_work(m));
-}
+int sym_eig_above(double* A, int m, double wmin, double* w, double* V, int* nkept, double* work,
+                  cudaStream_t s, KernelTimer* tm = nullptr, OzWork* oz = nullptr);
 
 }  // namespace caspt2

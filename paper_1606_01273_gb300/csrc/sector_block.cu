@@ -20,6 +20,7 @@
 #include "class_ag.cuh"
 #include "class_dev.cuh"
 #include "eig_dev.cuh"
+#include "linalg.cuh"
 #include "sector_block.cuh"
 
 namespace caspt2 {
@@ -130,11 +131,12 @@ __device__ void tridiagonalise(double* A, int ld, int m, const Vecs& q) {
   __syncthreads();
 }
 
-// Eigenpairs of A (destroyed; stride ld) with eigenvalue >= wmin: q.w holds all m eigenvalues
-// ascending, Z [m][nc] the vectors of the last nc.  scr: 4 m nc doubles and m nc bytes.
-// Returns nc, or -1 when the matrix holds a NaN or an infinity.
+// Eigenpairs of A (destroyed; stride ld): q.w holds all m eigenvalues ascending, Z [m][nc] the
+// vectors of the last nc, of which the last nk have eigenvalues >= wmin (eig_guard).  scr: 4 m
+// nc doubles and m nc bytes.  Returns nk, or -1 when the matrix holds a NaN or an infinity.
 __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, double* scr,
-                         const Vecs& q, double* sh) {
+                         const Vecs& q, double* sh, int& nc) {
+  nc = 0;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   tridiagonalise(A, ld, m, q);
   // Gershgorin interval
@@ -180,18 +182,23 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     }
   }
   __syncthreads();
-  const double tol = 4.0 * 2.2e-16 * fmax(1.0, tn);
+  const double tol = kEigTol * fmax(1.0, tn);
   for (int j = threadIdx.x; j < m; j += kNT)
-    q.w[j] = eigenvalue_f64(q.d, q.e2, m, j, glo, ghi, q.lo[j], q.hi[j], tol, wmin);
+    q.w[j] = eigenvalue_f64(q.d, q.e2, m, j, glo, ghi, q.lo[j], q.hi[j], tol,
+                             eig_guard(wmin, tn));
   __syncthreads();
   if (threadIdx.x == 0) {
     int c = 0;
     while (c < m && q.w[c] < wmin) ++c;
     sh[4] = (double)(m - c);
+    if (c < m)
+      while (c > 0 && q.w[c - 1] >= eig_guard(wmin, tn)) --c;
+    sh[5] = (double)(m - c);
   }
   __syncthreads();
-  const int nc = (int)sh[4];
-  if (nc == 0) return 0;
+  const int nk = (int)sh[4];
+  nc = (int)sh[5];
+  if (nk == 0) return 0;
   const double* wk = q.w + (m - nc);
   for (int j = threadIdx.x; j < nc; j += kNT)
     inverse_iteration(q.d, q.e, m, wk[j], tn, nc, j, scr, Z);
@@ -285,7 +292,7 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     }
     __syncthreads();
   }
-  return nc;
+  return nk;
 }
 
 // C[i * N + j] = sum_k A[i * ai + k * ak] B[k * bk + j * bj], two outputs a thread in flight.
@@ -306,6 +313,18 @@ __device__ void block_mm(int M, int N, int K, const double* A, int ai, int ak, c
   }
 }
 
+// Shared memory of an m-row problem: A [m][m | 1], Z [m][m], the vectors.
+__device__ __forceinline__ Vecs layout(double* sm, int m, double*& Z) {
+  Z = sm + (long)m * (m | 1);
+  double* v = Z + (long)m * m;
+  Vecs q;
+  q.d = v; q.e = v + m; q.e2 = v + 2 * m; q.tau = v + 3 * m; q.w = v + 4 * m;
+  q.u = v + 5 * m; q.p = v + 6 * m; q.lo = v + 7 * m; q.hi = v + 8 * m;
+  q.df = reinterpret_cast<float*>(v + 9 * m);
+  q.ef = q.df + m;
+  return q;
+}
+
 __global__ void __launch_bounds__(kNT)
 k_sector_block(const SectorJob* __restrict__ jobs, int* __restrict__ info) {
   extern __shared__ double sm[];
@@ -313,15 +332,8 @@ k_sector_block(const SectorJob* __restrict__ jobs, int* __restrict__ info) {
   const SectorJob J = jobs[blockIdx.x];
   const int m = J.msec, ld = m | 1;
   double* A = sm;
-  double* Z = A + (long)m * ld;
-  Vecs q;
-  {
-    double* v = Z + (long)m * m;
-    q.d = v; q.e = v + m; q.e2 = v + 2 * m; q.tau = v + 3 * m; q.w = v + 4 * m;
-    q.u = v + 5 * m; q.p = v + 6 * m; q.lo = v + 7 * m; q.hi = v + 8 * m;
-    q.df = reinterpret_cast<float*>(v + 9 * m);
-    q.ef = q.df + m;
-  }
+  double* Z;
+  const Vecs q = layout(sm, m, Z);
   const long mf = J.m, mm = mf * mf;
   auto element = [&](const double* in, int i, int j) {   // sym(in_id + sgn in_sw), selected rows
     const long ri = J.Lsel < 0 ? i : (long)i * J.n + J.Lsel;
@@ -332,19 +344,19 @@ k_sector_block(const SectorJob* __restrict__ jobs, int* __restrict__ info) {
   };
   for (int t = threadIdx.x; t < m * m; t += kNT) A[(t / m) * ld + t % m] = element(J.S, t / m, t % m);
   __syncthreads();
-  const int nk = eig_block(A, ld, m, J.thresh, Z, J.scr, q, sh);
+  int nz;
+  const int nk = eig_block(A, ld, m, J.thresh, Z, J.scr, q, sh, nz);
   if (nk <= 0) {
     if (threadIdx.x == 0) { info[2 * blockIdx.x] = 0; info[2 * blockIdx.x + 1] = nk; }
     return;
   }
-  // X = Q s^(-1/2) in Z and, for the product with P, in J.X; F over A
+  // X = Q s^(-1/2) in J.X and back in Z; F over A
   for (int t = threadIdx.x; t < nk; t += kNT) q.u[t] = 1.0 / sqrt(q.w[m - nk + t]);
   __syncthreads();
-  for (int t = threadIdx.x; t < m * nk; t += kNT) {
-    const double x = Z[t] * q.u[t % nk];
-    Z[t] = x;
-    J.X[t] = x;
-  }
+  for (int t = threadIdx.x; t < m * nk; t += kNT)
+    J.X[t] = Z[(t / nk) * nz + nz - nk + t % nk] * q.u[t % nk];
+  __syncthreads();
+  for (int t = threadIdx.x; t < m * nk; t += kNT) Z[t] = J.X[t];
   for (int t = threadIdx.x; t < m * m; t += kNT) A[(t / m) * ld + t % m] = element(J.F, t / m, t % m);
   __syncthreads();
   block_mm(m, nk, m, A, ld, 1, Z, nk, 1, J.scr);                   // F X (through L2)
@@ -360,7 +372,7 @@ k_sector_block(const SectorJob* __restrict__ jobs, int* __restrict__ info) {
     A[i * ld2 + j] = 0.5 * (Ft[t] + Ft[j * nk + i]);
   }
   __syncthreads();
-  const int nf = eig_block(A, ld2, nk, -1e300, Z, J.scr, q, sh);
+  const int nf = eig_block(A, ld2, nk, -1e300, Z, J.scr, q, sh, nz);
   if (nf != nk) {
     if (threadIdx.x == 0) { info[2 * blockIdx.x] = 0; info[2 * blockIdx.x + 1] = -1; }
     return;
@@ -368,6 +380,30 @@ k_sector_block(const SectorJob* __restrict__ jobs, int* __restrict__ info) {
   for (int t = threadIdx.x; t < nk; t += kNT) J.omega[t] = q.w[t];
   block_mm(m, nk, nk, J.X, nk, 1, Z, nk, 1, J.Y);                  // Y = X P
   if (threadIdx.x == 0) { info[2 * blockIdx.x] = nk; info[2 * blockIdx.x + 1] = 0; }
+}
+
+// Eigenpairs of one matrix A [m][m]: w [m], V [m][nk] of the eigenvalues >= wmin; info = {nk,
+// -1 on NaN}.  scr: 5 m^2 doubles.
+__global__ void __launch_bounds__(kNT)
+k_eig_block(const double* __restrict__ Ag, int m, double wmin, double* __restrict__ w,
+            double* __restrict__ V, double* __restrict__ scr, int* __restrict__ info) {
+  extern __shared__ double sm[];
+  __shared__ double sh[8 + kNT];
+  const int ld = m | 1;
+  double* Z;
+  const Vecs q = layout(sm, m, Z);
+  for (int t = threadIdx.x; t < m * m; t += kNT)
+    sm[(t / m) * ld + t % m] = 0.5 * (Ag[t] + Ag[(t % m) * m + t / m]);
+  __syncthreads();
+  int nz;
+  const int nk = eig_block(sm, ld, m, wmin, Z, scr, q, sh, nz);
+  if (threadIdx.x == 0) {
+    info[0] = max(nk, 0);
+    info[1] = nk < 0 ? -1 : 0;
+  }
+  if (nk < 0) return;
+  for (int t = threadIdx.x; t < m; t += kNT) w[t] = q.w[t];
+  for (int t = threadIdx.x; t < m * nk; t += kNT) V[t] = Z[(t / nk) * nz + nz - nk + t % nk];
 }
 
 size_t sector_smem(int m) {
@@ -388,6 +424,25 @@ cudaError_t sector_block_launch(const SectorJob* jobs, int njobs, int mmax, int*
   ++launch_counter();
   k_sector_block<<<njobs, kNT, sector_smem(mmax), s>>>(jobs, info);
   return cudaGetLastError();
+}
+
+int sym_eig_block(const double* A, int m, double* w, double* V, double* work, cudaStream_t s,
+                  double wmin, int* nkept) {
+  if (nkept) *nkept = 0;
+  if (m <= 0) return CASPT2_OK;
+  if (m > kSectorBlockMax) return CASPT2_EINVAL;
+  CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_eig_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sector_smem(kSectorBlockMax)));
+  int* info = reinterpret_cast<int*>(work + (size_t)5 * m * m + 32);
+  ++launch_counter();
+  k_eig_block<<<1, kNT, sector_smem(m), s>>>(A, m, wmin, w, V, work, info);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  int h[2] = {0, 0};
+  CASPT2_CUDA_TRY(cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, s));
+  CASPT2_CUDA_TRY(cudaStreamSynchronize(s));
+  if (h[1] != 0) return CASPT2_ENAN;
+  if (nkept) *nkept = h[0];
+  return CASPT2_OK;
 }
 
 }  // namespace caspt2
