@@ -126,71 +126,85 @@ __global__ void k_swap_tuples(const double* __restrict__ src, DevClass C, ExtDim
 // Split-K Gram product over a tensor viewed as [pre][Ns][post]:
 //   part[z][x][y] = sum_{k in chunk z} A(x, k) B(y, k),  k = (p, q) over pre x post,
 //   A(x, (p, q)) = A[(p * Ns + x) * post + q].
-// Output tile TS x TS per block (TS <= 32 fitted to Ns), up to 4 outputs per thread,
-// K staged in chunks of 16 through shared memory; FP64 FMA.
-constexpr int kGS = 32, kGK = 16;
+// Output tile 32 x 32 per block: lanes over y, rows x dealt to the eight warps and skipped
+// beyond Ns (Ns is often 4 to 20: every FP64 instruction of a warp costs its sub-partition
+// 64 clocks, idle lanes or not), K staged in chunks of 32 through shared memory.
+constexpr int kGS = 32, kGK = 32;
 __global__ void __launch_bounds__(256)
 k_gram(const double* __restrict__ A, const double* __restrict__ B, long Ns, unsigned post,
-       unsigned K, unsigned chunk, int TS, double* __restrict__ part) {
+       unsigned K, unsigned chunk, double* __restrict__ part) {
   __shared__ double sa[kGK][kGS + 1], sb[kGK][kGS + 1];
-  const long x0 = (long)blockIdx.y * TS, y0 = (long)blockIdx.x * TS;
+  const long x0 = (long)blockIdx.y * kGS, y0 = (long)blockIdx.x * kGS;
   const unsigned kbeg = blockIdx.z * chunk;
   const unsigned kend = min(K, kbeg + chunk);
   const bool xfast = post == 1u;
-  const int nout = TS * TS;
-  int ox[4], oy[4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int q = threadIdx.x + 256 * r;
-    ox[r] = q < nout ? q / TS : 0;
-    oy[r] = q < nout ? q % TS : 0;
-  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int nx = (int)min((long)kGS, Ns - x0), ny = (int)min((long)kGS, Ns - y0);
+  const int nr = max(0, min(4, (nx - warp + 7) / 8));
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   for (unsigned k0 = kbeg; k0 < kend; k0 += kGK) {
-    for (int l = threadIdx.x; l < kGK * TS; l += 256) {
+#pragma unroll
+    for (int u = 0; u < kGK * kGS / 256; ++u) {
+      const int l = threadIdx.x + 256 * u;
       int kk, ii;
-      if (xfast) { ii = l % TS; kk = l / TS; } else { kk = l % kGK; ii = l / kGK; }
+      if (xfast) { ii = l % kGS; kk = l / kGS; } else { kk = l % kGK; ii = l / kGK; }
       const unsigned gk = k0 + kk;
-      const long gx = x0 + ii, gy = y0 + ii;
       double va = 0.0, vb = 0.0;
-      if (gk < kend) {
+      if (gk < kend && (ii < nx || ii < ny)) {
         const unsigned p = gk / post, q = gk - p * post;
         const long base = (long)p * Ns * post + q;
-        if (gx < Ns) va = A[base + gx * post];
-        if (gy < Ns) vb = B[base + gy * post];
+        if (ii < nx) va = A[base + (x0 + ii) * post];
+        if (ii < ny) vb = B[base + (y0 + ii) * post];
       }
       sa[kk][ii] = va;
       sb[kk][ii] = vb;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kGK; ++kk) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r] = fma(sa[kk][ox[r]], sb[kk][oy[r]], acc[r]);
-    }
+    for (int r = 0; r < 4; ++r)
+      if (r < nr) {
+#pragma unroll 8
+        for (int kk = 0; kk < kGK; ++kk) acc[r] = fma(sa[kk][warp + 8 * r], sb[kk][lane], acc[r]);
+      }
     __syncthreads();
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int q = threadIdx.x + 256 * r;
-    const long gx = x0 + ox[r], gy = y0 + oy[r];
-    if (q < nout && gx < Ns && gy < Ns) part[((long)blockIdx.z * Ns + gx) * Ns + gy] = acc[r];
-  }
+  for (int r = 0; r < 4; ++r)
+    if (r < nr && lane < ny)
+      part[((long)blockIdx.z * Ns + x0 + warp + 8 * r) * Ns + y0 + lane] = acc[r];
 }
 
-// Fixed-order sum of the split-K partials.  mode 0: out[x][y] = X; mode 1 (closed
-// block): out[off + y][off + x] -= X; mode 2 (virtual block): out[off + x][off + y] += X.
+// Fixed-order sum of the split-K partials (a warp per element, lanes striding the partials,
+// then a shuffle tree).  mode 0: out[x][y] = X; mode 1 (closed block): out[off + y][off + x] -=
+// X; mode 2 (virtual block): out[off + x][off + y] += X.
 __global__ void k_gram_finish(const double* __restrict__ part, int nsplit, long Ns, int mode,
                               double* __restrict__ out, long ld, long off) {
   const long total = Ns * Ns;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
-       e += (long)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const long nw = (long)gridDim.x * (blockDim.x >> 5);
+  for (long e = blockIdx.x * (long)(blockDim.x >> 5) + (threadIdx.x >> 5); e < total; e += nw) {
     double s = 0.0;
-    for (int z = 0; z < nsplit; ++z) s += part[(long)z * total + e];
+    for (int z = lane; z < nsplit; z += 32) s += part[(long)z * total + e];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane != 0) continue;
     const long x = e / Ns, y = e % Ns;
     if (mode == 0) out[x * ld + y] = s;
     else if (mode == 1) out[(off + y) * ld + off + x] -= s;
     else out[(off + x) * ld + off + y] += s;
+  }
+}
+
+// The same with one partial: a thread per element.
+__global__ void k_gram_place(const double* __restrict__ X, long Ns, int mode,
+                             double* __restrict__ out, long ld, long off) {
+  const long total = Ns * Ns;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
+       e += (long)gridDim.x * blockDim.x) {
+    const long x = e / Ns, y = e % Ns;
+    if (mode == 0) out[x * ld + y] = X[e];
+    else if (mode == 1) out[(off + y) * ld + off + x] -= X[e];
+    else out[(off + x) * ld + off + y] += X[e];
   }
 }
 
@@ -502,24 +516,28 @@ int gram_product(const double* A, const double* B, long pre, long Ns, long post,
     CASPT2_CUDA_TRY(oz_matmul(*oz, va, vb, A == B, (int)Ns, (int)Ns, (int)K, 1.0, 0.0, part, Ns,
                               s));
     ++launch_counter();
-    k_gram_finish<<<launch_blocks(Ns * Ns), 256, 0, s>>>(part, 1, Ns, mode, out, ld, off);
+    k_gram_place<<<launch_blocks(Ns * Ns), 256, 0, s>>>(part, Ns, mode, out, ld, off);
     CASPT2_CUDA_TRY(cudaGetLastError());
     return CASPT2_OK;
   }
   const long ntile = (Ns + kGS - 1) / kGS;
-  const int TS = (int)((Ns + ntile - 1) / ntile);        // tile edge fitted to Ns
   const long tiles = ntile * ntile;
+  // four blocks a SM, each with at least four chunks of K
   long nsplit = std::max<long>(1, (152L * 4 + tiles - 1) / tiles);
-  nsplit = std::min(nsplit, std::max<long>(1, K / 256));
+  nsplit = std::min(nsplit, std::max<long>(1, K / (4 * kGK)));
   nsplit = std::min(nsplit, partmax / (Ns * Ns));
   long chunk = (K + nsplit - 1) / nsplit;
   chunk = (chunk + kGK - 1) / kGK * kGK;
   nsplit = (K + chunk - 1) / chunk;
   dim3 grid((unsigned)ntile, (unsigned)ntile, (unsigned)nsplit);
   ++launch_counter();
-  k_gram<<<grid, 256, 0, s>>>(A, B, Ns, (unsigned)post, (unsigned)K, (unsigned)chunk, TS, part);
+  k_gram<<<grid, 256, 0, s>>>(A, B, Ns, (unsigned)post, (unsigned)K, (unsigned)chunk, part);
   ++launch_counter();
-  k_gram_finish<<<launch_blocks(Ns * Ns), 256, 0, s>>>(part, (int)nsplit, Ns, mode, out, ld, off);
+  if (nsplit == 1)
+    k_gram_place<<<launch_blocks(Ns * Ns), 256, 0, s>>>(part, Ns, mode, out, ld, off);
+  else
+    k_gram_finish<<<launch_blocks(Ns * Ns * 32), 256, 0, s>>>(part, (int)nsplit, Ns, mode, out, ld,
+                                                             off);
   CASPT2_CUDA_TRY(cudaGetLastError());
   return CASPT2_OK;
 }
