@@ -77,6 +77,7 @@ struct caspt2_ctx {
   HDensWork hd{};
   std::map<int, double*> gblk;        // adjoint (pq|rt) blocks, keys of eri_blk
   EriBlocks g_tab{};
+  PresumBlocks gp_tab{};              // adjoints of the pre-summed blocks
   double *dd1 = nullptr, *dd2 = nullptr, *dgdf = nullptr, *gtmp = nullptr;
   // precision form: split BF16 tensor-core GEMMs, class-H pair integrals kept for the densities
   OzWork oz{};
@@ -315,12 +316,13 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       {
         std::vector<SrcPlan> pre;
         presum_src_plans(V, pre, c->presum);
-        split_src_plans(k, pre, w.hVs, w.hG);
+        // groups with three shared loops while their G (a^6 n^2 doubles) stays below 1 GB
+        const double g3 = std::pow((double)a, 6) * n * n;
+        split_src_plans(k, pre, w.hVs, w.hG, g3 <= (double)(1L << 27) ? 3 : 2);
       }
       if (c->presum.size() > (size_t)kMaxPresum) st = CASPT2_EINVAL;
       ALLOC(w.dS, S.size());
       ALLOC(w.dF, F.size());
-      ALLOC(w.dV, V.size());
       ALLOC(w.dVs, w.hVs.size());
       {
         size_t nx = 0;
@@ -334,7 +336,7 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
         }
         if (nx > 0) ALLOC(w.dX, nx);
       }
-      if (st == CASPT2_OK && class_upload_plans(w, S, F, V) != cudaSuccess) st = CASPT2_ECUDA;
+      if (st == CASPT2_OK && class_upload_plans(w, S, F) != cudaSuccess) st = CASPT2_ECUDA;
       ALLOC(w.Sact, 2 * (size_t)w.m * w.m);
       ALLOC(w.Fact, 2 * (size_t)w.m * w.m);
       vmax = std::max(vmax, w.vsize);   // the sources live only during the class's solve
@@ -949,6 +951,11 @@ int alloc_densities(caspt2_ctx* c) {
       c->gblk[kv.first] = p;
       c->g_tab.p[kv.first] = p;
     }
+    for (size_t k = 0; k < c->presum.size() && st == CASPT2_OK; ++k) {
+      double* p = nullptr;
+      ALLOC(p, (size_t)std::max<long>(presum_size(d, c->presum[k]), 1));
+      c->gp_tab.p[k] = p;
+    }
   }
   if (h_on) {
     HDensWork& h = c->hd;
@@ -1086,13 +1093,21 @@ int caspt2_densities(caspt2_ctx* c, unsigned class_mask, void* stream) {
   if (any_ag) {
     for (auto& kv : c->gblk)
       CASPT2_CUDA_TRY(cudaMemsetAsync(kv.second, 0, sizeof(double) * block_size(d, kv.first), s));
+    for (size_t k = 0; k < c->presum.size(); ++k)
+      CASPT2_CUDA_TRY(cudaMemsetAsync(const_cast<double*>(c->gp_tab.p[k]), 0,
+                                      sizeof(double) * presum_size(d, c->presum[k]), s));
     RdmPtrs g{{nullptr, c->rdm1r, c->rdm2r, c->rdm3r, c->rdm4r}};
     for (int k = 0; k < 7; ++k) {
       if (!(class_mask >> k & 1u) || !c->cw_on[k]) continue;
-      const int st = class_densities(c->cw[k], c->dw, d, o.scheme, o.shift, g, c->E0, c->eps, c->R,
-                                     P, c->lamNL + (long)k * n, c->g_tab, c->dd1, c->dd2, &c->oz,
-                                     s);
+      const int st = class_densities(c->cw[k], c->dw, c->sw, d, o.scheme, o.shift, g, c->E0,
+                                     c->eps, c->R, P, c->lamNL + (long)k * n, c->g_tab,
+                                     c->gp_tab, c->dd1, c->dd2, &c->oz, s);
       if (st != CASPT2_OK) return st;
+    }
+    for (size_t k = 0; k < c->presum.size(); ++k) {
+      const PresumSpec& sp = c->presum[k];
+      const int key = ((sp.space[0] * 3 + sp.space[1]) * 3 + sp.space[2]) * 3 + sp.space[3];
+      CASPT2_CUDA_TRY(presum_adjoint(d, sp, c->gp_tab.p[k], c->gblk.at(key), s));
     }
     for (auto& kv : c->gblk) {
       const int sp4[4] = {kv.first / 27, (kv.first / 9) % 3, (kv.first / 3) % 3, kv.first % 3};

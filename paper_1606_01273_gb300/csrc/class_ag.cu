@@ -11,6 +11,7 @@
 // and the pieces of the effective Hamiltonian are
 //   e[L][L'] = sum_tuples V(L')^T T(L),  norm[L] = T(L)^T S T(L).
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "class_ag.cuh"
@@ -20,15 +21,51 @@
 namespace caspt2 {
 
 
+// Work split of the plan interpreters: 256 threads as 256 / TG elements times TG groups that
+// deal the plan terms (group g takes terms g, g + TG, ..); TG = 1 or 8.  With TG = 8 a group is
+// a warp and an element a lane; reduce() adds the groups' sums in order and is true for the
+// threads that hold the result.  Every thread of the block makes the same calls.
+template <int TG>
+struct TermGroup {
+  static constexpr int kElems = 256 / TG;
+  __device__ long first() const { return (long)blockIdx.x * kElems; }
+  __device__ long stride() const { return (long)gridDim.x * kElems; }
+  __device__ int lane() const { return threadIdx.x % kElems; }
+  __device__ int group() const { return threadIdx.x / kElems; }
+  template <int NV>
+  __device__ bool reduce(double* acc) const {
+    if (TG == 1) return true;
+    __shared__ double part[NV][256];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) part[v][threadIdx.x] = acc[v];
+    __syncthreads();
+    if (group() == 0) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int g = 1; g < TG; ++g) acc[v] += part[v][g * kElems + lane()];
+    }
+    __syncthreads();
+    return group() == 0;
+  }
+};
+// Elements up to which the terms are dealt to eight warps: about four resident blocks an SM.
+constexpr long kTermSplitMax = 152L * 4 * 256;
+
 // S or F_act for all (row, col) of the m x m class matrix; out[pi][row][col].
 // row = ((fam * a^nact + act) * n + M), act digits in slot order (first slot slowest).
-__global__ void k_act_eval(const ActPlan* __restrict__ plans, int nplan, DevClass C, int a, int n,
+// TG warps share 32 elements and deal the plan terms among themselves, their sums added in
+// warp order: a small class matrix leaves the chip empty and each thread is a chain of
+// dependent gathers over every term (class A at m = 128: 0.19 ms with one thread an element).
+template <int TG>
+__global__ void __launch_bounds__(256) k_act_eval(const ActPlan* __restrict__ plans, int nplan, DevClass C, int a, int n,
                            RdmPtrs g, const double* __restrict__ f_act, double* __restrict__ out,
                            int m) {
   const long total = (long)m * m;
   const long A = ipow(a, C.nact);
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
-       e += (long)gridDim.x * blockDim.x) {
+  const TermGroup<TG> tg;
+  for (long e0 = tg.first(); e0 < total; e0 += tg.stride()) {
+    const long e = min(e0 + tg.lane(), total - 1);
     const int row = e / m, col = e % m;
     int vals[24];
     const int M = row % n, N = col % n;
@@ -43,7 +80,7 @@ __global__ void k_act_eval(const ActPlan* __restrict__ plans, int nplan, DevClas
       ak /= a;
     }
     double acc0 = 0.0, acc1 = 0.0;
-    for (int t = 0; t < nplan; ++t) {
+    for (int t = tg.group(); t < nplan; t += TG) {
       const ActPlan& P = plans[t];
       if (P.fb != fb || P.fk != fk) continue;
       bool ok = true;
@@ -62,8 +99,11 @@ __global__ void k_act_eval(const ActPlan* __restrict__ plans, int nplan, DevClas
       }
       if (P.pi == 0) acc0 += P.coeff * s; else acc1 += P.coeff * s;
     }
-    out[e] = acc0;
-    out[total + e] = acc1;
+    double acc[2] = {acc0, acc1};
+    if (tg.template reduce<2>(acc) && e0 + tg.lane() < total) {
+      out[e] = acc[0];
+      out[total + e] = acc[1];
+    }
   }
 }
 
@@ -245,18 +285,20 @@ __global__ void k_src_g(SrcGSig g, DevClass C, Dims d, RdmPtrs rdm, double* __re
   }
 }
 
-// Same sources with one thread per (fam, ext, act) holding all n^2 (M, L) results (n <=
-// NS): each plan term's integral value and RDM offset are formed once and applied to the
+// Same sources with one thread per (fam, ext, act) and term group holding all n^2 (M, L)
+// results (n = NS): each plan term's integral value and RDM offset are formed once and applied to the
 // n^2 state pairs (Gamma[M][L][off] at stride a^(2 rank)).
-template <int NS>
-__global__ void k_src_eval_ml(const SrcPlan* __restrict__ plans, int nplan, DevClass C, Dims d,
+template <int NS, int TG>
+__global__ void __launch_bounds__(256) k_src_eval_ml(const SrcPlan* __restrict__ plans, int nplan, DevClass C, Dims d,
                               RdmPtrs g, const double* __restrict__ h, EriBlocks eri,
                               PresumBlocks pb, double* __restrict__ V, long total2) {
-  const int n = d.n, a = d.a, nmo = d.nmo();
+  constexpr int n = NS;
+  const int a = d.a, nmo = d.nmo();
   const int dimsp[4] = {d.c, d.a, d.v, 1};
   const int offsp[3] = {0, d.c, d.c + d.a};
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total2;
-       e += (long)gridDim.x * blockDim.x) {
+  const TermGroup<TG> tg;
+  for (long e0 = tg.first(); e0 < total2; e0 += tg.stride()) {
+    const long e = min(e0 + tg.lane(), total2 - 1);
     long r = e;
     int vals[24];
     vals[kRefZero] = 0;
@@ -273,7 +315,7 @@ __global__ void k_src_eval_ml(const SrcPlan* __restrict__ plans, int nplan, DevC
     double acc[NS * NS];
 #pragma unroll
     for (int q = 0; q < NS * NS; ++q) acc[q] = 0.0;
-    for (int t = 0; t < nplan; ++t) {
+    for (int t = tg.group(); t < nplan; t += TG) {
       const SrcPlan& P = plans[t];
       if (P.fb != fam) continue;
       bool ok = true;
@@ -313,7 +355,7 @@ __global__ void k_src_eval_ml(const SrcPlan* __restrict__ plans, int nplan, DevC
         if (P.rank == 0) {
 #pragma unroll
           for (int M = 0; M < NS; ++M)
-            if (M < n) acc[M * NS + M] += x;
+            acc[M * NS + M] += x;
         } else {
           long off = 0;
           for (int j = 0; j < 2 * P.rank; ++j) off = off * a + vals[P.idx[j]];
@@ -322,16 +364,15 @@ __global__ void k_src_eval_ml(const SrcPlan* __restrict__ plans, int nplan, DevC
           for (int M = 0; M < NS; ++M)
 #pragma unroll
             for (int L = 0; L < NS; ++L)
-              if (M < n && L < n) acc[M * NS + L] += x * gp[(long)(M * n + L) * stride];
+              acc[M * NS + L] += x * gp[(long)(M * n + L) * stride];
         }
       }
     }
-    double* out = V + e * n * n;
+    if (tg.template reduce<NS * NS>(acc) && e0 + tg.lane() < total2) {
+      double* out = V + e * n * n;
 #pragma unroll
-    for (int M = 0; M < NS; ++M)
-#pragma unroll
-      for (int L = 0; L < NS; ++L)
-        if (M < n && L < n) out[M * n + L] = acc[M * NS + L];
+      for (int q = 0; q < NS * NS; ++q) out[q] = acc[q];
+    }
   }
 }
 
@@ -1193,12 +1234,58 @@ cudaError_t presum_block(const Dims& d, const PresumSpec& sp, const double* src,
   return cudaGetLastError();
 }
 
+// Adjoint of k_presum: blk[x0][x1][x2][x3] += adj[..] where every summed position carries its
+// variable's value (a variable that fills two positions: their diagonal).
+__global__ void k_presum_adj(const double* __restrict__ adj, PresumSpec sp, int d0, int d1, int d2,
+                             int d3, double* __restrict__ blk) {
+  const int sd[4] = {d0, d1, d2, d3};
+  const long total = (long)d0 * d1 * d2 * d3;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
+       e += (long)gridDim.x * blockDim.x) {
+    int x[4], val[2] = {-1, -1};
+    long q = e;
+    for (int p = 3; p >= 0; --p) {
+      x[p] = (int)(q % sd[p]);
+      q /= sd[p];
+    }
+    bool ok = true;
+    long o = 0;
+    for (int p = 0; p < 4; ++p) {
+      const int v = sp.var[p];
+      if (v < 0) o = o * sd[p] + x[p];
+      else if (val[v] < 0) val[v] = x[p];
+      else if (val[v] != x[p]) ok = false;
+    }
+    if (ok) blk[e] += adj[o];
+  }
+}
+
+cudaError_t presum_adjoint(const Dims& d, const PresumSpec& sp, const double* adj, double* blk,
+                           cudaStream_t s) {
+  long total = 1;
+  for (int p = 0; p < 4; ++p) total *= space_dim(d, sp.space[p]);
+  if (total == 0) return cudaSuccess;
+  ++launch_counter();
+  k_presum_adj<<<launch_blocks(total), 256, 0, s>>>(adj, sp, space_dim(d, sp.space[0]),
+                                                    space_dim(d, sp.space[1]),
+                                                    space_dim(d, sp.space[2]),
+                                                    space_dim(d, sp.space[3]), blk);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_src_g(const SrcGSig& g, const DevClass& C, const Dims& d, const RdmPtrs& rdm,
+                         double* srcG, cudaStream_t s) {
+  const long total = ipow_host(d.a, g.ns) * ipow_host(d.a, C.nact) * d.n * d.n;
+  ++launch_counter();
+  k_src_g<<<launch_blocks(total), 256, 0, s>>>(g, C, d, rdm, srcG);
+  return cudaGetLastError();
+}
+
 cudaError_t class_upload_plans(ClassWork& w, const std::vector<ActPlan>& S,
-                               const std::vector<ActPlan>& F, const std::vector<SrcPlan>& V) {
+                               const std::vector<ActPlan>& F) {
   cudaError_t e;
   if ((e = cudaMemcpy(w.dS, S.data(), sizeof(ActPlan) * S.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
   if ((e = cudaMemcpy(w.dF, F.data(), sizeof(ActPlan) * F.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
-  if ((e = cudaMemcpy(w.dV, V.data(), sizeof(SrcPlan) * V.size(), cudaMemcpyHostToDevice)) != cudaSuccess) return e;
   if (w.dVs && (e = cudaMemcpy(w.dVs, w.hVs.data(), sizeof(SrcPlan) * w.hVs.size(),
                                cudaMemcpyHostToDevice)) != cudaSuccess)
     return e;
@@ -1216,7 +1303,6 @@ cudaError_t class_upload_plans(ClassWork& w, const std::vector<ActPlan>& S,
   }
   w.nS = (int)S.size();
   w.nF = (int)F.size();
-  w.nV = (int)V.size();
   return cudaSuccess;
 }
 
@@ -1226,9 +1312,15 @@ int class_matrices(ClassWork& w, const Dims& d, RdmPtrs rdm, const double* f_act
   if (w.vsize == 0 || m == 0) return CASPT2_OK;
   const long mm = (long)m * m;
   ++launch_counter();
-  k_act_eval<<<launch_blocks(mm), 256, 0, s>>>(w.dS, w.nS, w.dc, d.a, n, rdm, f_act, w.Sact, m);
+  // few terms in S: one thread an element is enough
+  k_act_eval<1><<<launch_blocks(mm), 256, 0, s>>>(w.dS, w.nS, w.dc, d.a, n, rdm, f_act, w.Sact, m);
   ++launch_counter();
-  k_act_eval<<<launch_blocks(mm), 256, 0, s>>>(w.dF, w.nF, w.dc, d.a, n, rdm, f_act, w.Fact, m);
+  if (mm <= kTermSplitMax)
+    k_act_eval<8><<<launch_blocks(mm, 32), 256, 0, s>>>(w.dF, w.nF, w.dc, d.a, n, rdm, f_act,
+                                                        w.Fact, m);
+  else
+    k_act_eval<1><<<launch_blocks(mm), 256, 0, s>>>(w.dF, w.nF, w.dc, d.a, n, rdm, f_act, w.Fact,
+                                                    m);
   CASPT2_CUDA_TRY(cudaGetLastError());
   return CASPT2_OK;
 }
@@ -1324,8 +1416,19 @@ int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double 
   ++launch_counter();
   if (n <= 4) {
     const long total2 = w.vsize / ((long)n * n);
-    k_src_eval_ml<4><<<launch_blocks(total2), 256, 0, s>>>(w.dVs, w.nVs, w.dc, d, rdm, h, eri, pb,
-                                                          w.V, total2);
+    auto run = [&](auto ns) {
+      constexpr int NS = decltype(ns)::value;
+      if (total2 <= kTermSplitMax && w.nVs > 1)
+        k_src_eval_ml<NS, 8><<<launch_blocks(total2, 32), 256, 0, s>>>(w.dVs, w.nVs, w.dc, d, rdm,
+                                                                       h, eri, pb, w.V, total2);
+      else
+        k_src_eval_ml<NS, 1><<<launch_blocks(total2), 256, 0, s>>>(w.dVs, w.nVs, w.dc, d, rdm, h,
+                                                                   eri, pb, w.V, total2);
+    };
+    if (n == 1) run(std::integral_constant<int, 1>());
+    else if (n == 2) run(std::integral_constant<int, 2>());
+    else if (n == 3) run(std::integral_constant<int, 3>());
+    else run(std::integral_constant<int, 4>());
   } else if (n <= 8) {
     const long total2 = w.vsize / ((long)n * n);
     k_src_eval_m<8><<<launch_blocks(total2 * n), 256, 0, s>>>(w.dVs, w.nVs, w.dc, d, rdm, h, eri,
@@ -1343,9 +1446,7 @@ int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double 
       const SrcGemmGroup& G = w.hG[gi];
       const long K = ipow_host(d.a, G.g.ns);
       if (K * ncol > sw.srcGcap) return CASPT2_EINVAL;
-      ++launch_counter();
-      k_src_g<<<launch_blocks(K * ncol), 256, 0, s>>>(G.g, w.dc, d, rdm, sw.srcG);
-      CASPT2_CUDA_TRY(cudaGetLastError());
+      CASPT2_CUDA_TRY(launch_src_g(G.g, w.dc, d, rdm, sw.srcG, s));
       const long chunk = std::min<long>(rows, sw.srcXcap / K);
       if (chunk < 1) return CASPT2_EINVAL;
       for (long r0 = 0; r0 < rows; r0 += chunk) {

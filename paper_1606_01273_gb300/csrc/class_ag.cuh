@@ -48,9 +48,8 @@ struct ClassWork {
   long vsize = 0;
   ActPlan* dS = nullptr; int nS = 0;
   ActPlan* dF = nullptr; int nF = 0;
-  SrcPlan* dV = nullptr; int nV = 0;
-  SrcPlan* dVs = nullptr; int nVs = 0;   // the solve's variant: loop-only integrals pre-summed,
-  std::vector<SrcPlan> hVs;              // without the terms that run as GEMM groups
+  SrcPlan* dVs = nullptr; int nVs = 0;   // source terms: loop-only integrals pre-summed, without
+  std::vector<SrcPlan> hVs;              // the terms that run as GEMM groups
   std::vector<SrcGemmGroup> hG;          // source terms as X G products (see terms.h)
   SrcXTerm* dX = nullptr;                // every group's X terms, group g at dX + gx_off[g]
   std::vector<int> gx_off;
@@ -108,9 +107,9 @@ void class_setup(int cls, const Dims& d, ClassWork& w);   // host-only: sizes an
 // Fill w.keep with the sectors of the scheme (device pointers left to the caller).
 void class_keep_layout(ClassWork& w, const Dims& d, int scheme);
 long class_sector_wsize(const ClassWork& w, const Dims& d, int scheme, long* partsize);
-// Upload plans (allocated by the caller with cudaMalloc into w.dS/dF/dV).
+// Upload plans (allocated by the caller with cudaMalloc into w.dS/dF/dVs).
 cudaError_t class_upload_plans(ClassWork& w, const std::vector<ActPlan>& S,
-                               const std::vector<ActPlan>& F, const std::vector<SrcPlan>& V);
+                               const std::vector<ActPlan>& F);
 
 // The small sectors of all classes, solved in one launch (sector_block.cuh): jobs in class
 // order, class k's at [first[k], first[k + 1]).
@@ -149,6 +148,13 @@ int class_solve(ClassWork& w, SectorWork& sw, const Dims& d, int scheme, double 
 long presum_size(const Dims& d, const PresumSpec& sp);
 cudaError_t presum_block(const Dims& d, const PresumSpec& sp, const double* src, double* out,
                          cudaStream_t s);
+// blk += the adjoint of presum_block: every element of the block receives the adjoint of the
+// pre-summed element it was added to (elements off a repeated summed index receive none).
+cudaError_t presum_adjoint(const Dims& d, const PresumSpec& sp, const double* adj, double* blk,
+                           cudaStream_t s);
+// G of a source GEMM group (terms.h) into srcG.
+cudaError_t launch_src_g(const SrcGSig& g, const DevClass& C, const Dims& d, const RdmPtrs& rdm,
+                         double* srcG, cudaStream_t s);
 // e = -M1[L][L][.], norm = M2[L][L] of one class
 cudaError_t launch_moments_to_e(const double* mom, int n, double* e, double* nr, cudaStream_t s);
 // lambda pieces of the target state P of one class from its moments and R
@@ -168,10 +174,11 @@ int class_tuple_amplitudes(ClassWork& w, DensWork& dw, const Dims& d, double shi
 // out[fam][ext...][act...] = src[tuple][L][(fam, act..., N)] for one (L, N).
 cudaError_t gather_amplitudes(const ClassWork& w, const Dims& d, const double* src, int L, int N,
                               double* out, cudaStream_t s);
-int class_densities(ClassWork& w, DensWork& dw, const Dims& d, int scheme, double shift,
-                    RdmPtrs rdm, const double* E0, const double* eps_cv, const double* R, int P,
-                    const double* NL, const EriBlocks& G, double* d1, double* d2, OzWork* oz,
-                    cudaStream_t s);
+// GP: adjoints of the pre-summed blocks; sw: the source groups' X and G work arrays.
+int class_densities(ClassWork& w, DensWork& dw, SectorWork& sw, const Dims& d, int scheme,
+                    double shift, RdmPtrs rdm, const double* E0, const double* eps_cv,
+                    const double* R, int P, const double* NL, const EriBlocks& G,
+                    const PresumBlocks& GP, double* d1, double* d2, OzWork* oz, cudaStream_t s);
 
 // GDF[Q][p][q] += sum_rt G[pq][rt] B[Q][rt] and GDF[Q][r][t] += sum_pq G[pq][rt] B[Q][pq]
 // for one adjoint block with spaces sp; pack0/pack1/tmp hold X * (block pair) doubles.

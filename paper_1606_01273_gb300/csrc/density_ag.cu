@@ -14,6 +14,7 @@
 // All contractions reuse the access plans of the solve (transposed), so the device
 // path shares the solve's normal ordering and index conventions.
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "class_ag.cuh"
@@ -212,16 +213,20 @@ __global__ void k_gram_place(const double* __restrict__ X, long Ns, int mode,
 // Each thread takes its own (row, col) elements, evaluates every plan term once (as the
 // forward evaluation does) and adds coeff * D * Gamma into its private column of
 // acc[uw][thread] in shared memory at uw = (f index 0, f index 1); a fixed-order sum over
-// the threads gives part[block][a^2].
+// the threads gives part[block][a^2].  split: the warps of a block share 32 elements and deal
+// the plan terms (small class matrices).
 __global__ void k_act_adj(const ActPlan* __restrict__ plans, int nplan, DevClass C, int a, int n,
-                          RdmPtrs g, const double* __restrict__ Dm, int m,
+                          RdmPtrs g, const double* __restrict__ Dm, int m, int split,
                           double* __restrict__ part) {
   extern __shared__ double acc[];   // [a^2][blockDim.x]
   const int a2 = a * a, nt = blockDim.x, tid = threadIdx.x;
   for (int q = 0; q < a2; ++q) acc[q * nt + tid] = 0.0;
   const long total = (long)m * m;
   const long A = ipow(a, C.nact);
-  for (long e = (long)blockIdx.x * nt + tid; e < total; e += (long)gridDim.x * nt) {
+  const int per = split ? 32 : nt;                 // elements of a block at a time
+  const int t0 = split ? tid >> 5 : 0, ts = split ? nt >> 5 : 1;
+  for (long e = (long)blockIdx.x * per + (split ? tid & 31 : tid); e < total;
+       e += (long)gridDim.x * per) {
     const double D0 = Dm[e], D1 = Dm[total + e];
     if (D0 == 0.0 && D1 == 0.0) continue;
     const int row = e / m, col = e % m;
@@ -237,7 +242,7 @@ __global__ void k_act_adj(const ActPlan* __restrict__ plans, int nplan, DevClass
       vals[kRefKet + k] = ak % a;
       ak /= a;
     }
-    for (int t = 0; t < nplan; ++t) {
+    for (int t = t0; t < nplan; t += ts) {
       const ActPlan& P = plans[t];
       if (!P.has_f || P.fb != fb || P.fk != fk) continue;
       const double Dv = P.pi == 0 ? D0 : D1;
@@ -259,10 +264,12 @@ __global__ void k_act_adj(const ActPlan* __restrict__ plans, int nplan, DevClass
     }
   }
   __syncthreads();
-  for (int q = tid; q < a2; q += nt) {
+  for (int q = tid >> 5; q < a2; q += nt >> 5) {
     double t = 0.0;
-    for (int j = 0; j < nt; ++j) t += acc[q * nt + j];
-    part[(long)blockIdx.x * a2 + q] = t;
+    for (int j = tid & 31; j < nt; j += 32) t += acc[q * nt + j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((tid & 31) == 0) part[(long)blockIdx.x * a2 + q] = t;
   }
 }
 
@@ -271,26 +278,30 @@ __global__ void k_act_finish(const double* __restrict__ part, int nblk, int a, i
                              const double* __restrict__ NL, const double* __restrict__ g1, int n,
                              double* __restrict__ d2) {
   const int a2 = a * a;
-  for (int uw = threadIdx.x; uw < a2; uw += blockDim.x) {
+  for (int uw = threadIdx.x >> 5; uw < a2; uw += blockDim.x >> 5) {
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(long)b * a2 + uw];
+    for (int b = threadIdx.x & 31; b < nblk; b += 32) s += part[(long)b * a2 + uw];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) != 0) continue;
     for (int L = 0; L < n; ++L) s -= NL[L] * g1[((long)L * n + L) * a2 + uw];
     d2[(long)(c + uw / a) * nmo + c + uw % a] += s;
   }
 }
 
-// W[t][L'][row] = r_L' sum_L r_L T[t][L][row] + Lam[t][L'][row]
+// Source multipliers W = r_L' sum_L r_L T_L + Lam_L' in the layout of the sources V,
+// W[fam][t][act][M][L'], from T, Lam [t][L][(fam, act, M)].
 __global__ void k_wsrc(const double* __restrict__ T, const double* __restrict__ Lam,
-                       const double* __restrict__ R, int P, int n, long m, long total,
+                       const double* __restrict__ R, int P, int n, long m, long ntot, int nfam,
                        double* __restrict__ W) {
+  const long total = ntot * m, per = m / nfam;    // per = A n rows of a family
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
-    const long row = e % m;
-    const int Lp = (e / m) % n;
-    const long t = e / (m * n);
+    const long row = e % m, t = e / m;
     double acc = 0.0;
     for (int L = 0; L < n; ++L) acc += R[L * n + P] * T[(t * n + L) * m + row];
-    W[e] = R[Lp * n + P] * acc + Lam[e];
+    double* w = W + (((row / per) * ntot + t) * per + row % per) * n;
+    for (int Lp = 0; Lp < n; ++Lp) w[Lp] = R[Lp * n + P] * acc + Lam[(t * n + Lp) * m + row];
   }
 }
 
@@ -298,135 +309,67 @@ __device__ __forceinline__ void flush_add(double* p, double v) {
   if (p != nullptr && v != 0.0) atomicAdd(p, v);
 }
 
-// Adjoint of the sources: for every V element (fam, ext, act, M, L') with multiplier
-// W, each plan term coeff * I[...] * Gamma adds coeff * W * Gamma to dI[...] (d1 for the
-// one-electron part, G blocks for (pq|rt)).  Runs of equal targets are summed before
-// the atomic add.
-__global__ void k_src_adj(const SrcPlan* __restrict__ plans, int nplan, DevClass C, Dims d,
-                          RdmPtrs g, const double* __restrict__ W, long m, long vtotal,
-                          double* __restrict__ d1, EriBlocks G) {
-  const int n = d.n, a = d.a, nmo = d.nmo();
-  const int dimsp[3] = {d.c, d.a, d.v};
+// Target of an integral of a source term: element of d1 (kind 0), of the adjoint (pq|rt) block
+// (kind 1) or of the adjoint of a pre-summed block (kind 2).
+struct AdjTarget {
+  double* base;
+  long s0, s1, s2;             // strides of the first three indices (the last is contiguous)
+  int o0, o1;                  // offsets of the first two (kind 0)
+};
+__device__ __forceinline__ AdjTarget adj_target(int kind, int cb, const int8_t* sp, const Dims& d,
+                                                double* d1, const EriBlocks& G,
+                                                const PresumBlocks& GP) {
+  const int dimsp[4] = {d.c, d.a, d.v, 1};
   const int offsp[3] = {0, d.c, d.c + d.a};
-  const long A = ipow(a, C.nact);
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < vtotal;
-       e += (long)gridDim.x * blockDim.x) {
-    long r = e;
-    const int L = r % n; r /= n;
-    const int M = r % n; r /= n;
-    const long actlin = r % A; r /= A;
-    int vals[24];
-    long q = actlin;
-    for (int k = C.nact - 1; k >= 0; --k) {
-      vals[kRefBra + C.act[k]] = q % a;
-      q /= a;
-    }
-    int co[3];
-    for (int k = C.next - 1; k >= 0; --k) {
-      const int dm = dimsp[C.slot_space[C.ext[k]]];
-      co[k] = r % dm;
-      vals[kRefBra + C.ext[k]] = co[k];
-      r /= dm;
-    }
-    const int fam = (int)r;
-    long t = 0;
-    for (int k = 0; k < C.next; ++k) t = t * dimsp[C.slot_space[C.ext[k]]] + co[k];
-    const double Wv = W[(t * n + L) * m + (fam * A + actlin) * n + M];
-    if (Wv == 0.0) continue;
-    double* last = nullptr;
-    double run = 0.0;
-    for (int tp = 0; tp < nplan; ++tp) {
-      const SrcPlan& P = plans[tp];
-      if (P.fb != fam) continue;
-      bool ok = true;
-      for (int qq = 0; qq < P.neq; ++qq)
-        if (vals[P.eq[qq][0]] != vals[P.eq[qq][1]]) ok = false;
-      if (!ok) continue;
-      long niter = 1;
-      for (int j = 0; j < P.nloop; ++j) niter *= dimsp[P.loop_space[j]];
-      double* blk = nullptr;
-      long bd[4] = {1, 1, 1, 1};
-      if (P.kind == 1) {
-        const int key = ((P.ispace[0] * 3 + P.ispace[1]) * 3 + P.ispace[2]) * 3 + P.ispace[3];
-        blk = const_cast<double*>(G.p[key]);
-        for (int j = 0; j < 4; ++j) bd[j] = dimsp[P.ispace[j]];
-      }
-      const double cw = P.coeff * Wv;
-      for (long it = 0; it < niter; ++it) {
-        long qi = it;
-        for (int j = 0; j < P.nloop; ++j) {
-          const int dm = dimsp[P.loop_space[j]];
-          vals[kRefLoop + j] = qi % dm;
-          qi /= dm;
-        }
-        const double x = rdm_at(g.p, P.rank, n, a, M, L, vals, P.idx);
-        if (x == 0.0) continue;
-        double* tgt;
-        if (P.kind == 0) {
-          tgt = d1 + (long)(offsp[P.ispace[0]] + vals[P.iidx[0]]) * nmo + offsp[P.ispace[1]] +
-                vals[P.iidx[1]];
-        } else {
-          tgt = blk + ((vals[P.iidx[0]] * bd[1] + vals[P.iidx[1]]) * bd[2] + vals[P.iidx[2]]) *
-                          bd[3] + vals[P.iidx[3]];
-        }
-        if (tgt != last) {
-          flush_add(last, run);
-          last = tgt;
-          run = 0.0;
-        }
-        run += cw * x;
-      }
-    }
-    flush_add(last, run);
-  }
+  if (kind == 0) return {d1, 0, 0, d.nmo(), offsp[sp[0]], offsp[sp[1]]};
+  const long s2 = dimsp[sp[3]], s1 = s2 * dimsp[sp[2]], s0 = s1 * dimsp[sp[1]];
+  double* b = const_cast<double*>(
+      kind == 1 ? G.p[((sp[0] * 3 + sp[1]) * 3 + sp[2]) * 3 + sp[3]] : GP.p[cb]);
+  return {b, s0, s1, s2, 0, 0};
+}
+__device__ __forceinline__ double* adj_element(const AdjTarget& t, int kind, const int* vals,
+                                               const int8_t* idx) {
+  if (kind == 0) return t.base + (t.o0 + vals[idx[0]]) * t.s2 + t.o1 + vals[idx[1]];
+  return t.base + vals[idx[0]] * t.s0 + vals[idx[1]] * t.s1 + vals[idx[2]] * t.s2 + vals[idx[3]];
 }
 
-// Source adjoint with one thread per (fam, ext, act) and the n^2 multipliers W[M][L'] (n <=
-// NS) in registers: each plan term adds coeff * sum_(M,L') W Gamma[M][L'][off] to its
-// target with one atomic per run of equal targets.
-template <int NS>
-__global__ void k_src_adj_ml(const SrcPlan* __restrict__ plans, int nplan, DevClass C, Dims d,
-                             RdmPtrs g, const double* __restrict__ W, long m, long total2,
-                             double* __restrict__ d1, EriBlocks G) {
-  const int n = d.n, a = d.a, nmo = d.nmo();
-  const int dimsp[3] = {d.c, d.a, d.v};
-  const int offsp[3] = {0, d.c, d.c + d.a};
-  const long A = ipow(a, C.nact);
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total2;
-       e += (long)gridDim.x * blockDim.x) {
+// Adjoint of the sources that the plan interpreter forms: for every (fam, ext, act) and the
+// n^2 multipliers W[M][L'], each plan term adds coeff * sum_(M,L') W Gamma[M][L'][off] to its
+// integral's target, with one atomic add per run of equal targets.  NS = n holds the
+// multipliers in registers; NS = 0 reads them (any n).  TG warps share 32 elements and deal
+// the plan terms (TG = 1: one thread an element).
+template <int NS, int TG>
+__global__ void __launch_bounds__(256)
+k_src_adj(const SrcPlan* __restrict__ plans, int nplan, DevClass C, Dims d, RdmPtrs g,
+          const double* __restrict__ W, long total2, double* __restrict__ d1, EriBlocks G,
+          PresumBlocks GP) {
+  const int n = NS > 0 ? NS : d.n, a = d.a;
+  const int dimsp[4] = {d.c, d.a, d.v, 1};
+  constexpr int per = 256 / TG;
+  for (long e = (long)blockIdx.x * per + threadIdx.x % per; e < total2;
+       e += (long)gridDim.x * per) {
     long r = e;
-    const long actlin = r % A;
-    r /= A;
     int vals[24];
-    long q = actlin;
+    vals[kRefZero] = 0;
     for (int k = C.nact - 1; k >= 0; --k) {
-      vals[kRefBra + C.act[k]] = q % a;
-      q /= a;
+      vals[kRefBra + C.act[k]] = r % a;
+      r /= a;
     }
-    int co[3];
     for (int k = C.next - 1; k >= 0; --k) {
       const int dm = dimsp[C.slot_space[C.ext[k]]];
-      co[k] = r % dm;
-      vals[kRefBra + C.ext[k]] = co[k];
+      vals[kRefBra + C.ext[k]] = r % dm;
       r /= dm;
     }
     const int fam = (int)r;
-    long t = 0;
-    for (int k = 0; k < C.next; ++k) t = t * dimsp[C.slot_space[C.ext[k]]] + co[k];
-    double wv[NS * NS];
-    bool any = false;
+    const double* wp = W + e * n * n;
+    double wv[NS > 0 ? NS * NS : 1];
+    if (NS > 0) {
 #pragma unroll
-    for (int M = 0; M < NS; ++M)
-#pragma unroll
-      for (int L = 0; L < NS; ++L) {
-        const double x = (M < n && L < n) ? W[(t * n + L) * m + (fam * A + actlin) * n + M] : 0.0;
-        wv[M * NS + L] = x;
-        any = any || x != 0.0;
-      }
-    if (!any) continue;
+      for (int q = 0; q < NS * NS; ++q) wv[q] = wp[q];
+    }
     double* last = nullptr;
     double run = 0.0;
-    for (int tp = 0; tp < nplan; ++tp) {
+    for (int tp = threadIdx.x / per; tp < nplan; tp += TG) {
       const SrcPlan& P = plans[tp];
       if (P.fb != fam) continue;
       bool ok = true;
@@ -435,13 +378,7 @@ __global__ void k_src_adj_ml(const SrcPlan* __restrict__ plans, int nplan, DevCl
       if (!ok) continue;
       long niter = 1;
       for (int j = 0; j < P.nloop; ++j) niter *= dimsp[P.loop_space[j]];
-      double* blk = nullptr;
-      long bd[4] = {1, 1, 1, 1};
-      if (P.kind == 1) {
-        const int key = ((P.ispace[0] * 3 + P.ispace[1]) * 3 + P.ispace[2]) * 3 + P.ispace[3];
-        blk = const_cast<double*>(G.p[key]);
-        for (int j = 0; j < 4; ++j) bd[j] = dimsp[P.ispace[j]];
-      }
+      const AdjTarget at = adj_target(P.kind, P.cb, P.ispace, d, d1, G, GP);
       const long stride = ipow(a, 2 * P.rank);
       for (long it = 0; it < niter; ++it) {
         long qi = it;
@@ -452,27 +389,20 @@ __global__ void k_src_adj_ml(const SrcPlan* __restrict__ plans, int nplan, DevCl
         }
         double gs = 0.0;
         if (P.rank == 0) {
-#pragma unroll
-          for (int M = 0; M < NS; ++M) gs += wv[M * NS + M];
+          for (int M = 0; M < n; ++M) gs += NS > 0 ? wv[M * n + M] : wp[M * n + M];
         } else {
           long off = 0;
           for (int j = 0; j < 2 * P.rank; ++j) off = off * a + vals[P.idx[j]];
           const double* gp = g.p[P.rank] + off;
+          if (NS > 0) {
 #pragma unroll
-          for (int M = 0; M < NS; ++M)
-#pragma unroll
-            for (int L = 0; L < NS; ++L)
-              if (M < n && L < n) gs += wv[M * NS + L] * gp[(long)(M * n + L) * stride];
+            for (int q = 0; q < NS * NS; ++q) gs = fma(wv[q], gp[q * stride], gs);
+          } else {
+            for (int q = 0; q < n * n; ++q) gs = fma(wp[q], gp[q * stride], gs);
+          }
         }
         if (gs == 0.0) continue;
-        double* tgt;
-        if (P.kind == 0) {
-          tgt = d1 + (long)(offsp[P.ispace[0]] + vals[P.iidx[0]]) * nmo + offsp[P.ispace[1]] +
-                vals[P.iidx[1]];
-        } else {
-          tgt = blk + ((vals[P.iidx[0]] * bd[1] + vals[P.iidx[1]]) * bd[2] + vals[P.iidx[2]]) *
-                          bd[3] + vals[P.iidx[3]];
-        }
+        double* tgt = adj_element(at, P.kind, vals, P.iidx);
         if (tgt != last) {
           flush_add(last, run);
           last = tgt;
@@ -482,6 +412,54 @@ __global__ void k_src_adj_ml(const SrcPlan* __restrict__ plans, int nplan, DevCl
       }
     }
     flush_add(last, run);
+  }
+}
+
+// Adjoint of k_src_x: the adjoint XA[row][k] of a source group's X, over the external tuples
+// row0 .. row0 + nrow, times each integral term's coefficient, added to the term's target.
+__global__ void k_src_x_adj(const SrcXTerm* __restrict__ xt, int nx, DevClass C, Dims d, int ns,
+                            const double* __restrict__ XA, long row0, long nrow,
+                            double* __restrict__ d1, EriBlocks G, PresumBlocks GP) {
+  const int a = d.a;
+  const int dimsp[4] = {d.c, d.a, d.v, 1};
+  const long K = ipow(a, ns);
+  const long total = nrow * K;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
+       e += (long)gridDim.x * blockDim.x) {
+    const double xa = XA[e];
+    if (xa == 0.0) continue;
+    int vals[32];
+    vals[kRefZero] = 0;
+    long q = e % K;
+    for (int p = ns - 1; p >= 0; --p) {
+      vals[kRefLoop + p] = (int)(q % a);
+      q /= a;
+    }
+    long r = row0 + e / K;
+    for (int k = C.next - 1; k >= 0; --k) {
+      const int dm = dimsp[C.slot_space[C.ext[k]]];
+      vals[kRefBra + C.ext[k]] = (int)(r % dm);
+      r /= dm;
+    }
+    for (int t = 0; t < nx; ++t) {
+      const SrcXTerm& T = xt[t];
+      bool ok = true;
+      for (int u = 0; u < T.neq; ++u)
+        if (vals[T.eq[u][0]] != vals[T.eq[u][1]]) ok = false;
+      if (!ok) continue;
+      const AdjTarget at = adj_target(T.kind, T.cb, T.ispace, d, d1, G, GP);
+      long niter = 1;
+      for (int j = 0; j < T.nloop; ++j) niter *= dimsp[T.loop_space[j]];
+      for (long it = 0; it < niter; ++it) {
+        long w = it;
+        for (int j = 0; j < T.nloop; ++j) {
+          const int dm = dimsp[T.loop_space[j]];
+          vals[kRefLoop + ns + j] = (int)(w % dm);
+          w /= dm;
+        }
+        atomicAdd(adj_element(at, T.kind, vals, T.iidx), T.coeff * xa);
+      }
+    }
   }
 }
 
@@ -600,10 +578,10 @@ int class_tuple_amplitudes(ClassWork& w, DensWork& dw, const Dims& d, double shi
   return CASPT2_OK;
 }
 
-int class_densities(ClassWork& w, DensWork& dw, const Dims& d, int scheme, double shift,
-                    RdmPtrs rdm, const double* E0, const double* eps_cv, const double* R, int P,
-                    const double* NL, const EriBlocks& G, double* d1, double* d2, OzWork* oz,
-                    cudaStream_t s) {
+int class_densities(ClassWork& w, DensWork& dw, SectorWork& sw, const Dims& d, int scheme,
+                    double shift, RdmPtrs rdm, const double* E0, const double* eps_cv,
+                    const double* R, int P, const double* NL, const EriBlocks& G,
+                    const PresumBlocks& GP, double* d1, double* d2, OzWork* oz, cudaStream_t s) {
   (void)scheme;
   const int m = w.m, n = d.n, a = d.a, nmo = d.nmo();
   if (w.vsize == 0 || m == 0) return CASPT2_OK;
@@ -673,29 +651,66 @@ int class_densities(ClassWork& w, DensWork& dw, const Dims& d, int scheme, doubl
     const int nt = std::max(32, std::min(256, (int)(kActAdjSmem / (8L * a2)) / 32 * 32));
     const size_t smem = 8ull * a2 * nt;
     if (smem > (size_t)kActAdjSmem) return CASPT2_EINVAL;
-    const long nblk = std::max<long>(1, std::min<long>(152L * 4, (mm + nt - 1) / nt));
+    // terms dealt to the warps while a thread an element leaves the chip empty
+    const int split = mm <= 152L * 4 * nt;
+    const long nblk = std::max<long>(1, std::min<long>(152L * 4, split ? (mm + 31) / 32
+                                                                       : (mm + nt - 1) / nt));
     if (nblk * a2 > dw.partmax) return CASPT2_EINVAL;
     CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_act_adj, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kActAdjSmem));
     ++launch_counter();
-    k_act_adj<<<(unsigned)nblk, nt, smem, s>>>(w.dF, w.nF, C, a, n, rdm, dw.Dm, m, dw.part);
+    k_act_adj<<<(unsigned)nblk, nt, smem, s>>>(w.dF, w.nF, C, a, n, rdm, dw.Dm, m, split,
+                                                dw.part);
     ++launch_counter();
     k_act_finish<<<1, 256, 0, s>>>(dw.part, (int)nblk, a, d.c, nmo, NL, rdm.p[1], n, d2);
     CASPT2_CUDA_TRY(cudaGetLastError());
   }
   // ---- sources: d1 and the adjoint integral blocks
+  double* W = dw.U1;                 // [fam][tuple][act][M][L'], vsize doubles
   ++launch_counter();
-  k_wsrc<<<launch_blocks(tall), 256, 0, s>>>(dw.T, dw.Lam, R, P, n, m, tall, dw.U1);
-  ++launch_counter();
-  if (n <= 4) {
-    const long total2 = w.vsize / ((long)n * n);
-    k_src_adj_ml<4><<<launch_blocks(total2), 256, 0, s>>>(w.dV, w.nV, C, d, rdm, dw.U1, m, total2,
-                                                         d1, G);
-  } else {
-    k_src_adj<<<launch_blocks(w.vsize), 256, 0, s>>>(w.dV, w.nV, C, d, rdm, dw.U1, m, w.vsize, d1,
-                                                     G);
-  }
+  k_wsrc<<<launch_blocks(ntot * m), 256, 0, s>>>(dw.T, dw.Lam, R, P, n, m, ntot, C.nfam, W);
   CASPT2_CUDA_TRY(cudaGetLastError());
+  if (w.nVs > 0) {
+    const long total2 = w.vsize / ((long)n * n);
+    const bool deal = total2 <= 152L * 4 * 256 && w.nVs > 1;
+    auto run = [&](auto ns) {
+      constexpr int NS = decltype(ns)::value;
+      ++launch_counter();
+      if (deal)
+        k_src_adj<NS, 8><<<launch_blocks(total2, 32), 256, 0, s>>>(w.dVs, w.nVs, C, d, rdm, W,
+                                                                   total2, d1, G, GP);
+      else
+        k_src_adj<NS, 1><<<launch_blocks(total2), 256, 0, s>>>(w.dVs, w.nVs, C, d, rdm, W, total2,
+                                                               d1, G, GP);
+    };
+    if (n == 1) run(std::integral_constant<int, 1>());
+    else if (n == 2) run(std::integral_constant<int, 2>());
+    else if (n == 3) run(std::integral_constant<int, 3>());
+    else if (n == 4) run(std::integral_constant<int, 4>());
+    else run(std::integral_constant<int, 0>());
+    CASPT2_CUDA_TRY(cudaGetLastError());
+  }
+  // the terms of the GEMM groups: the adjoint of V += X G is XA = W G^T, added to the targets
+  // of X's integral terms (all of classes F and G: 17 of the 42 ms that one thread per source
+  // element and term took at c20 a8 v200 n3)
+  const long ncol = w.A * n * n;
+  for (size_t gi = 0; gi < w.hG.size(); ++gi) {
+    const SrcGemmGroup& Gr = w.hG[gi];
+    const long K = ipow_host(a, Gr.g.ns);
+    if (K * ncol > sw.srcGcap) return CASPT2_EINVAL;
+    CASPT2_CUDA_TRY(launch_src_g(Gr.g, C, d, rdm, sw.srcG, s));
+    const long chunk = std::min<long>(ntot, sw.srcXcap / K);
+    if (chunk < 1) return CASPT2_EINVAL;
+    for (long r0 = 0; r0 < ntot; r0 += chunk) {
+      const long nr = std::min(chunk, ntot - r0);
+      CASPT2_CUDA_TRY(dgemm((int)nr, (int)K, (int)ncol, 1.0, W + ((long)Gr.fb * ntot + r0) * ncol,
+                            (int)ncol, false, sw.srcG, (int)ncol, true, 0.0, sw.srcX, (int)K, s));
+      ++launch_counter();
+      k_src_x_adj<<<launch_blocks(nr * K), 256, 0, s>>>(w.dX + w.gx_off[gi], (int)Gr.x.size(), C,
+                                                        d, Gr.g.ns, sw.srcX, r0, nr, d1, G, GP);
+      CASPT2_CUDA_TRY(cudaGetLastError());
+    }
+  }
   return CASPT2_OK;
 }
 

@@ -393,7 +393,7 @@ void build_src_plans(int cls, std::vector<SrcPlan>& out) {
 }
 
 void split_src_plans(int cls, const std::vector<SrcPlan>& in, std::vector<SrcPlan>& rest,
-                     std::vector<SrcGemmGroup>& groups) {
+                     std::vector<SrcGemmGroup>& groups, int max_ns) {
   const ClassDef& C = kClasses[cls];
   rest.clear();
   groups.clear();
@@ -435,7 +435,7 @@ void split_src_plans(int cls, const std::vector<SrcPlan>& in, std::vector<SrcPla
     }
     for (int j = 0; j < P.nloop; ++j)
       if (cls_of[j] == 2) pos[j] = nx++;
-    if (ns > 2 || nr > 3) {
+    if (ns > max_ns || nr > 3) {
       rest.push_back(P);
       continue;
     }

@@ -105,9 +105,10 @@ struct SrcGemmGroup {
   std::vector<SrcXTerm> x;
 };
 // Split the (pre-summed) source plans of class cls into GEMM groups and the terms that stay
-// with the plan interpreter.
+// with the plan interpreter.  max_ns: the largest number of shared loops of a group (K = a^ns;
+// three of them occur in classes A and C, with the 3-RDM: G then holds a^6 n^2 doubles).
 void split_src_plans(int cls, const std::vector<SrcPlan>& in, std::vector<SrcPlan>& rest,
-                     std::vector<SrcGemmGroup>& groups);
+                     std::vector<SrcGemmGroup>& groups, int max_ns);
 
 // Build the plans of class cls (0..6).  Deterministic; a few hundred terms.
 void build_act_plans(int cls, bool with_fock, std::vector<ActPlan>& out);
