@@ -898,7 +898,7 @@ __global__ void k_sector_energy(const double* __restrict__ Vt, const double* __r
     for (int q = 0; q < n; ++q) m1[q] = 0.0;
     for (int mu = 0; mu < msec; ++mu) {
       const double D = ee + omega[mu] - E0[L] + shift;
-      const double inv = 1.0 / D;
+      const double inv = recip(D);
       const double* row = Vt + (long)mu * ncol + t * n;
       const double vn = row[N] * inv;
       for (int q = 0; q < n; ++q) m1[q] += vn * row[q];

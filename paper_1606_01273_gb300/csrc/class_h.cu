@@ -191,7 +191,7 @@ k_classH(const double* __restrict__ Bp, const double* __restrict__ eps,
     double e = 0.0, nr = 0.0, n3 = 0.0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const double inv = 1.0 / (d0[q] + sh);
+      const double inv = recip(d0[q] + sh);
       const double x = num[q] * inv;
       e += x;
       nr = fma(x, inv, nr);
@@ -267,7 +267,8 @@ __global__ void k_classH_combine(const double* __restrict__ sums, const double* 
   }
 }
 
-// Split form: KK[(ia)][(jb)] = K_ij^ab (2 K_ij^ab - K_ij^ba) from the full K matrix.
+// Split form: KK[(ia)][(jb)] = K_ij^ab (2 K_ij^ab - K_ij^ba) from the full K matrix, j >= i
+// (the sums below read no other).
 __global__ void k_classH_num(const double* __restrict__ K, int c, int v, int i0, int i1,
                              double* __restrict__ KK) {
   const long cv = (long)c * v, e0 = (long)i0 * v * cv, total = (long)i1 * v * cv;
@@ -275,46 +276,65 @@ __global__ void k_classH_num(const double* __restrict__ K, int c, int v, int i0,
        e += (long)gridDim.x * blockDim.x) {
     const long ia = e / cv, jb = e % cv;
     const int i = ia / v, a = ia % v, j = jb / v, b = jb % v;
+    if (j < i) continue;
     const double k1 = K[e];
     KK[e] = k1 * (2.0 * k1 - K[((long)i * v + b) * cv + (long)j * v + a]);
   }
 }
 
-// Split form: per-shift sums over all (i, j, a, b) of KK / D, KK / D^2, KK / D^3 and the
-// smallest |D| with KK != 0; grid (nblk, nshift), one row of partial per block with only
-// its own shift's columns set (the others zero, the min column +inf for no element), so the
-// fixed-order column reduction of the fused kernel applies unchanged.
+// Split form: the sums of KK / D, KK / D^2, KK / D^3 over all (i, j, a, b) for G shifts of a
+// block row (blockIdx.y) and the smallest |D| with KK != 0; one row of partial per block with
+// only its own shifts' columns set (the others zero, the min column +inf for no element), so
+// the fixed-order column reduction of the fused kernel applies unchanged.
+//
+// What bounds it: nine FP64 operations per element and shift (the reciprocal three, the three
+// sums five, the denominator one) at two a clock and SM, 16 shifts for four states.  The
+// elements (ia, jb) and (jb, ia) are equal (K and D are symmetric), so only jb >= ia is
+// summed, off-diagonal ones twice; the G shifts of an element share its loads and give G
+// independent chains.  c42 v350, 16 shifts: 82.9 ms with one shift a block over the full
+// square.
+template <int G>
 __global__ void k_classH_sums(const double* __restrict__ KK, const double* __restrict__ eps,
                               const double* __restrict__ shifts, int nshift, int c, int v,
                               int i0, int i1, double* __restrict__ partial) {
   __shared__ double red[32];
-  const int k = blockIdx.y;
-  const double sh = shifts[k];
+  const int k0 = blockIdx.y * G;
   const long cv = (long)c * v;
-  double e = 0.0, nr = 0.0, n3 = 0.0;
+  double sh[G], e[G], nr[G], n3[G];
   // smallest |D| with KK != 0, kept as the bit pattern of |D| (non-negative doubles order
   // like their bit patterns, so the minimum runs on the integer units)
   unsigned long long dminb = 0x7FF0000000000000ull;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    sh[g] = shifts[min(k0 + g, nshift - 1)];
+    e[g] = nr[g] = n3[g] = 0.0;
+  }
   // rows (i, a) over the blocks, (j, b) of a row over the threads: index arithmetic once
   // per row and per j, not per element
   for (long ia = (long)i0 * v + blockIdx.x; ia < (long)i1 * v; ia += gridDim.x) {
     const int i = (int)(ia / v), a = (int)(ia % v);
-    const double base = eps[c + a] - eps[i] + sh;
+    const double base = eps[c + a] - eps[i];
     const double* row = KK + ia * cv;
-    for (int j = 0; j < c; ++j) {
+    for (int j = i; j < c; ++j) {
       const double bj = base - eps[j];
       const double* rj = row + (long)j * v;
-      for (int b = threadIdx.x; b < v; b += blockDim.x) {
-        const double num = rj[b];
-        const double D = bj + eps[c + b];
-        const double inv = recip(D);
-        const double x = num * inv;
-        e += x;
-        nr = fma(x, inv, nr);
-        n3 = fma(x * inv, inv, n3);
-        const unsigned long long db =
-            (unsigned long long)__double_as_longlong(D) & 0x7FFFFFFFFFFFFFFFull;
-        if ((__double_as_longlong(num) << 1) != 0 && db < dminb) dminb = db;
+      for (int b = (j == i ? a : 0) + threadIdx.x; b < v; b += blockDim.x) {
+        double num = rj[b];
+        if (j != i || b != a) num += num;
+        const double D0 = bj + eps[c + b];
+        const bool live = (__double_as_longlong(num) << 1) != 0;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const double D = D0 + sh[g];
+          const double inv = recip(D);
+          const double x = num * inv;
+          e[g] += x;
+          nr[g] = fma(x, inv, nr[g]);
+          n3[g] = fma(x * inv, inv, n3[g]);
+          const unsigned long long db =
+              (unsigned long long)__double_as_longlong(D) & 0x7FFFFFFFFFFFFFFFull;
+          if (live && db < dminb) dminb = db;
+        }
       }
     }
   }
@@ -323,12 +343,15 @@ __global__ void k_classH_sums(const double* __restrict__ KK, const double* __res
   double* out = partial + ((long)blockIdx.y * gridDim.x + blockIdx.x) * ncol;
   for (int t = threadIdx.x; t < 3 * nshift; t += blockDim.x) out[t] = 0.0;
   __syncthreads();
-  e = block_sum(e, red);
-  if (threadIdx.x == 0) out[k] = e;
-  nr = block_sum(nr, red);
-  if (threadIdx.x == 0) out[nshift + k] = nr;
-  n3 = block_sum(n3, red);
-  if (threadIdx.x == 0) out[2 * nshift + k] = n3;
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const double s1 = block_sum(e[g], red), s2 = block_sum(nr[g], red), s3 = block_sum(n3[g], red);
+    if (threadIdx.x == 0 && k0 + g < nshift) {
+      out[k0 + g] = s1;
+      out[nshift + k0 + g] = s2;
+      out[2 * nshift + k0 + g] = s3;
+    }
+  }
   dmin = block_min(dmin, red);
   if (threadIdx.x == 0) out[3 * nshift] = dmin;
 }
@@ -443,15 +466,34 @@ cudaError_t launch_classH_split(const double* f, const double* B, const double* 
   ++launch_counter();
   k_classH_num<<<(int)std::min<long>((total + 255) / 256, 152L * 32), 256, 0, s>>>(K, d.c, d.v, i0,
                                                                                   i1, KK);
-  const int nblk = (int)std::max<long>(1, std::min<long>(w.nblocks / nshift, 152L * 4));
+  // shifts per block row: the group of three to five that pads nshift least (one shift: one)
+  int G = 1;
+  if (nshift > 1) {
+    G = 4;
+    for (int g : {5, 3})
+      if ((nshift + g - 1) / g * g < (nshift + G - 1) / G * G) G = g;
+  }
+  const int ng = (nshift + G - 1) / G;
+  const int nblk = (int)std::max<long>(1, std::min<long>(w.nblocks / ng, 152L * 8));
   // one pass over b per (i, a, j) when v fits a block (no idle tail of lanes)
-  const int hthreads = d.v <= 1024 ? std::max(64, (d.v + 31) / 32 * 32) : 256;
+  const int hthreads = d.v <= 512 ? std::max(64, (d.v + 31) / 32 * 32) : 256;
+  const dim3 grid(nblk, ng);
   ++launch_counter();
-  k_classH_sums<<<dim3(nblk, nshift), hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0,
-                                                        i1, w.partial);
+  if (G == 1)
+    k_classH_sums<1><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
+                                               w.partial);
+  else if (G == 3)
+    k_classH_sums<3><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
+                                               w.partial);
+  else if (G == 4)
+    k_classH_sums<4><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
+                                               w.partial);
+  else
+    k_classH_sums<5><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
+                                               w.partial);
   const int ncol = 3 * nshift + 1;
   ++launch_counter();
-  k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, (long)nblk * nshift, ncol, w.sums);
+  k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, (long)nblk * ng, ncol, w.sums);
   ++launch_counter();
   k_classH_combine<<<1, 256, 0, s>>>(w.sums, w.W, n, scheme, ecls, ncls, mom, mindenom, status);
   return cudaGetLastError();

@@ -39,17 +39,16 @@ __device__ __forceinline__ double block_sum(double v, double* smem32) {
   return v;
 }
 
-// 1/d for the energy denominators: Newton's iteration x <- x + x (1 - d x) from the
-// hardware's approximate double reciprocal (rcp.approx.ftz.f64, about 20 correct bits);
-// two steps take the seed past double precision (error within an ulp or so).  d must be
+// 1/d for the energy denominators: one third-order step x <- x + x (e + e^2), e = 1 - d x (the
+// first terms of the geometric series for 1 / (1 - e)), from the hardware's approximate double
+// reciprocal (rcp.approx.ftz.f64, about 20 correct bits): e^3 is below 2^-60, so the result is
+// within an ulp or so, in three FP64 operations where two Newton steps take four.  d must be
 // a normal number.
 __device__ __forceinline__ double recip(double d) {
   double x;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(x) : "d"(d));
-  double e = fma(-d, x, 1.0);
-  x = fma(x, e, x);
-  e = fma(-d, x, 1.0);
-  return fma(x, e, x);
+  const double e = fma(-d, x, 1.0);
+  return fma(x, fma(e, e, e), x);
 }
 
 __device__ __forceinline__ double block_min(double v, double* smem32) {
