@@ -27,6 +27,8 @@ struct GemmArgs {
   const double* B; long bk, bj;
   double* C; long ci, cj;
   long sA, sB, sC;                   // batch strides (blockIdx.y)
+  unsigned akin, bkin;               // K in runs of akin (bkin) elements, the runs akout
+  long akout, bkout;                 // (bkout) apart; a run as long as K: one run
   int tn, kc, split, sym;            // column tiles, K per block (multiple of kGK), cluster size
 };
 
@@ -60,13 +62,18 @@ __global__ void __launch_bounds__(256) k_dgemm(GemmArgs g) {
     if (g.bj == 1) { jb[u] = l % kGT; kb[u] = l / kGT; } else { kb[u] = l % kGK; jb[u] = l / kGK; }
   }
   double va[2], vb[2];
+  auto at = [](int k, long st, unsigned kin, long kout) {
+    if ((unsigned)k < kin) return k * st;
+    const unsigned p = (unsigned)k / kin;
+    return p * kout + (k - p * kin) * st;
+  };
   auto load = [&](int k0) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int gi = i0 + ia[u], gk = k0 + ka[u];
-      va[u] = (gi < g.M && gk < kend) ? A[gi * g.ai + gk * g.ak] : 0.0;
+      va[u] = (gi < g.M && gk < kend) ? A[gi * g.ai + at(gk, g.ak, g.akin, g.akout)] : 0.0;
       const int gj = j0 + jb[u], gq = k0 + kb[u];
-      vb[u] = (gj < g.N && gq < kend) ? B[gq * g.bk + gj * g.bj] : 0.0;
+      vb[u] = (gj < g.N && gq < kend) ? B[at(gq, g.bk, g.bkin, g.bkout) + gj * g.bj] : 0.0;
     }
   };
   auto store = [&](int buf) {
@@ -195,6 +202,8 @@ cudaError_t gemm_timer_collect(GemmTimer& t, double* ms, double* flops, long* la
 namespace {
 // tiles: output tiles of one product; the rest of the grid and the launch.
 cudaError_t launch_dgemm(GemmArgs g, long tiles, int batch, double flops, cudaStream_t s) {
+  if (g.akin == 0) g.akin = 0xFFFFFFFFu;
+  if (g.bkin == 0) g.bkin = 0xFFFFFFFFu;
   // K over a cluster while the blocks do not fill the chip (two a SM) and a block keeps at
   // least two chunks: 48 tiles of K = 1024 take 8.1 us a unit of K unsplit and 8.1 / 6 split
   int split = 1;
@@ -249,6 +258,27 @@ cudaError_t dgemm(int M, int N, int K, double alpha, const double* A, int lda, b
   g.tn = (g.N + kGT - 1) / kGT;
   const long tiles = (long)((g.M + kGT - 1) / kGT) * g.tn;
   return launch_dgemm(g, tiles, batch, 2.0 * M * N * (double)K * batch, s);
+}
+
+cudaError_t dgemm_views(int M, int N, int K, double alpha, const KView& A, const KView& B,
+                        double beta, double* C, long ldc, cudaStream_t s) {
+  if (M <= 0 || N <= 0) return cudaSuccess;
+  const long straight = (long)((M + 7) / 8) * ((N + 31) / 32);
+  const long turned = (long)((N + 7) / 8) * ((M + 31) / 32);
+  const bool t = turned < straight;
+  const KView &a = t ? B : A, &b = t ? A : B;
+  GemmArgs g{};
+  g.M = t ? N : M;
+  g.N = t ? M : N;
+  g.K = K;
+  g.alpha = alpha;
+  g.beta = beta;
+  g.A = a.X; g.ai = a.rs; g.ak = a.cs; g.akin = (unsigned)a.kin; g.akout = a.kout;
+  g.B = b.X; g.bj = b.rs; g.bk = b.cs; g.bkin = (unsigned)b.kin; g.bkout = b.kout;
+  g.C = C; g.ci = t ? 1 : ldc; g.cj = t ? ldc : 1;
+  g.tn = (g.N + kGT - 1) / kGT;
+  const long tiles = (long)((g.M + kGT - 1) / kGT) * g.tn;
+  return launch_dgemm(g, tiles, 1, 2.0 * M * N * (double)K, s);
 }
 
 cudaError_t dgemm_sym(int N, int K, double alpha, const double* A, int lda, bool ta,

@@ -43,6 +43,11 @@ cudaError_t gemm_timer_collect(GemmTimer& t, double* ms, double* flops, long* la
 cudaError_t dgemm(int M, int N, int K, double alpha, const double* A, int lda, bool ta,
                   const double* B, int ldb, bool tb, double beta, double* C, int ldc,
                   cudaStream_t s, int batch = 1, long sA = 0, long sB = 0, long sC = 0);
+// C[i][j] (ldc) = alpha * sum_k A(i, k) B(j, k) + beta * C, with general strides and K in runs:
+// A(i, k) = A[i * ars + (k / akin) * akout + (k % akin) * acs], B alike.
+struct KView { const double* X; long rs, cs, kin, kout; };
+cudaError_t dgemm_views(int M, int N, int K, double alpha, const KView& A, const KView& B,
+                        double beta, double* C, long ldc, cudaStream_t s);
 // Same product when the N x N result is known to be symmetric (A^T A, X^T F X): only the
 // upper-triangle tiles are computed, each written to both triangles.
 cudaError_t dgemm_sym(int N, int K, double alpha, const double* A, int lda, bool ta,

@@ -26,12 +26,14 @@
 #include <cstdint>
 #include <mutex>
 
+#include "linalg.cuh"
 #include "ozaki.cuh"
 
 namespace caspt2 {
 
 namespace {
 
+constexpr double kOzDirectFmas = 33554432.0;        // products up to 2^25 FMAs run in FP64
 constexpr int kOzM = 128, kOzN = 64;
 constexpr int kOzThreads = 320;                     // warps: TMA, MMA, eight epilogue
 constexpr long kOzSpin = 1L << 22;
@@ -572,6 +574,15 @@ cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc) {
 cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, int M, int N,
                       int K, double alpha, double beta, double* C, long ldc, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  // Small products run as plain FP64: slicing, scaling and the split GEMM are at least six
+  // launches (30 to 90 us for the products of a c5 a3 v70 solve), where the FP64 kernel needs
+  // one and is exact to FP64 rounding.  2^25 multiply-adds take it about 60 us, provided its
+  // blocks fill the chip (K is split over at most eight).
+  const long blocks = (long)((M + 31) / 32) * ((N + 31) / 32) * std::max(1, std::min(8, K / 32));
+  const double fmas = (double)M * N * K;
+  if (fmas <= kOzDirectFmas && (blocks >= 152 || fmas <= kOzDirectFmas * blocks / 152.0))
+    return dgemm_views(M, N, K, alpha, KView{A.X, A.rs, A.cs, A.kin, A.kout},
+                       KView{B.X, B.rs, B.cs, B.kin, B.kout}, beta, C, ldc, s);
   const int Kp = oz_kpad(std::max(K, 1));
   const size_t a_bytes = oz_slice_bytes(M, std::max(K, 1), w.S);
   const size_t b_bytes = same ? 0 : oz_slice_bytes(N, std::max(K, 1), w.S);
