@@ -121,10 +121,19 @@ __device__ __forceinline__ void tma_load3(uint32_t dst, const CUtensorMap* map, 
       : "memory");
 }
 
+// Output tiles of one K split: all, or for a symmetric result (C = A A^T) those that reach the
+// diagonal or lie right of it, n tile >= 2 m tile.
+__host__ __device__ inline long oz_tiles(int ntm, int ntn, int sym) {
+  if (!sym) return (long)ntm * ntn;
+  long t = 0;
+  for (int m = 0; m < ntm && 2 * m < ntn; ++m) t += ntn - 2 * m;
+  return t;
+}
+
 __global__ void __launch_bounds__(kOzThreads, 1)
 k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const double* __restrict__ sa, const double* __restrict__ sb, int M, int N, int Kp,
-          int S, int chunks_per_split, int nsplit, double alpha, double beta,
+          int S, int chunks_per_split, int nsplit, int sym, double alpha, double beta,
           double* __restrict__ C, long ldc, double* __restrict__ part, int* err) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[kOzStages], empty[kOzStages], tfull, tempty;
@@ -162,12 +171,22 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   // tiles (n tile, m tile, K split) in a persistent loop; every role walks the same
   // sequence, and the stage ring and barrier phases run on across tiles
   const int ntn = (N + kOzN - 1) / kOzN, ntm = (M + kOzM - 1) / kOzM;
-  const long ntiles = (long)ntn * ntm * nsplit;
+  const long per_split = oz_tiles(ntm, ntn, sym);
+  const long ntiles = per_split * nsplit;
   const int spc = kOzKChunk / kOzKs;              // stages per exact chunk
   auto tile_of = [&](long ti, int& m0, int& n0, int& z, int& gbeg, int& nst) {
-    n0 = (int)(ti % ntn) * kOzN;
-    m0 = (int)((ti / ntn) % ntm) * kOzM;
-    z = (int)(ti / ((long)ntn * ntm));
+    z = (int)(ti / per_split);
+    long t = ti % per_split;
+    int mt = 0;
+    if (sym) {                                    // row mt holds the n tiles 2 mt .. ntn - 1
+      while (t >= ntn - 2 * mt) { t -= ntn - 2 * mt; ++mt; }
+      t += 2 * mt;
+    } else {
+      mt = (int)(t / ntn);
+      t %= ntn;
+    }
+    n0 = (int)t * kOzN;
+    m0 = mt * kOzM;
     gbeg = z * chunks_per_split * spc;            // stages of K split z
     nst = max(0, min(Kp / kOzKs, gbeg + chunks_per_split * spc) - gbeg);
   };
@@ -306,6 +325,10 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
             if (col < N) {
               const double v = sr * sb[col] * acc[j];
               crow[col] = beta == 0.0 ? v : v + beta * crow[col];
+              if (sym && n0 >= m0 + kOzM) {       // right of the diagonal block: mirrored
+                double* ct = C + (long)col * ldc + row;
+                *ct = beta == 0.0 ? v : v + beta * *ct;
+              }
             }
           }
         }
@@ -331,15 +354,18 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   }
 }
 
-// C[i][j] = sum_z part[z][i][j] (fixed order) + beta C[i][j]
-__global__ void k_oz_reduce(const double* __restrict__ part, int nsplit, int M, int N,
+// C[i][j] = sum_z part[z][i][j] (fixed order) + beta C[i][j]; sym: blocks left of the diagonal
+// were not formed, their elements are read at (j, i)
+__global__ void k_oz_reduce(const double* __restrict__ part, int nsplit, int M, int N, int sym,
                             double beta, double* __restrict__ C, long ldc) {
   const long total = (long)M * N;
   for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
        e += (long)gridDim.x * blockDim.x) {
     double v = 0.0;
-    for (int z = 0; z < nsplit; ++z) v += part[(long)z * total + e];
-    double* c = C + (e / N) * ldc + e % N;
+    const long i = e / N, j = e % N;
+    const long src = sym && j / kOzN < 2 * (i / kOzM) ? j * N + i : e;
+    for (int z = 0; z < nsplit; ++z) v += part[(long)z * total + src];
+    double* c = C + i * ldc + j;
     *c = beta == 0.0 ? v : v + beta * *c;
   }
 }
@@ -495,7 +521,8 @@ bool slice_map(CUtensorMap* map, const __nv_bfloat16* X, int R, int Kp, int S, i
 
 cudaError_t oz_gemm(const __nv_bfloat16* As, const double* sa, const __nv_bfloat16* Bs,
                     const double* sb, int M, int N, int Kp, int S, double alpha, double beta,
-                    double* C, long ldc, int* err, cudaStream_t s, int nsplit, double* part) {
+                    double* C, long ldc, int* err, cudaStream_t s, int nsplit, double* part,
+                    bool sym) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (S < 1 || S > kOzMaxSlices || Kp % kOzKStage != 0) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(As) | reinterpret_cast<uintptr_t>(Bs)) & 15)
@@ -516,19 +543,19 @@ cudaError_t oz_gemm(const __nv_bfloat16* As, const double* sa, const __nv_bfloat
   nsplit = (nchunk + cps - 1) / cps;
   if (nsplit > 1 && !part) return cudaErrorInvalidValue;
   // persistent CTAs (one per SM: the ring and all 512 TMEM columns) over the tiles
-  const long ntiles = (long)((N + kOzN - 1) / kOzN) * ((M + kOzM - 1) / kOzM) * nsplit;
+  const long ntiles = oz_tiles((M + kOzM - 1) / kOzM, (N + kOzN - 1) / kOzN, sym) * nsplit;
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const int grid = (int)std::min<long>(ntiles, nsm);
   ++launch_counter();
-  k_oz_gemm<<<grid, kOzThreads, smem, s>>>(ma, mb, sa, sb, M, N, Kp, S, cps, nsplit, alpha, beta,
-                                           C, ldc, nsplit > 1 ? part : nullptr, err);
+  k_oz_gemm<<<grid, kOzThreads, smem, s>>>(ma, mb, sa, sb, M, N, Kp, S, cps, nsplit, sym ? 1 : 0,
+                                           alpha, beta, C, ldc, nsplit > 1 ? part : nullptr, err);
   if (nsplit > 1) {
     const long total = (long)M * N;
     ++launch_counter();
     k_oz_reduce<<<(int)std::max<long>(1, std::min<long>((total + 255) / 256, 152L * 8)), 256, 0, s>>>(
-        part, nsplit, M, N, beta, C, ldc);
+        part, nsplit, M, N, sym ? 1 : 0, beta, C, ldc);
   }
   return cudaGetLastError();
 }
@@ -595,7 +622,7 @@ cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, in
   if ((e = oz_split(A, M, K, Kp, w.S, as, sa, s)) != cudaSuccess) return e;
   if (!same && (e = oz_split(B, N, K, Kp, w.S, bs, sb, s)) != cudaSuccess) return e;
   // split K over CTAs when the output has few tiles (about two waves of 152 SMs)
-  const long tiles = (long)((M + 127) / 128) * ((N + 63) / 64);
+  const long tiles = oz_tiles((M + kOzM - 1) / kOzM, (N + kOzN - 1) / kOzN, same);
   const int nchunk = (Kp + kOzKChunk - 1) / kOzKChunk;
   int nsplit = (int)std::max<long>(1, std::min<long>(nchunk, (304 + tiles - 1) / tiles));
   if (nsplit > 1) {
@@ -608,7 +635,8 @@ cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, in
       w.part_n = need;
     }
   }
-  return oz_gemm(as, sa, bs, sb, M, N, Kp, w.S, alpha, beta, C, ldc, w.err, s, nsplit, w.part);
+  return oz_gemm(as, sa, bs, sb, M, N, Kp, w.S, alpha, beta, C, ldc, w.err, s, nsplit, w.part,
+                 same);
 }
 
 }  // namespace caspt2

@@ -38,10 +38,11 @@ cudaError_t oz_split(const OzView& v, int R, int K, int Kp, int S, __nv_bfloat16
 // C[i][j] (ldc) = alpha * sum_k A(i,k) B(j,k) + beta * C[i][j] from the slices of A
 // (M x Kp) and B (N x Kp).  err receives a nonzero code if a bounded wait gave up.
 // nsplit > 1 splits K (in exact chunks) over CTAs; part then holds nsplit * M * N doubles.
+// sym: B is A, only the tiles at and right of the diagonal are formed and mirrored.
 cudaError_t oz_gemm(const __nv_bfloat16* As, const double* sa, const __nv_bfloat16* Bs,
                     const double* sb, int M, int N, int Kp, int S, double alpha, double beta,
                     double* C, long ldc, int* err, cudaStream_t s, int nsplit = 1,
-                    double* part = nullptr);
+                    double* part = nullptr, bool sym = false);
 
 // Device workspace of the split GEMMs, grown on demand (growth synchronises the device)
 // and owned by the caller.  on = false selects the plain FP64 paths.
@@ -59,7 +60,7 @@ struct OzWork {
 void oz_release(OzWork& w);
 
 // C (ldc) = alpha * A B^T + beta * C for an M x K view A and an N x K view B (same: B is A,
-// sliced once).
+// sliced once, half of the symmetric result formed).  C does not overlap A or B.
 cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, int M, int N,
                       int K, double alpha, double beta, double* C, long ldc, cudaStream_t s);
 
