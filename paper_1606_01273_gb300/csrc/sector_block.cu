@@ -98,12 +98,14 @@ __device__ void tridiagonalise(double* A, int ld, int m, const Vecs& q) {
       }
     }
     __syncthreads();
-    // w = tau p - (tau^2 / 2)(u . p) u, in place of p
+    // w = tau p - (tau^2 / 2)(u . p) u, in place of p.  A sector without overlap is rounding
+    // noise that shrinks by 1e-17 a step: tau reaches 1e280 and tau^2 leaves the FP64 range,
+    // tau (u . p), of the size of A22, does not.
     if (warp == 0) {
       double s = 0.0;
       for (int j = lane; j < n1; j += 32) s = fma(q.u[j], q.p[j], s);
       s = warp_sum(s);
-      const double t = q.tau[k], g = 0.5 * t * t * s;
+      const double t = q.tau[k], ts = t * s, g = 0.5 * t * ts;
       for (int j = lane; j < n1; j += 32) q.p[j] = fma(-g, q.u[j], t * q.p[j]);
     }
     __syncthreads();

@@ -49,3 +49,20 @@ def test_sector_sizes_match_oracle(cp, name, scheme):
         scale = max(np.abs(e).max(), np.abs(nr).max(), 1e-12)
         assert np.abs(r.e_class[cls] - e).max() <= RTOL * scale, cls
         assert np.abs(r.norm_class[cls] - nr).max() <= RTOL * scale, cls
+
+
+@pytest.mark.parametrize("size", [dict(nclosed=13, nact=3, nvirt=108, naux=372, seed=5011),
+                                  dict(nclosed=2, nact=3, nvirt=3, naux=24, seed=11),
+                                  dict(nclosed=2, nact=3, nvirt=3, naux=24, seed=12),
+                                  dict(nclosed=2, nact=2, nvirt=3, naux=24, seed=13)])
+def test_sectors_without_overlap(cp, size):
+    """Two active electrons: the antisymmetric sector of class F has no overlap, its matrix is
+    rounding noise of 1e-17 whose reduction passes through elements of 1e-80 and below."""
+    p = make_problem(nstate=2, nelact=2, **size)
+    st = o2.setup(p, xms=True, kmax=4)
+    M1, M2, _ = oc.class_moments(p, st, "F", shift=0.2)
+    e, nr = -np.einsum("llk->lk", M1), np.diagonal(M2)
+    r = cp.solve_problem(p, xms=1, shift=0.2)
+    scale = max(np.abs(e).max(), np.abs(nr).max(), 1e-12)
+    assert np.abs(r.e_class["F"] - e).max() <= RTOL * scale
+    assert np.abs(r.norm_class["F"] - nr).max() <= RTOL * scale
