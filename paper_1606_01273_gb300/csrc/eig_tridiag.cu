@@ -279,21 +279,61 @@ __device__ void house_vec(const double* __restrict__ x, int n1, double* __restri
   __syncthreads();
 }
 
+// Bounded barrier of all blocks of a cooperative launch: arrivals add to one counter that only
+// grows, and every block polls it for G times the number of barriers passed (target).  One
+// trip to L2 for the arrival and one for the poll, where a reset counter and a generation
+// word take four.  A wait that gives up sets *err, which the others see in theirs.
+__device__ bool grid_sync_count(unsigned* count, unsigned target, int* err) {
+  __syncthreads();
+  __shared__ int ok;
+  if (threadIdx.x == 0) {
+    ok = 1;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    for (long it = 0;; ++it) {
+      unsigned cur;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(count) : "memory");
+      if (cur >= target) break;
+      if ((it & 63) == 63 && *(volatile int*)err != 0) { ok = 0; break; }
+      if (it > kSpinLimit) {
+        atomicExch(err, 1);
+        ok = 0;
+        break;
+      }
+      if (it > 512) __nanosleep(32);
+    }
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
+// Sum over the lanes of an aligned group of `width` (a power of two), in every lane.
+__device__ __forceinline__ double group_sum(double v, int width) {
+  for (int o = width >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // Householder reduction with the matrix resident in shared memory: block b owns the
 // rows r = b (mod gridDim.x).  One bounded grid barrier per step:
 //   p_i = tau sum_j A_ij v_j for owned rows (published)                | barrier
-//   every block: w = p - (tau/2)(p.v) v, update of its rows, and — redundantly — the
-//   update of row k+1 (published by its owner after the previous step) and the next
-//   reflector, so no second barrier is needed; the owner of row k+2 publishes it.
-// Shared layout: rows [nloc][m], v[m], w[m], r[m] (all indexed by absolute column).
-// pbuf[2][m], rowbuf[2][m] are double-buffered by step parity; sync[0..1] barrier state,
-// sync[2] error flag.
+//   every block: w = p - (tau/2)(p.v) v, and — redundantly — the update of row k+1
+//   (published by its owner after the previous step) with the norm of its trailing part; the
+//   next reflector's scalars by warp 0 while the other warps update the owned rows; the
+//   owner of row k+2 publishes it.
+// Shared layout: rows [nloc][m], v[m], w[m] (they change places each step), r[m] (all indexed
+// by absolute column).  pbuf[2][m], rowbuf[2][m] are double-buffered by step parity; sync[0]
+// barrier count, sync[2] error flag.
+//
+// What bounds it: at m = 1536 a third of the time is the FP64 unit (3 m^2 / 152 lane operations a
+// block and step), the rest, and below m = 400 nearly all of it, the chain of a step: barrier,
+// two block sums and the reflector's scalars.  An FP64 warp instruction takes 64 clocks of a
+// sub-partition whether its lanes carry anything or not, so a block sum costs 5 x 64 clocks a
+// warp and sub-partition: as few warps as the rows need (tridiag_threads).
 __global__ void __launch_bounds__(512)
 k_tridiag_smem(const double* __restrict__ A, int m, double* __restrict__ vbuf,
                double* __restrict__ tau, double* __restrict__ d, double* __restrict__ e,
                double* __restrict__ pbuf, double* __restrict__ rowbuf, unsigned* sync) {
   extern __shared__ double smem[];
-  __shared__ double red[32];
+  __shared__ double red[32], red2[32];
   __shared__ double sh[4];
   int* err = reinterpret_cast<int*>(sync + 2);
   const int G = gridDim.x, b = blockIdx.x;
@@ -316,8 +356,9 @@ k_tridiag_smem(const double* __restrict__ A, int m, double* __restrict__ vbuf,
     for (int i = threadIdx.x; i < m - 1; i += blockDim.x) vbuf[1 + i] = v[1 + i];
     if (threadIdx.x == 0) { tau[0] = t; d[0] = r[0]; e[0] = sh[2]; }
   }
+  unsigned target = 0;
   for (int k = 0; k + 2 < m; ++k) {
-    const int k1 = k + 1;
+    const int k1 = k + 1, k2 = k + 2;
     // p = tau A v for the owned trailing rows (one warp per row, four partial sums)
     const int lfirst = (k1 - b + G - 1) / G;       // first owned row index >= k+1
     for (int li = lfirst + warp; li < nloc; li += nwarp) {
@@ -325,62 +366,97 @@ k_tridiag_smem(const double* __restrict__ A, int m, double* __restrict__ vbuf,
       double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
       int j = k1 + lane;
       for (; j + 96 < m; j += 128) {
-        s0 += row[j] * v[j];
-        s1 += row[j + 32] * v[j + 32];
-        s2 += row[j + 64] * v[j + 64];
-        s3 += row[j + 96] * v[j + 96];
+        s0 = fma(row[j], v[j], s0);
+        s1 = fma(row[j + 32], v[j + 32], s1);
+        s2 = fma(row[j + 64], v[j + 64], s2);
+        s3 = fma(row[j + 96], v[j + 96], s3);
       }
-      for (; j < m; j += 32) s0 += row[j] * v[j];
-      double s = (s0 + s1) + (s2 + s3);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      for (; j < m; j += 32) s0 = fma(row[j], v[j], s0);
+      const double s = group_sum((s0 + s1) + (s2 + s3), 32);
       if (lane == 0) pbuf[(long)(k & 1) * m + b + li * G] = t * s;
     }
-    if (!grid_sync_bounded(sync, sync + 1, err)) return;
+    target += (unsigned)G;
+    if (!grid_sync_count(sync, target, err)) return;
     // g = (tau/2) p.v; with w = p - g v the update A -= v w^T + w v^T reads
-    // A_ij -= v_i p_j + (p_i - 2 g v_i) v_j  (two FMAs per element)
+    // A_ij -= v_i p_j + (p_i - 2 g v_i) v_j  (two FMAs per element); the old row k+1 (the
+    // copy published before the barrier) comes in with p
+    const double* old = (k == 0) ? A + (long)k1 * m : rowbuf + (long)(k1 & 1) * m;
     double s = 0.0;
+#pragma unroll 4
     for (int j = k1 + threadIdx.x; j < m; j += blockDim.x) {
-      const double pj = __ldcg(pbuf + (long)(k & 1) * m + j);
+      const double pj = __ldcg(pbuf + (long)(k & 1) * m + j), oj = __ldcg(old + j);
       w[j] = pj;
-      s += pj * v[j];
+      r[j] = oj;
+      s = fma(pj, v[j], s);
     }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) sh[3] = t * s;             // 2 g
+    s = group_sum(s, 32);
+    if (lane == 0) red[warp] = s;
     __syncthreads();
-    const double g2 = sh[3];
+    const double g2 = t * group_sum(red[lane & (nwarp - 1)], nwarp);   // 2 g
+    // row k+1 after this step and the square of its part right of the subdiagonal
+    double q = 0.0;
+    {
+      const double vi = v[k1], bi = fma(-g2, vi, w[k1]);
+#pragma unroll 4
+      for (int j = k1 + threadIdx.x; j < m; j += blockDim.x) {
+        const double x = fma(-bi, v[j], fma(-vi, w[j], r[j]));
+        r[j] = x;
+        if (j > k2) q = fma(x, x, q);
+      }
+    }
+    const bool next = k + 3 < m;
+    if (next) {
+      q = group_sum(q, 32);
+      if (lane == 0) red2[warp] = q;
+    }
+    __syncthreads();
+    if (next && warp == 0) {
+      // beta = -sign(alpha) |x|, tau = 1 + |alpha| / |x|, v = x / (alpha - beta) with v_0 = 1;
+      // |x| and 1 / |x| from the hardware's approximate reciprocal root y by the binomial
+      // series (1 - z)^(-1/2) = 1 + z/2 + 3 z^2/8, z = 1 - |x|^2 y^2 below 2^-19
+      q = group_sum(red2[lane & (nwarp - 1)], nwarp);
+      const double al = r[k2], sig = fma(al, al, q);
+      double beta = al, tn = 0.0, scale = 0.0;
+      if (q != 0.0 && !(sig < 1e-280)) {
+        double y;
+        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(sig));
+        const double s0 = sig * y, z = fma(-s0, y, 1.0), c = z * fma(0.375, z, 0.5);
+        const double nr = fma(s0, c, s0), ir = fma(y, c, y);
+        beta = -copysign(nr, al);
+        tn = fma(fabs(al), ir, 1.0);
+        scale = copysign(recip(fabs(al) + nr), al);
+      }
+      if (lane == 0) { sh[0] = tn; sh[1] = scale; sh[2] = beta; }
+    }
     // update of the owned rows
     for (int li = lfirst; li < nloc; ++li) {
       const int i = b + li * G;
       const double vi = v[i], bi = fma(-g2, vi, w[i]);
       double* row = rows + (long)li * m;
+#pragma unroll 4
       for (int j = k1 + threadIdx.x; j < m; j += blockDim.x)
         row[j] = fma(-bi, v[j], fma(-vi, w[j], row[j]));
     }
-    // row k+1 after this step (every block, from the copy published before the barrier)
-    const double* old = (k == 0) ? A + (long)k1 * m : rowbuf + (long)(k1 & 1) * m;
-    {
-      const double vi = v[k1], bi = fma(-g2, vi, w[k1]);
-      for (int j = k1 + threadIdx.x; j < m; j += blockDim.x)
-        r[j] = fma(-bi, v[j], fma(-vi, w[j], __ldcg(old + j)));
-    }
     __syncthreads();
     // the owner of row k+2 publishes it for the next step
-    const int k2 = k + 2;
-    if (k2 < m && (k2 % G) == b) {
+    if ((k2 % G) == b) {
       const double* row = rows + (long)(k2 / G) * m;
       for (int j = k2 + threadIdx.x; j < m; j += blockDim.x)
         rowbuf[(long)(k2 & 1) * m + j] = row[j];
     }
-    if (k + 3 < m) {
-      // next reflector from row k+1's trailing part (v is free again)
-      house_vec(r + k2, m - k2, v + k2, red, sh);
+    if (next) {
+      // next reflector from row k+1's trailing part, in the place of p
       t = sh[0];
-      if (b == 0) {
-        for (int i = threadIdx.x; i < m - k2; i += blockDim.x)
-          vbuf[(long)k1 * m + k2 + i] = v[k2 + i];
-        if (threadIdx.x == 0) { tau[k1] = t; d[k1] = r[k1]; e[k1] = sh[2]; }
+      const double scale = sh[1];
+      for (int j = k2 + threadIdx.x; j < m; j += blockDim.x) {
+        const double x = j == k2 ? 1.0 : r[j] * scale;
+        w[j] = x;
+        if (b == 0) vbuf[(long)k1 * m + j] = x;
       }
+      double* x = v;
+      v = w;
+      w = x;
+      if (b == 0 && threadIdx.x == 0) { tau[k1] = t; d[k1] = r[k1]; e[k1] = sh[2]; }
     } else if (b == 0 && threadIdx.x == 0) {
       d[m - 2] = r[m - 2];
       e[m - 2] = r[m - 1];
@@ -388,9 +464,16 @@ k_tridiag_smem(const double* __restrict__ A, int m, double* __restrict__ vbuf,
     __syncthreads();
   }
   // last diagonal element from its owner
-  if (m >= 2 && ((m - 1) % G) == b && threadIdx.x == 0)
+  if (m >= 2 && ((m - 1) % G) == b && threadIdx.x == 0) {
     d[m - 1] = rows[(long)((m - 1) / G) * m + m - 1];
+    e[m - 1] = 0.0;
+  }
 }
+
+// Threads of a block of k_tridiag_smem: with up to three rows a block the block sums decide
+// (m = 216: 1.01 ms with 128, 1.04 with 256, 1.29 with 512 threads; 1.58 before with 512; m = 384:
+// 2.08, 2.09, 2.47), with more the rows (m = 864: 7.3, 6.3, 7.2 ms; m = 1536: 22.5, 17.7, 18.7 ms).
+int tridiag_threads(int m, int G) { return (m + G - 1) / G <= 3 ? 128 : 256; }
 
 // Shared memory of k_tridiag_smem for m columns on G blocks (0 if it does not fit).
 constexpr size_t kTridiagSmemMax = 200ull * 1024;
@@ -879,7 +962,8 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
     void* args[] = {&Ac, (void*)&m, &vbuf, &tau, &d, &e, &pbuf, &rowbuf, &sync};
     ++launch_counter();
     if (tm && tm->e0) CASPT2_CUDA_TRY(cudaEventRecord(tm->e0, s));
-    CASPT2_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_tridiag_smem, Gs, 512, args, smem_b, s));
+    CASPT2_CUDA_TRY(cudaLaunchCooperativeKernel((void*)k_tridiag_smem, Gs,
+                                                tridiag_threads(m, Gs), args, smem_b, s));
     if (tm && tm->e1) CASPT2_CUDA_TRY(cudaEventRecord(tm->e1, s));
     int herr = 0;
     CASPT2_CUDA_TRY(cudaMemcpyAsync(&herr, sync + 2, sizeof(int), cudaMemcpyDeviceToHost, s));
