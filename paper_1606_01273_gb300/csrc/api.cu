@@ -82,6 +82,8 @@ struct caspt2_ctx {
   // precision form: split BF16 tensor-core GEMMs, class-H pair integrals kept for the densities
   OzWork oz{};
   double *hK = nullptr, *hKK = nullptr, *hpack = nullptr;
+  double* hsl = nullptr;              // plain form: K chunk of launch_classH_sliced
+  long hslcap = 0;                    // its doubles, 0: the fused kernel serves
   // one-body couplings between classes: dbar2 off-diagonal blocks (opt.dens_offdiag)
   bool x_alloc = false;
   CrossWork xw{};
@@ -262,7 +264,7 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
   ALLOC(c->R, n * n);
   ALLOC(c->status, 1);
   // class H work
-  c->hw.nblocks = classH_blocks(d);
+  c->hw.nblocks = classH_partial_rows(d, o.scheme, o.precision == CASPT2_BF16X);
   const size_t nshift = (size_t)classH_nshift(d, o.scheme);
   ALLOC(c->hw.Bp, (size_t)d.c * X * d.v);
   ALLOC(c->hw.eps, nmo);
@@ -280,6 +282,16 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       ALLOC(c->hK, cv * cv);
       ALLOC(c->hKK, cv * cv);
       ALLOC(c->hpack, (size_t)d.X * cv);
+    }
+  }
+  if (st == CASPT2_OK && o.precision == CASPT2_FP64 && (o.class_mask >> CASPT2_CLASS_H & 1u)) {
+    // without the memory for it the fused kernel serves
+    c->hslcap = classH_sliced_work(d, o.scheme);
+    if (c->hslcap > 0 && (c->alloc(&c->hsl, (size_t)c->hslcap) != CASPT2_OK ||
+                          classH_sliced_reserve(d, c->oz) != cudaSuccess)) {
+      oz_release(c->oz);
+      cudaGetLastError();
+      c->hslcap = 0;
     }
   }
   ALLOC(c->lamNL, (size_t)CASPT2_NCLASS * n);
@@ -616,6 +628,12 @@ int solve_impl(caspt2_ctx* c, void* stream) {
                                         c->mom + (long)CASPT2_CLASS_H * msz, c->mindenom, c->oz,
                                         c->hpack, c->hK, c->hKK, s, o.closed_begin,
                                         o.closed_end));
+  } else if ((o.class_mask >> CASPT2_CLASS_H & 1u) && c->hslcap > 0) {
+    CASPT2_CUDA_TRY(launch_classH_sliced(c->f, c->B, c->Ftil, c->E0, o.shift, o.scheme, d, c->hw,
+                                         c->status, c->ecls + (long)CASPT2_CLASS_H * n * n,
+                                         c->ncls + (long)CASPT2_CLASS_H * n,
+                                         c->mom + (long)CASPT2_CLASS_H * msz, c->mindenom, c->oz,
+                                         c->hsl, c->hslcap, s, o.closed_begin, o.closed_end));
   } else if (o.class_mask >> CASPT2_CLASS_H & 1u) {
     CASPT2_CUDA_TRY(launch_classH(c->f, c->B, c->Ftil, c->E0, o.shift, o.scheme, d, c->hw,
                                   c->status, c->ecls + (long)CASPT2_CLASS_H * n * n,

@@ -293,13 +293,14 @@ __global__ void k_classH_num(const double* __restrict__ K, int c, int v, int i0,
 // summed, off-diagonal ones twice; the G shifts of an element share its loads and give G
 // independent chains.  c42 v350, 16 shifts: 82.9 ms with one shift a block over the full
 // square.
+// KK: element (ia, jb) at KK[ia * ld + jb - off].
 template <int G>
-__global__ void k_classH_sums(const double* __restrict__ KK, const double* __restrict__ eps,
-                              const double* __restrict__ shifts, int nshift, int c, int v,
-                              int i0, int i1, double* __restrict__ partial) {
+__global__ void k_classH_sums(const double* __restrict__ KK, long ld, long off,
+                              const double* __restrict__ eps, const double* __restrict__ shifts,
+                              int nshift, int c, int v, int i0, int i1,
+                              double* __restrict__ partial) {
   __shared__ double red[32];
   const int k0 = blockIdx.y * G;
-  const long cv = (long)c * v;
   double sh[G], e[G], nr[G], n3[G];
   // smallest |D| with KK != 0, kept as the bit pattern of |D| (non-negative doubles order
   // like their bit patterns, so the minimum runs on the integer units)
@@ -314,7 +315,7 @@ __global__ void k_classH_sums(const double* __restrict__ KK, const double* __res
   for (long ia = (long)i0 * v + blockIdx.x; ia < (long)i1 * v; ia += gridDim.x) {
     const int i = (int)(ia / v), a = (int)(ia % v);
     const double base = eps[c + a] - eps[i];
-    const double* row = KK + ia * cv;
+    const double* row = KK + (ia * ld - off);
     for (int j = i; j < c; ++j) {
       const double bj = base - eps[j];
       const double* rj = row + (long)j * v;
@@ -419,6 +420,34 @@ cudaError_t launch_classH(const double* f, const double* B, const double* Ftil, 
   return cudaGetLastError();
 }
 
+namespace {
+// Shifts per block row of k_classH_sums: the group of three to five that pads nshift least (one
+// shift: one).
+int shift_group(int nshift) {
+  if (nshift <= 1) return 1;
+  int G = 4;
+  for (int g : {5, 3})
+    if ((nshift + g - 1) / g * g < (nshift + G - 1) / G * G) G = g;
+  return G;
+}
+
+void launch_sums(int G, int nblk, const double* KK, long ld, long off, const ClassHWork& w,
+                 int nshift, const Dims& d, int i0, int i1, double* partial, cudaStream_t s) {
+  const dim3 grid(nblk, (nshift + G - 1) / G);
+  // one pass over b per (i, a, j) when v fits a block (no idle tail of lanes)
+  const int threads = d.v <= 512 ? std::max(64, (d.v + 31) / 32 * 32) : 256;
+  auto run = [&](auto kernel) {
+    kernel<<<grid, threads, 0, s>>>(KK, ld, off, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
+                                    partial);
+  };
+  ++launch_counter();
+  if (G == 1) run(k_classH_sums<1>);
+  else if (G == 3) run(k_classH_sums<3>);
+  else if (G == 4) run(k_classH_sums<4>);
+  else run(k_classH_sums<5>);
+}
+}  // namespace
+
 cudaError_t launch_classH_split(const double* f, const double* B, const double* Ftil,
                                 const double* E0, double shift, int scheme, const Dims& d,
                                 ClassHWork& w, int* status, double* ecls, double* ncls,
@@ -466,34 +495,138 @@ cudaError_t launch_classH_split(const double* f, const double* B, const double* 
   ++launch_counter();
   k_classH_num<<<(int)std::min<long>((total + 255) / 256, 152L * 32), 256, 0, s>>>(K, d.c, d.v, i0,
                                                                                   i1, KK);
-  // shifts per block row: the group of three to five that pads nshift least (one shift: one)
-  int G = 1;
-  if (nshift > 1) {
-    G = 4;
-    for (int g : {5, 3})
-      if ((nshift + g - 1) / g * g < (nshift + G - 1) / G * G) G = g;
-  }
-  const int ng = (nshift + G - 1) / G;
+  const int G = shift_group(nshift), ng = (nshift + G - 1) / G;
   const int nblk = (int)std::max<long>(1, std::min<long>(w.nblocks / ng, 152L * 8));
-  // one pass over b per (i, a, j) when v fits a block (no idle tail of lanes)
-  const int hthreads = d.v <= 512 ? std::max(64, (d.v + 31) / 32 * 32) : 256;
-  const dim3 grid(nblk, ng);
-  ++launch_counter();
-  if (G == 1)
-    k_classH_sums<1><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
-                                               w.partial);
-  else if (G == 3)
-    k_classH_sums<3><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
-                                               w.partial);
-  else if (G == 4)
-    k_classH_sums<4><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
-                                               w.partial);
-  else
-    k_classH_sums<5><<<grid, hthreads, 0, s>>>(KK, w.eps, w.shifts, nshift, d.c, d.v, i0, i1,
-                                               w.partial);
+  launch_sums(G, nblk, KK, cv, 0, w, nshift, d, i0, i1, w.partial, s);
   const int ncol = 3 * nshift + 1;
   ++launch_counter();
   k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, (long)nblk * ng, ncol, w.sums);
+  ++launch_counter();
+  k_classH_combine<<<1, 256, 0, s>>>(w.sums, w.W, n, scheme, ecls, ncls, mom, mindenom, status);
+  return cudaGetLastError();
+}
+
+// In place: K_ij^ab -> K_ij^ab (2 K_ij^ab - K_ij^ba) for i in [i0, i0 + ni), j >= i0; element
+// (ia, jb) at K[(ia - i0 v) ld + jb - i0 v].  Both 32 x 32 tiles of a pair (a, b), (b, a) go through
+// shared memory, so that all global accesses run along b (c42 v350: the transposed read of
+// k_classH_num costs 1.27 ms where the bytes take 0.4).  grid (tile pairs ta <= tb, (i, j)).
+__global__ void __launch_bounds__(256)
+k_classH_num_tiles(double* __restrict__ K, long ld, int v, int ni, int nj) {
+  __shared__ double t1[32][33], t2[32][33];
+  const int nt = (v + 31) / 32;
+  int ta = 0, rem = blockIdx.x;
+  while (rem >= nt - ta) { rem -= nt - ta; ++ta; }
+  const int a0 = 32 * ta, b0 = 32 * (ta + rem);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (long ij = blockIdx.y; ij < (long)ni * nj; ij += gridDim.y) {
+    const int i = (int)(ij / nj), j = (int)(ij % nj);
+    if (j < i) continue;                       // the same for the whole block
+    double* base = K + (long)i * v * ld + (long)j * v;
+    for (int r = warp; r < 32; r += 8) {
+      t1[r][lane] = a0 + r < v && b0 + lane < v ? base[(a0 + r) * ld + b0 + lane] : 0.0;
+      t2[r][lane] = b0 + r < v && a0 + lane < v ? base[(b0 + r) * ld + a0 + lane] : 0.0;
+    }
+    __syncthreads();
+    for (int r = warp; r < 32; r += 8) {
+      const double x = t1[r][lane], y = t2[r][lane];
+      if (a0 + r < v && b0 + lane < v) base[(a0 + r) * ld + b0 + lane] = x * (2.0 * x - t2[lane][r]);
+      if (a0 != b0 && b0 + r < v && a0 + lane < v)
+        base[(b0 + r) * ld + a0 + lane] = y * (2.0 * y - t1[lane][r]);
+    }
+    __syncthreads();
+  }
+}
+
+namespace {
+int sliced_rows(const Dims& d, int i, long cap) {   // closed orbitals of the chunk from i on
+  return (int)std::min<long>(d.c - i, cap / ((long)d.v * (d.c - i) * d.v));
+}
+}  // namespace
+
+// Doubles of the K workspace, or 0 where the fused kernel serves: up to 2^26 multiply-adds of
+// the full product it takes less than the dozen launches here (c4 v20 X84: 0.17 ms).  The
+// workspace is one chunk of rows, 128 MB unless a single closed orbital needs more.
+long classH_sliced_work(const Dims& d, int scheme) {
+  const double cv = (double)d.c * d.v, fmas = cv * cv * d.X;
+  if (fmas <= 67108864.0 || d.X > (1 << 17) || cv > 1e9) return 0;
+  return std::min<long>((long)(cv * cv), std::max<long>(1L << 24, (long)(cv * d.v)));
+}
+
+// Rows of the partial sums: a block's each in the fused kernel; the split forms take up to
+// eight blocks a SM and shift group (c8 v61, nine shifts: the fused kernel's 36 rows left 12 blocks a
+// group, 0.27 ms), in at most 64 MB.
+long classH_partial_rows(const Dims& d, int scheme, bool split) {
+  const long kcap = split ? (long)d.c * d.v * d.c * d.v : classH_sliced_work(d, scheme);
+  if (kcap <= 0) return classH_blocks(d);
+  const int nshift = classH_nshift(d, scheme), G = shift_group(nshift);
+  long chunks = 0;
+  for (int i = 0; i < d.c; i += sliced_rows(d, i, kcap)) ++chunks;
+  const long per = chunks * ((nshift + G - 1) / G);
+  const long nblk = std::min({152L * 8, (long)d.c * d.v, (1L << 23) / (per * (3 * nshift + 1))});
+  return std::max(classH_blocks(d), per * std::max(1L, nblk));
+}
+
+cudaError_t classH_sliced_reserve(const Dims& d, OzWork& oz) {
+  const int cv = d.c * d.v;
+  return oz_reserve(oz, oz_slice_bytes(cv, d.X, kOzFp64Slices), cv);
+}
+
+// Plain form at sizes where the FP64 units decide (classH_sliced_work): the products of
+// k_classH as exact BF16 slices on the tensor cores, eight an operand, which is what the FP64
+// kernel's own rounding resolves.  B_cv is sliced once; chunks of closed orbitals i form K for
+// their rows and j >= i in a bounded workspace, the numerators in its place and the sums.
+// c30 v300 X990: 76.3 ms fused, of which the FMAs alone take 69; 6.6 ms here (GEMMs 4.9, sums
+// 1.2, numerators 0.3, slicing 0.15); the energies' error against 64 bits 1.6e-16 (fused
+// 2.3e-16).
+cudaError_t launch_classH_sliced(const double* f, const double* B, const double* Ftil,
+                                 const double* E0, double shift, int scheme, const Dims& d,
+                                 ClassHWork& w, int* status, double* ecls, double* ncls,
+                                 double* mom, double* mindenom, OzWork& oz, double* K, long kcap,
+                                 cudaStream_t s, int i0, int i1) {
+  const int n = d.n, nshift = classH_nshift(d, scheme);
+  if (i1 < 0 || i1 > d.c) i1 = d.c;
+  cudaError_t e;
+  if (i1 <= i0) {
+    if ((e = cudaMemsetAsync(ecls, 0, sizeof(double) * n * n, s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(mom, 0, sizeof(double) * (n * n * n + n * n + n), s)) != cudaSuccess)
+      return e;
+    return cudaMemsetAsync(ncls, 0, sizeof(double) * n, s);
+  }
+  if ((e = launch_eps_cv(f, d, w.eps, s)) != cudaSuccess) return e;
+  if ((e = launch_sym_eig(Ftil, n, w.W, w.omega, 0, status, s)) != cudaSuccess) return e;
+  ++launch_counter();
+  k_classH_shifts<<<1, kMaxShift, 0, s>>>(w.omega, E0, shift, n, scheme, w.shifts);
+  if ((e = launch_pack_block(B, d, SP_C, SP_V, w.Bp, s)) != cudaSuccess) return e;
+  if (w.ev_gemm0) cudaEventRecord(w.ev_gemm0, s);
+  const int cv = d.c * d.v, Kp = oz_kpad(d.X), S = kOzFp64Slices;
+  if ((e = classH_sliced_reserve(d, oz)) != cudaSuccess) return e;
+  const OzView vb{w.Bp, 1, cv, (long)d.X, 0};        // rows (ia), K = P
+  if ((e = oz_split(vb, cv, d.X, Kp, S, oz.sl, oz.sc, s)) != cudaSuccess) return e;
+  const long plane = (long)cv * Kp;
+  int chunks = 0;
+  for (int i = 0; i < d.c; i += sliced_rows(d, i, kcap)) ++chunks;
+  const int G = shift_group(nshift), ng = (nshift + G - 1) / G, ncol = 3 * nshift + 1;
+  const int nblk = (int)std::max<long>(1, std::min<long>(w.nblocks / ((long)ng * chunks), 152L * 8));
+  long used = 0;
+  const int nt = (d.v + 31) / 32;
+  for (int i = i0; i < i1;) {
+    const int ni = std::min(sliced_rows(d, i, kcap), i1 - i), nj = d.c - i;
+    const long r0 = (long)i * d.v;
+    const int M = ni * d.v, N = nj * d.v;
+    const __nv_bfloat16* sl = oz.sl + r0 * Kp;
+    if ((e = oz_gemm(sl, oz.sc + r0, sl, oz.sc + r0, M, N, Kp, S, 1.0, 0.0, K, N, oz.err, s, 1,
+                     nullptr, false, plane, plane)) != cudaSuccess)
+      return e;
+    ++launch_counter();
+    k_classH_num_tiles<<<dim3(nt * (nt + 1) / 2, std::min(ni * nj, 65535)), 256, 0, s>>>(K, N, d.v,
+                                                                                        ni, nj);
+    launch_sums(G, nblk, K, N, r0 * N + r0, w, nshift, d, i, i + ni, w.partial + used * ncol, s);
+    used += (long)nblk * ng;
+    i += ni;
+  }
+  if (w.ev_gemm1) cudaEventRecord(w.ev_gemm1, s);
+  ++launch_counter();
+  k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, used, ncol, w.sums);
   ++launch_counter();
   k_classH_combine<<<1, 256, 0, s>>>(w.sums, w.W, n, scheme, ecls, ncls, mom, mindenom, status);
   return cudaGetLastError();

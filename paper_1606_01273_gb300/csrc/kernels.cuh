@@ -93,6 +93,17 @@ cudaError_t launch_classH_split(const double* f, const double* B, const double* 
                                 ClassHWork& w, int* status, double* ecls, double* ncls,
                                 double* mom, double* mindenom, OzWork& oz, double* pack,
                                 double* K, double* KK, cudaStream_t s, int i0 = 0, int i1 = -1);
+// Class H of the plain form at larger sizes, K from eight slices an operand in chunks of kcap
+// doubles: classH_sliced_work gives kcap (0: launch_classH serves), classH_sliced_reserve the
+// slice storage.
+long classH_sliced_work(const Dims& d, int scheme);
+long classH_partial_rows(const Dims& d, int scheme, bool split);
+cudaError_t classH_sliced_reserve(const Dims& d, OzWork& oz);
+cudaError_t launch_classH_sliced(const double* f, const double* B, const double* Ftil,
+                                 const double* E0, double shift, int scheme, const Dims& d,
+                                 ClassHWork& w, int* status, double* ecls, double* ncls,
+                                 double* mom, double* mindenom, OzWork& oz, double* K, long kcap,
+                                 cudaStream_t s, int i0 = 0, int i1 = -1);
 // oz (optional, on): the DF and Gram products run as split BF16 GEMMs; k_ready: hd.K
 // already holds K[(ia)][(jb)] (formed by the split class-H energy path).
 int classH_densities(const double* B, const Dims& d, const ClassHWork& hw, int scheme,

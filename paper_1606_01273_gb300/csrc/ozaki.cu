@@ -39,6 +39,8 @@ constexpr int kOzThreads = 320;                     // warps: TMA, MMA, eight ep
 constexpr long kOzSpin = 1L << 22;
 constexpr int kOzKs = 16;                           // K per shared-memory stage (one MMA)
 constexpr int kOzStages = 5;                        // stage ring
+constexpr int kOzStages8 = 4;                       // with eight slices (48 KB a stage)
+__host__ __device__ inline int oz_ring(int S) { return S > kOzMaxSlices ? kOzStages8 : kOzStages; }
 constexpr int kOzABox = kOzM * 8 * 2;               // bytes of one slice of an A box (8 K)
 constexpr int kOzBBox = kOzN * 8 * 2;
 __host__ __device__ inline int oz_stage_bytes(int S) { return 2 * S * (kOzABox + kOzBBox); }
@@ -143,7 +145,7 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int stage_bytes = oz_stage_bytes(S);
+  const int stage_bytes = oz_stage_bytes(S), ring = oz_ring(S);
   const uint32_t tcols = 512;
 
   if (warp == 1) {
@@ -198,8 +200,8 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         int m0, n0, z, gbeg, nst;
         tile_of(ti, m0, n0, z, gbeg, nst);
         for (int g = 0; g < nst; ++g, ++G) {
-          const int b = G % kOzStages;
-          if (G >= kOzStages && !bar_wait(&empty[b], (uint32_t)(((G / kOzStages) - 1) & 1))) {
+          const int b = G % ring;
+          if (G >= ring && !bar_wait(&empty[b], (uint32_t)(((G / ring) - 1) & 1))) {
             *abort_v = 1;
             break;
           }
@@ -225,13 +227,13 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         int m0, n0, z, gbeg, nst;
         tile_of(ti, m0, n0, z, gbeg, nst);
         for (int g = 0; g < nst; ++g, ++G) {
-          const int b = G % kOzStages;
+          const int b = G % ring;
           const bool first = (g % spc) == 0;
           if (first && Cc > 0 && !bar_wait(&tempty, (uint32_t)((Cc - 1) & 1))) {
             *abort_v = 1;
             break;
           }
-          if (!bar_wait(&full[b], (uint32_t)((G / kOzStages) & 1))) {
+          if (!bar_wait(&full[b], (uint32_t)((G / ring) & 1))) {
             *abort_v = 1;
             break;
           }
@@ -340,11 +342,11 @@ k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     // drain: copies in flight must land and committed MMAs finish before the CTA leaves
     if (tid == 0) atomicExch(err, 1);
     if (tid == 0)
-      for (int g = max(0, n_issued - kOzStages); g < n_issued; ++g)
-        bar_wait(&full[g % kOzStages], (uint32_t)((g / kOzStages) & 1));
+      for (int g = max(0, n_issued - ring); g < n_issued; ++g)
+        bar_wait(&full[g % ring], (uint32_t)((g / ring) & 1));
     if (tid == 32)
-      for (int g = max(0, n_committed - kOzStages); g < n_committed; ++g)
-        bar_wait(&empty[g % kOzStages], (uint32_t)((g / kOzStages) & 1));
+      for (int g = max(0, n_committed - ring); g < n_committed; ++g)
+        bar_wait(&empty[g % ring], (uint32_t)((g / ring) & 1));
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -415,13 +417,14 @@ __global__ void k_oz_rowmax(OzView v, int R, int K, bool split_k,
   }
 }
 
-// sigma_r = 2^(floor(log2 max|x_r|) + 1) (1 for a zero row).
+// sigma_r = 2^(floor(log2 max|x_r|) + 1) (1 for a zero row, NaN for one with a NaN or an infinity,
+// which every result of that row then is).
 __global__ void k_oz_scale(const unsigned long long* __restrict__ mx, int R,
                            double* __restrict__ scale) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   const double m = __longlong_as_double((long long)mx[r]);
-  scale[r] = m > 0.0 ? ldexp(1.0, ilogb(m) + 1) : 1.0;
+  scale[r] = m == 0.0 ? 1.0 : isfinite(m) ? ldexp(1.0, ilogb(m) + 1) : nan("");
 }
 
 // S slices of x / sigma_r into out[s][r][Kp] (zeros for K <= k < Kp); grid (Kp tiles,
@@ -434,8 +437,10 @@ __global__ void k_oz_split(OzView v, int R, int K, int Kp, int S, bool split_k,
   const long plane = (long)R * Kp;
   for (int r0 = blockIdx.y * kOzTile; r0 < R; r0 += gridDim.y * kOzTile) {
     oz_load_tile(v, R, K, r0, k0, split_k, t);
-    if (threadIdx.x < kOzTile)
-      er[threadIdx.x] = r0 + (int)threadIdx.x < R ? ilogb(scale[r0 + threadIdx.x]) : 0;
+    if (threadIdx.x < kOzTile) {
+      const double sc = r0 + (int)threadIdx.x < R ? scale[r0 + threadIdx.x] : 1.0;
+      er[threadIdx.x] = isfinite(sc) ? ilogb(sc) : 0;
+    }
     __syncthreads();
     for (int q = threadIdx.x; q < kOzTile * kOzTile; q += blockDim.x) {
       const int kk = q % kOzTile, rr = q / kOzTile;
@@ -449,7 +454,7 @@ __global__ void k_oz_split(OzView v, int R, int K, int Kp, int S, bool split_k,
       if (ex != 0) {
         const long long mant = (bits & 0xFFFFFFFFFFFFFLL) | (1LL << 52);
         const int sh = ex - 1023 + 4 - er[rr];
-        if (sh >= 0) X = mant << sh;
+        if (sh >= 0) X = sh <= 3 ? mant << sh : 0;   // more only in a row that is not finite
         else if (sh > -60) X = (mant + (1LL << (-sh - 1))) >> (-sh);
         if (bits < 0) X = -X;
       }
@@ -458,7 +463,7 @@ __global__ void k_oz_split(OzView v, int R, int K, int Kp, int S, bool split_k,
       const long e = (long)r * Kp + k;
       for (int s = 0; s < S; ++s) {
         const int sh = 49 - 7 * s;
-        const long long a = (X + (1LL << (sh - 1))) >> sh;
+        const long long a = sh > 0 ? (X + (1LL << (sh - 1))) >> sh : X;
         X -= a << sh;
         out[(long)s * plane + e] = __float2bfloat16_rn((float)a);
       }
@@ -505,12 +510,14 @@ PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
   return fn;
 }
 
-// 3-D map of slices out[s][r][Kp] (BF16): dims (Kp, R, S), box (8 K, rows, S).
-bool slice_map(CUtensorMap* map, const __nv_bfloat16* X, int R, int Kp, int S, int rows) {
+// 3-D map of slices out[s][r][Kp] (BF16), `plane` elements apart: dims (Kp, R, S), box (8 K,
+// rows, S).
+bool slice_map(CUtensorMap* map, const __nv_bfloat16* X, int R, int Kp, int S, int rows,
+               long plane) {
   auto enc = tmap_encoder();
   if (!enc) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)R, (cuuint64_t)S};
-  const cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)R * Kp * 2};
+  const cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)plane * 2};
   const cuuint32_t box[3] = {8u, (cuuint32_t)rows, (cuuint32_t)S};
   const cuuint32_t es[3] = {1u, 1u, 1u};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<__nv_bfloat16*>(X), dims,
@@ -522,17 +529,20 @@ bool slice_map(CUtensorMap* map, const __nv_bfloat16* X, int R, int Kp, int S, i
 cudaError_t oz_gemm(const __nv_bfloat16* As, const double* sa, const __nv_bfloat16* Bs,
                     const double* sb, int M, int N, int Kp, int S, double alpha, double beta,
                     double* C, long ldc, int* err, cudaStream_t s, int nsplit, double* part,
-                    bool sym) {
+                    bool sym, long pa, long pb) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  if (S < 1 || S > kOzMaxSlices || Kp % kOzKStage != 0) return cudaErrorInvalidValue;
+  if (S < 1 || S > kOzFp64Slices || Kp % kOzKStage != 0) return cudaErrorInvalidValue;
+  if (pa == 0) pa = (long)M * Kp;
+  if (pb == 0) pb = (long)N * Kp;
+  if (pa % 8 != 0 || pb % 8 != 0) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(As) | reinterpret_cast<uintptr_t>(Bs)) & 15)
     return cudaErrorInvalidValue;
   CUtensorMap ma, mb;
-  if (!slice_map(&ma, As, M, Kp, S, kOzM) || !slice_map(&mb, Bs, N, Kp, S, kOzN))
+  if (!slice_map(&ma, As, M, Kp, S, kOzM, pa) || !slice_map(&mb, Bs, N, Kp, S, kOzN, pb))
     return cudaErrorInvalidValue;
-  // the ring of five stages (1 KB alignment slack); the attribute is global to the kernel,
-  // so it is set to the fixed maximum (7 slices)
-  const int smem = kOzStages * oz_stage_bytes(S) + 1024;
+  // the ring of stages (1 KB alignment slack); the attribute is global to the kernel,
+  // so it is set to the fixed maximum (five stages of 7 slices, more than four of 8)
+  const int smem = oz_ring(S) * oz_stage_bytes(S) + 1024;
   const int smem_max = kOzStages * oz_stage_bytes(kOzMaxSlices) + 1024;
   cudaError_t e =
       cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max);
@@ -573,7 +583,6 @@ void oz_release(OzWork& w) {
   w.sl_bytes = w.sc_n = 0;
 }
 
-namespace {
 cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc) {
   cudaError_t e = cudaSuccess;
   if (!w.err) {
@@ -596,7 +605,6 @@ cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc) {
   }
   return cudaSuccess;
 }
-}  // namespace
 
 cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, int M, int N,
                       int K, double alpha, double beta, double* C, long ldc, cudaStream_t s) {

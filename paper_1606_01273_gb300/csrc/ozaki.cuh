@@ -19,7 +19,11 @@
 
 namespace caspt2 {
 
-constexpr int kOzMaxSlices = 7;
+constexpr int kOzMaxSlices = 7;      // of the precision form
+// Slices that hold every operand to 2^-57 of its row's scale, the whole 2^56 fixed-point integer:
+// what is dropped (levels s + t >= 8, at most 2^-55 and typically 2^-58 of sigma_i tau_j a
+// term) is below the rounding of an FP64 dot product of the same terms.
+constexpr int kOzFp64Slices = 8;
 constexpr int kOzKChunk = 256;     // exact FP32 accumulation span
 constexpr int kOzKStage = 32;      // K per shared-memory stage
 
@@ -38,11 +42,12 @@ cudaError_t oz_split(const OzView& v, int R, int K, int Kp, int S, __nv_bfloat16
 // C[i][j] (ldc) = alpha * sum_k A(i,k) B(j,k) + beta * C[i][j] from the slices of A
 // (M x Kp) and B (N x Kp).  err receives a nonzero code if a bounded wait gave up.
 // nsplit > 1 splits K (in exact chunks) over CTAs; part then holds nsplit * M * N doubles.
-// sym: B is A, only the tiles at and right of the diagonal are formed and mirrored.
+// sym: B is A, only the tiles at and right of the diagonal are formed and mirrored.  pa, pb:
+// elements between the slices of A and B where they are rows of larger operands (0: M Kp, N Kp).
 cudaError_t oz_gemm(const __nv_bfloat16* As, const double* sa, const __nv_bfloat16* Bs,
                     const double* sb, int M, int N, int Kp, int S, double alpha, double beta,
                     double* C, long ldc, int* err, cudaStream_t s, int nsplit = 1,
-                    double* part = nullptr, bool sym = false);
+                    double* part = nullptr, bool sym = false, long pa = 0, long pb = 0);
 
 // Device workspace of the split GEMMs, grown on demand (growth synchronises the device)
 // and owned by the caller.  on = false selects the plain FP64 paths.
@@ -58,6 +63,8 @@ struct OzWork {
   size_t part_n = 0;
 };
 void oz_release(OzWork& w);
+// At least `bytes` of slices and nsc scales (and the error flag).
+cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc);
 
 // C (ldc) = alpha * A B^T + beta * C for an M x K view A and an N x K view B (same: B is A,
 // sliced once, half of the symmetric result formed).  C does not overlap A or B.
