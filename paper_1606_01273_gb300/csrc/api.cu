@@ -63,7 +63,6 @@ struct caspt2_ctx {
   SectorWork sw{};
   SectorBatch sb{};
   double *rdm3r = nullptr, *rdm4r = nullptr, *h = nullptr, *fact = nullptr, *eps = nullptr;
-  double* hk = nullptr;               // precision form: core exchange block for h
   double *pack0 = nullptr, *pack1 = nullptr;
   std::map<int, double*> eri_blk;     // canonical space key -> (pq|rt) block
   EriBlocks eri_tab{};
@@ -425,7 +424,6 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       q.srcGcap = std::max<long>(1, srcg_max);
       ALLOC(q.srcX, q.srcXcap); ALLOC(q.srcG, q.srcGcap);
       ALLOC(c->h, nmo * nmo);
-      if (o.precision == CASPT2_BF16X) ALLOC(c->hk, nmo * nmo);
       ALLOC(c->fact, a2);
       ALLOC(c->eps, nmo);
       if (packmax > 0) {
@@ -607,7 +605,7 @@ int solve_impl(caspt2_ctx* c, void* stream) {
   // ---- stage 0: setup (Sec. II.A, II.B)
   CASPT2_CUDA_TRY(cudaEventRecord(c->ev[0], s));
   CASPT2_CUDA_TRY(launch_dsa(c->rdm1, d, c->dact, s));
-  CASPT2_CUDA_TRY(launch_gmat(c->B, c->dact, d, c->gam, c->Y, c->g, s));
+  CASPT2_CUDA_TRY(launch_gmat(c->B, c->dact, d, c->gam, c->Y, c->g, s, &c->oz));
   CASPT2_CUDA_TRY(launch_ecore(c->f, c->g, c->B, d, c->bsum, c->bfro, c->ecore, s));
   CASPT2_CUDA_TRY(launch_fref(c->f, c->rdm1, d, c->fref, s));
   CASPT2_CUDA_TRY(launch_sym_eig(c->fref, n, c->U, c->Etil, o.xms ? 0 : 1, c->status, s));
@@ -647,7 +645,7 @@ int solve_impl(caspt2_ctx* c, void* stream) {
     bool any = false;
     for (int k = 0; k < 7; ++k) any = any || c->cw_on[k];
     if (any) {
-      CASPT2_CUDA_TRY(launch_hcore(c->f, c->g, c->B, c->bsum, d, c->h, s, &c->oz, c->hk));
+      CASPT2_CUDA_TRY(launch_hcore(c->f, c->g, c->B, c->bsum, d, c->h, s, &c->oz));
       CASPT2_CUDA_TRY(launch_active_block(c->f, d, c->fact, s));
       CASPT2_CUDA_TRY(launch_eps_cv(c->f, d, c->eps, s));
       if (c->kmax >= 3)

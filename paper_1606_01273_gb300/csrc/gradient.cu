@@ -257,7 +257,7 @@ int assemble_orbital_derivative(const Dims& d, const double* f, const double* g_
   CASPT2_CUDA_TRY(launch_symmetrize(gf, nmo, 1, s));
   CASPT2_CUDA_TRY(launch_symmetrize(gBh, nmo, d.X, s));
   // h = f - g(d_sa) over all orbital pairs (plain FP64 form)
-  CASPT2_CUDA_TRY(launch_hcore(f, g_act, B, bsum, d, h, s, nullptr, nullptr));
+  CASPT2_CUDA_TRY(launch_hcore(f, g_act, B, bsum, d, h, s));
   CASPT2_CUDA_TRY(dgemm(nmo, nmo, nmo, 2.0, h, nmo, false, gf, nmo, false, 0.0, Y, nmo, s));
   // sum_Q B_Q gBh_Q = B^T gBh with B and gBh read as (X nmo) x nmo matrices (row (Q, q));
   // partial products over chunks of Q (into gw.M, free again) summed in chunk order

@@ -29,12 +29,17 @@ int canonicalize_inputs(double* f, double* B, const Dims& d, double* C, cudaStre
 cudaError_t canon_back(const double* C, const double* M, int nmo, int batch, double* tmp,
                        double* out, cudaStream_t s);
 
+struct OzWork;
 // ---- setup (setup.cu) --------------------------------------------------------
 // d_act = (1/n) sum_N rdm1[N][N]                         (Sec. II.B, d^(0)sa)
 cudaError_t launch_dsa(const double* rdm1, const Dims& d, double* dact, cudaStream_t s);
 // g = g(d_act) over all nmo x nmo (Sec. II.B, g(d) with d nonzero in the active block)
 cudaError_t launch_gmat(const double* B, const double* dact, const Dims& d, double* gam,
-                        double* Y, double* g, cudaStream_t s);
+                        double* Y, double* g, cudaStream_t s, OzWork* oz = nullptr);
+// out = alpha sum_P coef[P] B[P][.] + beta out (+ p - q) over len elements
+cudaError_t launch_coulomb(const double* B, const double* coef, int X, long len, double alpha,
+                           double beta, const double* p, const double* q, double* out,
+                           cudaStream_t s);
 // E_core = <core|H|core>, with h = f - g(d_sa)
 cudaError_t launch_ecore(const double* f, const double* g, const double* B, const Dims& d,
                          double* bsum, double* bfro, double* ecore, cudaStream_t s);
@@ -85,7 +90,6 @@ struct HDensWork {
 };
 // Class-H share of d2 (closed, active, virtual blocks) and GDF of target state P
 // (Sec. II.D), accumulated; needs the W, shifts and eps left by launch_classH.
-struct OzWork;
 // Class H with K[(ia)][(jb)] (cv x cv, in K) formed by the split BF16 tensor-core GEMM
 // and the energy sums taken over the stored matrix (KK: cv x cv work, pack: X c v).
 cudaError_t launch_classH_split(const double* f, const double* B, const double* Ftil,

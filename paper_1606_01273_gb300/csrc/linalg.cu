@@ -261,8 +261,9 @@ cudaError_t dgemm(int M, int N, int K, double alpha, const double* A, int lda, b
 }
 
 cudaError_t dgemm_views(int M, int N, int K, double alpha, const KView& A, const KView& B,
-                        double beta, double* C, long ldc, cudaStream_t s) {
+                        double beta, double* C, long ldc, cudaStream_t s, bool sym) {
   if (M <= 0 || N <= 0) return cudaSuccess;
+  if (sym && (M != N || beta != 0.0)) return cudaErrorInvalidValue;
   const long straight = (long)((M + 7) / 8) * ((N + 31) / 32);
   const long turned = (long)((N + 7) / 8) * ((M + 31) / 32);
   const bool t = turned < straight;
@@ -277,7 +278,8 @@ cudaError_t dgemm_views(int M, int N, int K, double alpha, const KView& A, const
   g.B = b.X; g.bj = b.rs; g.bk = b.cs; g.bkin = (unsigned)b.kin; g.bkout = b.kout;
   g.C = C; g.ci = t ? 1 : ldc; g.cj = t ? ldc : 1;
   g.tn = (g.N + kGT - 1) / kGT;
-  const long tiles = (long)((g.M + kGT - 1) / kGT) * g.tn;
+  g.sym = sym ? 1 : 0;
+  const long tiles = sym ? (long)g.tn * (g.tn + 1) / 2 : (long)((g.M + kGT - 1) / kGT) * g.tn;
   return launch_dgemm(g, tiles, 1, 2.0 * M * N * (double)K, s);
 }
 

@@ -46,8 +46,9 @@ cudaError_t dgemm(int M, int N, int K, double alpha, const double* A, int lda, b
 // C[i][j] (ldc) = alpha * sum_k A(i, k) B(j, k) + beta * C, with general strides and K in runs:
 // A(i, k) = A[i * ars + (k / akin) * akout + (k % akin) * acs], B alike.
 struct KView { const double* X; long rs, cs, kin, kout; };
+// sym: the result is known to be symmetric (M = N, beta = 0), half of its tiles are formed.
 cudaError_t dgemm_views(int M, int N, int K, double alpha, const KView& A, const KView& B,
-                        double beta, double* C, long ldc, cudaStream_t s);
+                        double beta, double* C, long ldc, cudaStream_t s, bool sym = false);
 // Same product when the N x N result is known to be symmetric (A^T A, X^T F X): only the
 // upper-triangle tiles are computed, each written to both triangles.
 cudaError_t dgemm_sym(int N, int K, double alpha, const double* A, int lda, bool ta,
