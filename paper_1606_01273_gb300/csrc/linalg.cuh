@@ -55,7 +55,7 @@ cudaError_t dgemm_sym(int N, int K, double alpha, const double* A, int lda, bool
                       const double* B, int ldb, bool tb, double beta, double* C, int ldc,
                       cudaStream_t s);
 
-// Eigenpairs of a symmetric m x m matrix by Householder tridiagonalisation, bisection,
+// Eigenpairs of a symmetric m x m matrix by Householder tridiagonalisation, eigenvalues,
 // inverse iteration and back-transformation (eig_tridiag.cu).  A is destroyed; w[m]
 // ascending; V[m][m] eigenvectors as columns.  work >= sym_eig_tridiag_work(m) doubles.
 size_t sym_eig_tridiag_work(int m);
