@@ -15,7 +15,8 @@ __host__ __device__ inline double eig_guard(double wmin, double tnorm) {
   return g < wmin ? g : wmin;
 }
 
-// Bracket width at which an eigenvalue is taken (times max(1, ||T||)): half an FP64 rounding,
+// Bracket width at which an eigenvalue is taken (times ||T||, in the large-matrix path times
+// max(1, ||T||)): half an FP64 rounding,
 // so that the search adds nothing to the rounding of T.  The overlap's small eigenvalues
 // normalise the range basis, s^(-1/2): at s = 1e-6 one rounding of ||T|| = 10 is 2e-9 of s.
 constexpr double kEigTol = 1.1e-16;

@@ -42,6 +42,11 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// 2^e, -1022 <= e <= 1023
+__device__ __forceinline__ double exp2i(int e) {
+  return __longlong_as_double((long long)(e + 1023) << 52);
+}
+
 // Householder reduction of the symmetric A (rows of stride ld): d, e, and the reflectors
 // H_k = 1 - tau_k u u^T with u in row k right of the diagonal (not normalised:
 // u = x + sign(x_0) |x| e_0, tau = 1 / (|x| (|x| + |x_0|))).
@@ -135,6 +140,9 @@ __device__ void tridiagonalise(double* A, int ld, int m, const Vecs& q) {
 // Eigenpairs of A (destroyed; stride ld): q.w holds all m eigenvalues ascending, Z [m][nc] the
 // vectors of the last nc, of which the last nk have eigenvalues >= wmin (eig_guard).  scr: 4 m
 // nc doubles and m nc bytes.  Returns nk, or -1 when the matrix holds a NaN or an infinity.
+// T is scaled by a power of two to a norm in [1, 2): the brackets' widths and the ranges of the
+// recurrences are then relative to the norm (a sector of weakly occupied orbitals has a norm of
+// 1e-6 and keeps all its digits), and no rounding changes.
 __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, double* scr,
                          const Vecs& q, double* sh, int& nc) {
   nc = 0;
@@ -150,9 +158,6 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
       ghi = fmax(ghi, q.d[i] + r);
       tn = fmax(tn, fabs(q.d[i]) + r);
       bad = bad || !(fabs(q.d[i]) + r < 1e300);
-      q.e2[i] = q.e[i] * q.e[i];
-      q.df[i] = (float)q.d[i];
-      q.ef[i] = (float)q.e2[i];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -161,17 +166,32 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
       tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, o));
     }
     bad = __any_sync(0xffffffffu, bad);
+    const int ex = tn > 0x1p-1000 ? (int)(abits(tn) >> 52) - 1023 : 0;
+    const double sc = exp2i(-ex);
+    __syncwarp();
+    for (int i = lane; i < m; i += 32) {
+      const double di = q.d[i] * sc, ei = q.e[i] * sc;
+      q.d[i] = di;
+      q.e[i] = ei;
+      q.e2[i] = ei * ei;
+      q.df[i] = (float)di;
+      q.ef[i] = (float)(ei * ei);
+    }
     if (lane == 0) {
-      const double pad = 2.2e-16 * fmax(1.0, tn) * 4.0;
-      sh[0] = glo - pad;
-      sh[1] = ghi + pad;
+      tn *= sc;
+      const double pad = 2.2e-16 * tn * 4.0;
+      sh[0] = glo * sc - pad;
+      sh[1] = ghi * sc + pad;
       sh[2] = tn;
       sh[3] = bad ? 1.0 : 0.0;
+      sh[6] = sc;
+      sh[7] = exp2i(ex);
     }
   }
   __syncthreads();
   if (sh[3] != 0.0) return -1;
-  const double glo = sh[0], ghi = sh[1], tn = sh[2];
+  const double glo = sh[0], ghi = sh[1], tn = sh[2], unscale = sh[7];
+  wmin *= sh[6];
   // single-precision brackets, eight lanes an eigenvalue; then FP64, one lane each
   for (int j0 = 0; j0 < m; j0 += kNT / 8) {
     const int j = j0 + (threadIdx.x >> 3);
@@ -183,7 +203,7 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     }
   }
   __syncthreads();
-  const double tol = kEigTol * fmax(1.0, tn);
+  const double tol = kEigTol * tn;
   for (int j = threadIdx.x; j < m; j += kNT)
     q.w[j] = eigenvalue_f64(q.d, q.e2, m, j, glo, ghi, q.lo[j], q.hi[j], tol,
                              eig_guard(wmin, tn));
@@ -199,7 +219,11 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
   __syncthreads();
   const int nk = (int)sh[4];
   nc = (int)sh[5];
-  if (nk == 0) return 0;
+  if (nk == 0) {
+    for (int j = threadIdx.x; j < m; j += kNT) q.w[j] *= unscale;
+    __syncthreads();
+    return 0;
+  }
   const double* wk = q.w + (m - nc);
   for (int j = threadIdx.x; j < nc; j += kNT)
     inverse_iteration(q.d, q.e, m, wk[j], tn, nc, j, scr, Z);
@@ -257,6 +281,8 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     }
     __syncthreads();
   }
+  for (int j = threadIdx.x; j < m; j += kNT) q.w[j] *= unscale;
+  __syncthreads();
   // back-transformation Z <- H_0 ... H_{m-3} Z: lanes over 32 columns, the block's warps
   // split over column chunks and row groups
   const int nch = (nc + 31) / 32;              // column chunks
