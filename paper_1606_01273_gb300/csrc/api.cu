@@ -605,7 +605,7 @@ int solve_impl(caspt2_ctx* c, void* stream) {
   // ---- stage 0: setup (Sec. II.A, II.B)
   CASPT2_CUDA_TRY(cudaEventRecord(c->ev[0], s));
   CASPT2_CUDA_TRY(launch_dsa(c->rdm1, d, c->dact, s));
-  CASPT2_CUDA_TRY(launch_gmat(c->B, c->dact, d, c->gam, c->Y, c->g, s, &c->oz));
+  CASPT2_CUDA_TRY(launch_gmat(c->B, c->dact, d, c->gam, c->Y, c->g, s));
   CASPT2_CUDA_TRY(launch_ecore(c->f, c->g, c->B, d, c->bsum, c->bfro, c->ecore, s));
   CASPT2_CUDA_TRY(launch_fref(c->f, c->rdm1, d, c->fref, s));
   CASPT2_CUDA_TRY(launch_sym_eig(c->fref, n, c->U, c->Etil, o.xms ? 0 : 1, c->status, s));

@@ -35,7 +35,7 @@ struct OzWork;
 cudaError_t launch_dsa(const double* rdm1, const Dims& d, double* dact, cudaStream_t s);
 // g = g(d_act) over all nmo x nmo (Sec. II.B, g(d) with d nonzero in the active block)
 cudaError_t launch_gmat(const double* B, const double* dact, const Dims& d, double* gam,
-                        double* Y, double* g, cudaStream_t s, OzWork* oz = nullptr);
+                        double* Y, double* g, cudaStream_t s);
 // out = alpha sum_P coef[P] B[P][.] + beta out (+ p - q) over len elements
 cudaError_t launch_coulomb(const double* B, const double* coef, int X, long len, double alpha,
                            double beta, const double* p, const double* q, double* out,

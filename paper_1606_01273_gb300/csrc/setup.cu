@@ -7,7 +7,6 @@
 // coalesced along the fastest index, with fixed-order reductions.
 #include "kernels.cuh"
 #include "linalg.cuh"
-#include "ozaki.cuh"
 
 namespace caspt2 {
 
@@ -100,10 +99,10 @@ cudaError_t launch_coulomb(const double* B, const double* coef, int X, long len,
 }
 
 // g[x][y] = sum_P B[P][x][y] gam[P] - 1/2 sum_P sum_u Y[P][x][u] B[P][c+u][y]: the exchange is one
-// product over (P, u), in FP64 or, where that is large and the tensor cores are in use, from
-// eight slices.  One thread an element took 0.31 ms at c9 a6 v83 and 2.8 ms at c42 a6 v350.
+// FP64 product over (P, u) in both forms, since g enters E_core and H^ref directly.  One thread an
+// element took 0.31 ms at c9 a6 v83 and 2.8 ms at c42 a6 v350.
 cudaError_t launch_gmat(const double* B, const double* dact, const Dims& d, double* gam,
-                        double* Y, double* g, cudaStream_t s, OzWork* oz) {
+                        double* Y, double* g, cudaStream_t s) {
   const int nmo = d.nmo();
   if (d.a == 0) {
     cudaError_t e = cudaMemsetAsync(g, 0, sizeof(double) * nmo * nmo, s);
@@ -115,19 +114,10 @@ cudaError_t launch_gmat(const double* B, const double* dact, const Dims& d, doub
   ++launch_counter();
   k_Yact<<<(int)std::min<long>((ty + 255) / 256, 152 * 16), 256, 0, s>>>(B, dact, d.X, nmo, d.c, d.a, Y);
   const long nn = (long)nmo * nmo, na = (long)nmo * d.a;
-  const int K = d.X * d.a;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (oz && oz->on && K <= (1 << 17)) {
-    const OzView vy{Y, d.a, 1, d.a, na}, vb{B + (long)d.c * nmo, 1, nmo, d.a, nn};
-    const int S = oz->S;
-    oz->S = kOzFp64Slices;
-    e = oz_matmul(*oz, vy, vb, false, nmo, nmo, K, -0.5, 0.0, g, nmo, s);
-    oz->S = S;
-  } else {
-    const KView vy{Y, d.a, 1, d.a, na}, vb{B + (long)d.c * nmo, 1, nmo, d.a, nn};
-    e = dgemm_views(nmo, nmo, K, -0.5, vy, vb, 0.0, g, nmo, s);
-  }
+  const KView vy{Y, d.a, 1, d.a, na}, vb{B + (long)d.c * nmo, 1, nmo, d.a, nn};
+  e = dgemm_views(nmo, nmo, d.X * d.a, -0.5, vy, vb, 0.0, g, nmo, s);
   if (e != cudaSuccess) return e;
   return launch_coulomb(B, gam, d.X, nn, 1.0, 1.0, nullptr, nullptr, g, s);
 }
