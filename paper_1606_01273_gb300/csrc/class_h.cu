@@ -191,7 +191,7 @@ k_classH(const double* __restrict__ Bp, const double* __restrict__ eps,
     double e = 0.0, nr = 0.0, n3 = 0.0;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const double inv = recip(d0[q] + sh);
+      const double inv = 1.0 / (d0[q] + sh);
       const double x = num[q] * inv;
       e += x;
       nr = fma(x, inv, nr);

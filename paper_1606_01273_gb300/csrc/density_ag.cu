@@ -52,13 +52,12 @@ __global__ void k_sector_amp(const double* __restrict__ Vt, const double* __rest
       ee += (C.slot_space[C.ext[k]] == SP_V) ? eps[c + co[k]] : -eps[co[k]];
     const double D = ee + omega[mu] - E0[L] + shift;
     const double* row = Vt + mu * ncolV + t * n;
-    const double inv = recip(D);
-    const double am = -row[L] * inv;
+    const double am = -row[L] / D;
     double acc = 0.0;
     for (int N = 0; N < n; ++N) acc += R[N * n + P] * row[N];
     const double rl = R[L * n + P];
     amp[e] = am;
-    lam[e] = -(rl * acc - 2.0 * shift * rl * rl * am) * inv;
+    lam[e] = -(rl * acc - 2.0 * shift * rl * rl * am) / D;
   }
 }
 

@@ -74,7 +74,7 @@ __global__ void k_h_wt(const double* __restrict__ Kb, const double* __restrict__
     const double D0 = eps[c + a] + eps[c + b] - eps[i] - eps[j];
     double phi = 0.0;
     for (int s = 0; s < ns; ++s) {
-      const double inv = recip(D0 + coef[6 * s]);
+      const double inv = 1.0 / (D0 + coef[6 * s]);
       phi += (coef[6 * s + 1] + coef[6 * s + 2] * inv) * inv;
     }
     const double tk = 2.0 * K - Kx;
@@ -96,7 +96,7 @@ __global__ void k_h_lt(const double* __restrict__ Kb, const double* __restrict__
     const int i = ia / v, a = ia % v, j = jb / v, b = jb % v;
     const double K = Kb[e];
     const double Kx = Kb[((long)i * v + b) * cv + (long)j * v + a];
-    const double inv = recip(eps[c + a] + eps[c + b] - eps[i] - eps[j] + sig);
+    const double inv = 1.0 / (eps[c + a] + eps[c + b] - eps[i] - eps[j] + sig);
     Lb[e] = -2.0 * (gam + del * inv) * K * inv;
     Tb[e] = -wt * (2.0 * K - Kx) * inv;
   }
@@ -119,7 +119,7 @@ __global__ void k_h_ov(const double* __restrict__ KK, const double* __restrict__
     const long ia = e / cv, jb = e % cv;
     const int i = ia / v, a = ia % v, j = jb / v, b = jb % v;
     const double D0 = eps[c + a] + eps[c + b] - eps[i] - eps[j];
-    const double i1 = recip(D0 + s1), i2 = recip(D0 + s2);
+    const double i1 = 1.0 / (D0 + s1), i2 = 1.0 / (D0 + s2);
     const double x = KK[e] * i1 * i2;
     sa += x;
     sb += x * i1;
@@ -160,7 +160,7 @@ __global__ void k_h_ov_reg(const double* __restrict__ KK, const double* __restri
     const double kk = KK[e];
     double inv[NM];
 #pragma unroll
-    for (int q = 0; q < NM; ++q) inv[q] = q < n ? recip(D0 + sig[q]) : 0.0;
+    for (int q = 0; q < NM; ++q) inv[q] = q < n ? 1.0 / (D0 + sig[q]) : 0.0;
 #pragma unroll
     for (int p = 0; p < NM; ++p) {
       const double x1 = kk * inv[p];

@@ -411,17 +411,13 @@ k_tridiag_smem(const double* __restrict__ A, int m, double* __restrict__ vbuf,
     }
     __syncthreads();
     if (next && warp == 0) {
-      // beta = -sign(alpha) |x|, tau = 1 + |alpha| / |x|, v = x / (alpha - beta) with v_0 = 1;
-      // |x| and 1 / |x| from the hardware's approximate reciprocal root y by the binomial
-      // series (1 - z)^(-1/2) = 1 + z/2 + 3 z^2/8, z = 1 - |x|^2 y^2 below 2^-19
+      // beta = -sign(alpha) |x|, tau = 1 + |alpha| / |x|, v = x / (alpha - beta) with v_0 = 1
       q = group_sum(red2[lane & (nwarp - 1)], nwarp);
       const double al = r[k2], sig = fma(al, al, q);
       double beta = al, tn = 0.0, scale = 0.0;
       if (q != 0.0 && !(sig < 1e-280)) {
-        double y;
-        asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(sig));
-        const double s0 = sig * y, z = fma(-s0, y, 1.0), c = z * fma(0.375, z, 0.5);
-        const double nr = fma(s0, c, s0), ir = fma(y, c, y);
+        double nr, ir;
+        root_and_recip(sig, nr, ir);
         beta = -copysign(nr, al);
         tn = fma(fabs(al), ir, 1.0);
         scale = copysign(recip(fabs(al) + nr), al);

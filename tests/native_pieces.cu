@@ -10,6 +10,11 @@ __global__ void k_recip(const double* x, long n, double* y) {
     y[i] = caspt2::recip(x[i]);
 }
 
+__global__ void k_root(const double* x, long n, double* r, double* ir) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+    caspt2::root_and_recip(x[i], r[i], ir[i]);
+}
+
 struct Dev {
   double* p = nullptr;
   explicit Dev(size_t n) { if (cudaMalloc(&p, (n ? n : 1) * sizeof(double)) != cudaSuccess) p = nullptr; }
@@ -27,6 +32,17 @@ int np_recip(const double* x, long n, double* y) {
   k_recip<<<152, 256>>>(dx.p, n, dy.p);
   CASPT2_CUDA_TRY(cudaGetLastError());
   CASPT2_CUDA_TRY(cudaMemcpy(y, dy.p, n * sizeof(double), cudaMemcpyDeviceToHost));
+  return CASPT2_OK;
+}
+
+int np_root(const double* x, long n, double* r, double* ir) {
+  Dev dx(n), dr(n), di(n);
+  if (!dx.p || !dr.p || !di.p) return CASPT2_ENOMEM;
+  CASPT2_CUDA_TRY(cudaMemcpy(dx.p, x, n * sizeof(double), cudaMemcpyHostToDevice));
+  k_root<<<152, 256>>>(dx.p, n, dr.p, di.p);
+  CASPT2_CUDA_TRY(cudaGetLastError());
+  CASPT2_CUDA_TRY(cudaMemcpy(r, dr.p, n * sizeof(double), cudaMemcpyDeviceToHost));
+  CASPT2_CUDA_TRY(cudaMemcpy(ir, di.p, n * sizeof(double), cudaMemcpyDeviceToHost));
   return CASPT2_OK;
 }
 

@@ -1,5 +1,6 @@
 """Single pieces of the library on the GPU, called directly (tests/native_pieces.cu): the symmetric
-eigensolver on either side of its border (96 rows)."""
+eigensolver on either side of its border (96 rows), and the reciprocal and the root that stand in
+for a division and a square root."""
 import ctypes as C
 import os
 import subprocess
@@ -80,3 +81,31 @@ def test_small_matrix_scaled_by_a_power_of_two(native, m, power):
     assert a[0] == b[0] == 0
     assert np.array_equal(a[1] * f, b[1])
     assert np.array_equal(a[2], b[2])
+
+
+def _arguments():
+    """Mantissas over [1, 4) with every edge, exponents over the range of a denominator or norm."""
+    rng = np.random.default_rng(3)
+    x = rng.uniform(1.0, 4.0, 1 << 20)
+    x[:3] = 1.0, np.nextafter(2.0, 0.0), np.nextafter(4.0, 0.0)
+    return np.concatenate([x * 2.0 ** e for e in (-300, -20, -1, 0, 1, 10, 300)])
+
+
+def test_reciprocal(native):
+    """0.5 units for the last rounding and 2^-60 relative (below 2^-7 units) for the series."""
+    x = _arguments()
+    x = np.concatenate([x, -x])
+    y = np.zeros_like(x)
+    assert native.np_recip(_p(x), C.c_long(x.size), _p(y)) == 0
+    exact = 1 / x.astype(np.longdouble)
+    assert float((np.abs(y - exact) / np.spacing(np.abs(y))).max()) <= 0.51
+
+
+def test_root_and_reciprocal_root(native):
+    """Relative to 2^-53: 1 for the last rounding, 1/2 for the product's, 2^-5 for the series."""
+    x = _arguments()
+    r, ir = np.zeros_like(x), np.zeros_like(x)
+    assert native.np_root(_p(x), C.c_long(x.size), _p(r), _p(ir)) == 0
+    exact = np.sqrt(x.astype(np.longdouble))
+    for got, ref in ((r, exact), (ir, 1 / exact)):
+        assert float((np.abs(got - ref) / ref).max()) <= 1.6 * 2.0 ** -53
