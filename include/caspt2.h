@@ -49,7 +49,8 @@ extern "C" {
 #define CASPT2_MSMR          0
 #define CASPT2_SSSR          1
 /* precision forms */
-#define CASPT2_FP64          0   /* FP64 (large class-H products: 8 exact slices, as accurate) */
+#define CASPT2_FP64          0   /* FP64; the class-H sums of larger sizes from 8 BF16 slices   */
+                                 /* where the data bound their error by that of FP64 products */
 #define CASPT2_BF16X         1   /* exact BF16 splitting on the tcgen05 tensor cores: the DF  */
                                  /* integral contractions, the class-H pair integrals and the */
                                  /* density Gram products run as S-slice split GEMMs (see    */

@@ -286,8 +286,10 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
   if (st == CASPT2_OK && o.precision == CASPT2_FP64 && (o.class_mask >> CASPT2_CLASS_H & 1u)) {
     // without the memory for it the fused kernel serves
     c->hslcap = classH_sliced_work(d, o.scheme);
-    if (c->hslcap > 0 && (c->alloc(&c->hsl, (size_t)c->hslcap) != CASPT2_OK ||
-                          classH_sliced_reserve(d, c->oz) != cudaSuccess)) {
+    if (c->hslcap > 0 &&
+        (c->alloc(&c->hsl, (size_t)c->hslcap) != CASPT2_OK ||
+         c->alloc(&c->hw.guard, classH_guard_size(d, o.scheme)) != CASPT2_OK ||
+         classH_sliced_reserve(d, c->oz) != cudaSuccess)) {
       oz_release(c->oz);
       cudaGetLastError();
       c->hslcap = 0;

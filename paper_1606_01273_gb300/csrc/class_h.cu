@@ -27,9 +27,10 @@ constexpr int kHK = 16;   // DF-index chunk
 constexpr int kHThreads = 256;
 constexpr int kMaxShift = kMaxStates * kMaxStates;
 
-// Bp[i][P][a] = B[P][i][vo + a]
+// Bp[i][P][a] = B[P][i][vo + a]; go: nothing is done where it points to zero
 __global__ void k_pack_cv(const double* __restrict__ B, int c, int v, int X, int nmo, int vo,
-                          double* __restrict__ Bp) {
+                          double* __restrict__ Bp, const int* __restrict__ go) {
+  if (go && *go == 0) return;
   long total = (long)c * X * v;
   for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total;
        idx += (long)gridDim.x * blockDim.x) {
@@ -64,11 +65,12 @@ __global__ void k_classH_shifts(const double* __restrict__ omega, const double* 
 // so each thread holds both K_ij^ab and K_ij^ba for its elements and the K_ij block
 // is computed exactly once.  On a diagonal tile (ta == tb) K_ij^ba is read from the
 // transposed tile staged in shared memory.  Block (j, i) equals block (i, j) with a
-// and b swapped, so i < j carries weight 2; for i == j, K_ii^ba = K_ii^ab.
+// and b swapped, so i < j carries weight 2; for i == j, K_ii^ba = K_ii^ab.  go: as in k_pack_cv.
 __global__ void __launch_bounds__(kHThreads)
 k_classH(const double* __restrict__ Bp, const double* __restrict__ eps,
          const double* __restrict__ shifts, int nshift, int c, int v, int X, int ntile,
-         int pair0, double* __restrict__ partial) {
+         int pair0, double* __restrict__ partial, const int* __restrict__ go) {
+  if (go && *go == 0) return;
   __shared__ double sbuf[4 * kHK * kHT];   // operand tiles; reused for the diagonal transpose
   __shared__ double sEa[kHT], sEb[kHT];
   __shared__ double sShift[kMaxShift];
@@ -209,10 +211,13 @@ k_classH(const double* __restrict__ Bp, const double* __restrict__ eps,
   if (threadIdx.x == 0) out[3 * nshift] = dmin;
 }
 
-// sums[col] = fixed-order reduction of partial[.][col]; the last column is a min.
+// sums[col] = fixed-order reduction of partial[.][col]; the last column is a min.  go: where it
+// points to a nonzero, nblocks_go rows.
 __global__ void k_reduce_cols(const double* __restrict__ partial, long nblocks, int ncol,
-                              double* __restrict__ sums) {
+                              double* __restrict__ sums, const int* __restrict__ go = nullptr,
+                              long nblocks_go = 0) {
   __shared__ double red[32];
+  if (go && *go != 0) nblocks = nblocks_go;
   const int col = blockIdx.x;
   const bool is_min = (col == ncol - 1);
   double acc = is_min ? 1e300 : 0.0;
@@ -372,6 +377,30 @@ long classH_blocks(const Dims& d) {
 
 int classH_nshift(const Dims& d, int scheme) { return scheme == CASPT2_SSSR ? 1 : d.n * d.n; }
 
+namespace {
+// The pair sums of closed orbitals [i0, i1) by the fused kernel into the first `rows` rows of
+// w.partial (go: only where it points to a nonzero).
+cudaError_t launch_fused(const double* B, const Dims& d, int nshift, ClassHWork& w, int i0, int i1,
+                         const int* go, long& rows, cudaStream_t s) {
+  const int ntile = (d.v + kHT - 1) / kHT;
+  // pairs (i <= j) with i in [i0, i1): a contiguous run of the row-major pair order
+  auto start = [&](long i) { return i * d.c - i * (i - 1) / 2; };
+  const long pair0 = start(i0), npair = start(i1) - start(i0);
+  rows = npair * ((long)ntile * (ntile + 1) / 2);
+  if (rows == 0) return cudaSuccess;
+  const long tp = (long)d.c * d.X * d.v;
+  ++launch_counter();
+  k_pack_cv<<<(int)std::min<long>((tp + 255) / 256, 152 * 32), 256, 0, s>>>(
+      B, d.c, d.v, d.X, d.nmo(), d.c + d.a, w.Bp, go);
+  if (w.ev_gemm0 && !go) cudaEventRecord(w.ev_gemm0, s);
+  ++launch_counter();
+  k_classH<<<(unsigned)rows, kHThreads, 0, s>>>(w.Bp, w.eps, w.shifts, nshift, d.c, d.v, d.X,
+                                               ntile, (int)pair0, w.partial, go);
+  if (w.ev_gemm1 && !go) cudaEventRecord(w.ev_gemm1, s);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_classH(const double* f, const double* B, const double* Ftil, const double* E0,
                           double shift, int scheme, const Dims& d, ClassHWork& w, int* status,
                           double* ecls, double* ncls, double* mom, double* mindenom,
@@ -386,20 +415,13 @@ cudaError_t launch_classH(const double* f, const double* B, const double* Ftil, 
   }
   ++launch_counter();
   k_eps_cv<<<(d.c + d.v + 127) / 128, 128, 0, s>>>(f, nmo, d.c, d.a, d.v, w.eps);
-  long tp = (long)d.c * d.X * d.v;
-  ++launch_counter();
-  k_pack_cv<<<(int)std::min<long>((tp + 255) / 256, 152 * 32), 256, 0, s>>>(
-      B, d.c, d.v, d.X, nmo, d.c + d.a, w.Bp);
   e = launch_sym_eig(Ftil, n, w.W, w.omega, 0, status, s);
   if (e != cudaSuccess) return e;
   ++launch_counter();
   k_classH_shifts<<<1, kMaxShift, 0, s>>>(w.omega, E0, shift, n, scheme, w.shifts);
-  const int ntile = (d.v + kHT - 1) / kHT;
   if (i1 < 0 || i1 > d.c) i1 = d.c;
-  // pairs (i <= j) with i in [i0, i1): a contiguous run of the row-major pair order
-  auto start = [&](long i) { return i * d.c - i * (i - 1) / 2; };
-  const long pair0 = start(i0), npair = start(i1) - start(i0);
-  const long nb = npair * ((long)ntile * (ntile + 1) / 2);
+  long nb = 0;
+  if ((e = launch_fused(B, d, nshift, w, i0, i1, nullptr, nb, s)) != cudaSuccess) return e;
   if (nb == 0) {
     e = cudaMemsetAsync(ecls, 0, sizeof(double) * n * n, s);
     if (e != cudaSuccess) return e;
@@ -407,11 +429,6 @@ cudaError_t launch_classH(const double* f, const double* B, const double* Ftil, 
     if (e != cudaSuccess) return e;
     return cudaMemsetAsync(ncls, 0, sizeof(double) * n, s);
   }
-  if (w.ev_gemm0) cudaEventRecord(w.ev_gemm0, s);
-  ++launch_counter();
-  k_classH<<<(unsigned)nb, kHThreads, 0, s>>>(w.Bp, w.eps, w.shifts, nshift, d.c, d.v, d.X, ntile,
-                                             (int)pair0, w.partial);
-  if (w.ev_gemm1) cudaEventRecord(w.ev_gemm1, s);
   const int ncol = 3 * nshift + 1;
   ++launch_counter();
   k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, nb, ncol, w.sums);
@@ -537,9 +554,135 @@ k_classH_num_tiles(double* __restrict__ K, long ld, int v, int ni, int nj) {
   }
 }
 
+// What the slices may cost, checked on the data of every solve.  An element of K from eight
+// slices is off by up to 1.13 2^-55 X s_ia s_jb (kOzFp64Slices; s: row scales), whatever its size, one
+// from FP64 fused multiply-adds by up to 2^-53 X sum_P |B_P,ia B_P,jb|, which is at least
+// 2^-53 X |K|.  To first order a returned sum O = sum_ijab w K (2K - K'), w = |D|^-p, moves by
+// sum w |K| (4 s_ia s_jb + 2 s_ib s_ja) times the element's error, so slicing costs O no more than
+// FP64 products may where
+//   g = 0.29 |K| (4 s_ia s_jb + 2 s_ib s_ja) + c2 (s_ia s_jb)^2 - 4 K^2
+// (c2 = 1.3 2^-55 X: the second order) has sum w g <= 0 for every shift and p = 1, 2, 3.  It holds by
+// a factor of 4 to 40 for factors of evenly sized elements, by 2 to 7 for local orbitals, and by 1.2
+// for elements that fall by e^20 over P, and fails where the pairs that matter have their large
+// elements at different P (rows graded in opposite directions and a range of closed orbitals whose
+// own pairs are small): those solves take the fused kernel.
+// FP32 throughout (the units are idle and the sum's sign is far from its rounding): s as multiples
+// of the largest among the rows i, and among the rows j, of the call; K from the bits of its upper
+// word.  One pass over K.
+__global__ void __launch_bounds__(1024)
+k_guard_scale(const double* __restrict__ sc, const double* __restrict__ eps, int r0, int r1, int cv,
+              int ne, float* __restrict__ sgi, float* __restrict__ sgj, float* __restrict__ ef,
+              int* __restrict__ es) {
+  __shared__ int red[2][32];
+  // largest exponent fields (the scales are powers of two, 0 or NaN) over [r0, r1) and [r0, cv)
+  int mi = 1, mj = 1;
+  for (int r = r0 + threadIdx.x; r < cv; r += blockDim.x) {
+    const int b = __double2hiint(sc[r]) >> 20;
+    if (b >= 2047) continue;
+    mj = max(mj, b);
+    if (r < r1) mi = max(mi, b);
+  }
+  mi = __reduce_max_sync(0xffffffffu, mi);
+  mj = __reduce_max_sync(0xffffffffu, mj);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = mi;
+    red[1][threadIdx.x >> 5] = mj;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    mi = __reduce_max_sync(0xffffffffu, red[0][threadIdx.x]);
+    mj = __reduce_max_sync(0xffffffffu, red[1][threadIdx.x]);
+    if (threadIdx.x == 0) {
+      red[0][0] = mi;
+      red[1][0] = mj;
+      *es = mi + mj - 2046;
+    }
+  }
+  __syncthreads();
+  mi = red[0][0];
+  mj = red[1][0];
+  for (int r = threadIdx.x; r < cv; r += blockDim.x) {
+    const int b = __double2hiint(sc[r]) >> 20;
+    sgi[r] = b == 0 ? 0.f : b == 2047 ? nanf("") : exp2f((float)(b - mi));
+    sgj[r] = b == 0 ? 0.f : b == 2047 ? nanf("") : exp2f((float)(b - mj));
+  }
+  for (int k = threadIdx.x; k < ne; k += blockDim.x) ef[k] = (float)eps[k];
+}
+
+// Grid as k_classH_sums; out[((block) ng + group) 3G + 3 g + p - 1].
+template <int G>
+__global__ void k_classH_guard(const double* __restrict__ K, long ld, long off,
+                               const float* __restrict__ sgi, const float* __restrict__ sgj,
+                               const float* __restrict__ ef, const int* __restrict__ es,
+                               const double* __restrict__ shifts, int nshift, int c, int v, int i0, int i1, float c2,
+                               double* __restrict__ out) {
+  __shared__ double red[32];
+  const int k0 = blockIdx.y * G, e2 = *es;
+  float sh[G], a1[G], a2[G], a3[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    sh[g] = (float)shifts[min(k0 + g, nshift - 1)];
+    a1[g] = a2[g] = a3[g] = 0.f;
+  }
+  for (long ia = (long)i0 * v + blockIdx.x; ia < (long)i1 * v; ia += gridDim.x) {
+    const int i = (int)(ia / v), a = (int)(ia % v);
+    const float base = ef[c + a] - ef[i], sia = sgi[ia];
+    const double* row = K + (ia * ld - off);
+    for (int j = i; j < c; ++j) {
+      const float bj = base - ef[j], sja = sgj[(long)j * v + a];
+      const double* rj = row + (long)j * v;
+      for (int b = (j == i ? a : 0) + threadIdx.x; b < v; b += blockDim.x) {
+        // |K| / (s_max s_max') from the upper word: exponent field moved, 20 bits of the significand
+        const unsigned hi = (unsigned)__double2hiint(rj[b]) & 0x7FFFFFFFu;
+        const int ex = (int)(hi >> 20);
+        const int fx = ex == 2047 ? 255 : max(0, min(254, ex - 1023 - e2 + 127));
+        const float k = fx == 0 || ex == 0 ? 0.f
+                        : __uint_as_float((unsigned)fx << 23 | (hi & 0xFFFFFu) << 3 | (ex == 2047));
+        const float s1 = sia * sgj[(long)j * v + b], s2 = sgi[(long)i * v + b] * sja;
+        float q = fmaf(k, 0.29f * fmaf(4.f, s1, 2.f * s2), fmaf(c2 * s1, s1, -4.f * k * k));
+        if (j != i || b != a) q += q;
+        const float D0 = bj + ef[c + b];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const float w = __fdividef(1.f, fabsf(D0 + sh[g])), x = q * w, y = x * w;
+          a1[g] += x;
+          a2[g] += y;
+          a3[g] = fmaf(y, w, a3[g]);
+        }
+      }
+    }
+  }
+  double* o = out + ((long)blockIdx.x * gridDim.y + blockIdx.y) * (3 * G);
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const double t1 = block_sum((double)a1[g], red), t2 = block_sum((double)a2[g], red),
+                 t3 = block_sum((double)a3[g], red);
+    if (threadIdx.x == 0) {
+      o[3 * g] = t1;
+      o[3 * g + 1] = t2;
+      o[3 * g + 2] = t3;
+    }
+  }
+}
+
+// *go = 1 where a column's sum over the rows is above zero or not a number; a block a column.
+__global__ void k_guard_decide(const double* __restrict__ part, long rows, int ncol,
+                               int* __restrict__ go) {
+  __shared__ double red[32];
+  double s = 0.0;
+  for (long r = threadIdx.x; r < rows; r += blockDim.x) s += part[r * ncol + blockIdx.x];
+  s = block_sum(s, red);
+  if (threadIdx.x == 0 && !(s <= 0.0)) *go = 1;
+}
+
 namespace {
 int sliced_rows(const Dims& d, int i, long cap) {   // closed orbitals of the chunk from i on
   return (int)std::min<long>(d.c - i, cap / ((long)d.v * (d.c - i) * d.v));
+}
+int sliced_chunks(const Dims& d, long kcap) {
+  int n = 0;
+  for (int i = 0; i < d.c; i += sliced_rows(d, i, kcap)) ++n;
+  return n;
 }
 }  // namespace
 
@@ -559,11 +702,41 @@ long classH_partial_rows(const Dims& d, int scheme, bool split) {
   const long kcap = split ? (long)d.c * d.v * d.c * d.v : classH_sliced_work(d, scheme);
   if (kcap <= 0) return classH_blocks(d);
   const int nshift = classH_nshift(d, scheme), G = shift_group(nshift);
-  long chunks = 0;
-  for (int i = 0; i < d.c; i += sliced_rows(d, i, kcap)) ++chunks;
+  const long chunks = sliced_chunks(d, kcap);
   const long per = chunks * ((nshift + G - 1) / G);
   const long nblk = std::min({152L * 8, (long)d.c * d.v, (1L << 23) / (per * (3 * nshift + 1))});
   return std::max(classH_blocks(d), per * std::max(1L, nblk));
+}
+
+namespace {
+constexpr int kGuardBlocks = 152 * 4;                // of a chunk and shift group
+
+// The guard's arrays in w.guard: partial sums, then row scales and orbital energies in FP32, the
+// scales' exponent and the decision.
+struct GuardArrays {
+  double* part;
+  float *sgi, *sgj, *ef;
+  int *es, *go;
+};
+size_t guard_part(const Dims& d, int scheme) {
+  const int nshift = classH_nshift(d, scheme), G = shift_group(nshift);
+  return (size_t)sliced_chunks(d, classH_sliced_work(d, scheme)) * kGuardBlocks *
+         ((nshift + G - 1) / G) * 3 * G;
+}
+GuardArrays guard_arrays(const Dims& d, int scheme, double* g) {
+  GuardArrays a;
+  a.part = g;
+  a.sgi = reinterpret_cast<float*>(g + guard_part(d, scheme));
+  a.sgj = a.sgi + (size_t)d.c * d.v;
+  a.ef = a.sgj + (size_t)d.c * d.v;
+  a.es = reinterpret_cast<int*>(a.ef + d.c + d.v);
+  a.go = a.es + 1;
+  return a;
+}
+}  // namespace
+
+size_t classH_guard_size(const Dims& d, int scheme) {
+  return guard_part(d, scheme) + (2 * (size_t)d.c * d.v + d.c + d.v + 2 + 1) / 2;
 }
 
 cudaError_t classH_sliced_reserve(const Dims& d, OzWork& oz) {
@@ -571,13 +744,33 @@ cudaError_t classH_sliced_reserve(const Dims& d, OzWork& oz) {
   return oz_reserve(oz, oz_slice_bytes(cv, d.X, kOzFp64Slices), cv);
 }
 
+namespace {
+void launch_guard(int G, const double* K, long ld, long off, const ClassHWork& w,
+                  const GuardArrays& ga, int nshift, const Dims& d, int i0, int i1, float c2,
+                  long at, cudaStream_t s) {
+  const dim3 grid(kGuardBlocks, (nshift + G - 1) / G);
+  const int threads = d.v <= 512 ? std::max(64, (d.v + 31) / 32 * 32) : 256;
+  auto run = [&](auto kernel) {
+    kernel<<<grid, threads, 0, s>>>(K, ld, off, ga.sgi, ga.sgj, ga.ef, ga.es, w.shifts, nshift,
+                                    d.c, d.v, i0, i1, c2, ga.part + at);
+  };
+  ++launch_counter();
+  if (G == 1) run(k_classH_guard<1>);
+  else if (G == 3) run(k_classH_guard<3>);
+  else if (G == 4) run(k_classH_guard<4>);
+  else run(k_classH_guard<5>);
+}
+}  // namespace
+
 // Plain form at sizes where the FP64 units decide (classH_sliced_work): the products of
-// k_classH as exact BF16 slices on the tensor cores, eight an operand, which is what the FP64
-// kernel's own rounding resolves.  B_cv is sliced once; chunks of closed orbitals i form K for
-// their rows and j >= i in a bounded workspace, the numerators in its place and the sums.
-// c30 v300 X990: 76.3 ms fused, of which the FMAs alone take 69; 6.6 ms here (GEMMs 4.9, sums
-// 1.2, numerators 0.3, slicing 0.15); the energies' error against 64 bits 1.6e-16 (fused
-// 2.3e-16).
+// k_classH as exact BF16 slices on the tensor cores, eight an operand.  B_cv is sliced once; chunks
+// of closed orbitals i form K for their rows and j >= i in a bounded workspace, the numerators in
+// its place and the sums.  Where k_guard_decide finds that the slices may cost a returned sum
+// more than FP64 products do, the fused kernel forms the sums instead (its launches return at once
+// otherwise, so the host need not wait for the decision).
+// c30 v300 X990, a pass with inputs: 77.7 ms fused (the FMAs alone take 69), 7.9 here: GEMMs 4.9,
+// sums 1.2, numerators 0.3, guard 0.25, slicing 0.15; the energies' error against 64 bits
+// 2.7e-16.
 cudaError_t launch_classH_sliced(const double* f, const double* B, const double* Ftil,
                                  const double* E0, double shift, int scheme, const Dims& d,
                                  ClassHWork& w, int* status, double* ecls, double* ncls,
@@ -603,11 +796,16 @@ cudaError_t launch_classH_sliced(const double* f, const double* B, const double*
   const OzView vb{w.Bp, 1, cv, (long)d.X, 0};        // rows (ia), K = P
   if ((e = oz_split(vb, cv, d.X, Kp, S, oz.sl, oz.sc, s)) != cudaSuccess) return e;
   const long plane = (long)cv * Kp;
-  int chunks = 0;
-  for (int i = 0; i < d.c; i += sliced_rows(d, i, kcap)) ++chunks;
+  const int chunks = sliced_chunks(d, kcap);
+  const GuardArrays ga = guard_arrays(d, scheme, w.guard);
+  if ((e = cudaMemsetAsync(ga.go, 0, sizeof(int), s)) != cudaSuccess) return e;
+  ++launch_counter();
+  k_guard_scale<<<1, 1024, 0, s>>>(oz.sc, w.eps, i0 * d.v, i1 * d.v, cv, d.c + d.v, ga.sgi, ga.sgj,
+                                   ga.ef, ga.es);
+  const float c2 = (float)(1.3 * 0x1p-55 * d.X);
   const int G = shift_group(nshift), ng = (nshift + G - 1) / G, ncol = 3 * nshift + 1;
   const int nblk = (int)std::max<long>(1, std::min<long>(w.nblocks / ((long)ng * chunks), 152L * 8));
-  long used = 0;
+  long used = 0, gused = 0;
   const int nt = (d.v + 31) / 32;
   for (int i = i0; i < i1;) {
     const int ni = std::min(sliced_rows(d, i, kcap), i1 - i), nj = d.c - i;
@@ -617,6 +815,8 @@ cudaError_t launch_classH_sliced(const double* f, const double* B, const double*
     if ((e = oz_gemm(sl, oz.sc + r0, sl, oz.sc + r0, M, N, Kp, S, 1.0, 0.0, K, N, oz.err, s, 1,
                      nullptr, false, plane, plane)) != cudaSuccess)
       return e;
+    launch_guard(G, K, N, r0 * N + r0, w, ga, nshift, d, i, i + ni, c2, gused * ng * 3 * G, s);
+    gused += kGuardBlocks;
     ++launch_counter();
     k_classH_num_tiles<<<dim3(nt * (nt + 1) / 2, std::min(ni * nj, 65535)), 256, 0, s>>>(K, N, d.v,
                                                                                         ni, nj);
@@ -624,9 +824,13 @@ cudaError_t launch_classH_sliced(const double* f, const double* B, const double*
     used += (long)nblk * ng;
     i += ni;
   }
+  ++launch_counter();
+  k_guard_decide<<<ng * 3 * G, 256, 0, s>>>(ga.part, gused, ng * 3 * G, ga.go);
+  long fused = 0;
+  if ((e = launch_fused(B, d, nshift, w, i0, i1, ga.go, fused, s)) != cudaSuccess) return e;
   if (w.ev_gemm1) cudaEventRecord(w.ev_gemm1, s);
   ++launch_counter();
-  k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, used, ncol, w.sums);
+  k_reduce_cols<<<ncol, 256, 0, s>>>(w.partial, used, ncol, w.sums, ga.go, fused);
   ++launch_counter();
   k_classH_combine<<<1, 256, 0, s>>>(w.sums, w.W, n, scheme, ecls, ncls, mom, mindenom, status);
   return cudaGetLastError();

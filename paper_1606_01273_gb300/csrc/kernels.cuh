@@ -77,6 +77,8 @@ struct ClassHWork {
   double* partial;   // [nblocks][3*nshift + 1]
   double* sums;      // [3*nshift + 1]
   long    nblocks;
+  // launch_classH_sliced: classH_guard_size doubles (its error bound); null without it
+  double* guard = nullptr;
   cudaEvent_t ev_gemm0 = nullptr, ev_gemm1 = nullptr;  // optional: bracket the GEMM kernel
 };
 long classH_blocks(const Dims& d);
@@ -103,6 +105,7 @@ cudaError_t launch_classH_split(const double* f, const double* B, const double* 
 long classH_sliced_work(const Dims& d, int scheme);
 long classH_partial_rows(const Dims& d, int scheme, bool split);
 cudaError_t classH_sliced_reserve(const Dims& d, OzWork& oz);
+size_t classH_guard_size(const Dims& d, int scheme);
 cudaError_t launch_classH_sliced(const double* f, const double* B, const double* Ftil,
                                  const double* E0, double shift, int scheme, const Dims& d,
                                  ClassHWork& w, int* status, double* ecls, double* ncls,

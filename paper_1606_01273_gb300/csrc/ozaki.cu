@@ -417,14 +417,14 @@ __global__ void k_oz_rowmax(OzView v, int R, int K, bool split_k,
   }
 }
 
-// sigma_r = 2^(floor(log2 max|x_r|) + 1) (1 for a zero row, NaN for one with a NaN or an infinity,
+// sigma_r = 2^(floor(log2 max|x_r|) + 1) (0 for a zero row, NaN for one with a NaN or an infinity,
 // which every result of that row then is).
 __global__ void k_oz_scale(const unsigned long long* __restrict__ mx, int R,
                            double* __restrict__ scale) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   const double m = __longlong_as_double((long long)mx[r]);
-  scale[r] = m == 0.0 ? 1.0 : isfinite(m) ? ldexp(1.0, ilogb(m) + 1) : nan("");
+  scale[r] = m == 0.0 ? 0.0 : isfinite(m) ? ldexp(1.0, ilogb(m) + 1) : nan("");
 }
 
 // S slices of x / sigma_r into out[s][r][Kp] (zeros for K <= k < Kp); grid (Kp tiles,

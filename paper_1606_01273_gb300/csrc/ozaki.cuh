@@ -20,9 +20,11 @@
 namespace caspt2 {
 
 constexpr int kOzMaxSlices = 7;      // of the precision form
-// Slices that hold every operand to 2^-57 of its row's scale, the whole 2^56 fixed-point integer:
-// what is dropped (levels s + t >= 8, at most 2^-55 and typically 2^-58 of sigma_i tau_j a
-// term) is below the rounding of an FP64 dot product of the same terms.
+// Slices that hold every operand to 2^-57 of its row's scale, the whole 2^56 fixed-point integer.
+// What is dropped of a product (levels s + t >= 8) and rounded in the operands is at most
+// 1.13 2^-55 sigma_i tau_j a term: relative to the row scales, not to the term.  An FP64 dot
+// product errs by up to 2^-53 K sum_k |a_k b_k|, so eight slices match it where the large elements of
+// the two rows share their k and not in general (class_h.cu checks its sums).
 constexpr int kOzFp64Slices = 8;
 constexpr int kOzKChunk = 256;     // exact FP32 accumulation span
 constexpr int kOzKStage = 32;      // K per shared-memory stage
