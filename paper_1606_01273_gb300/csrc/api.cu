@@ -3,6 +3,7 @@
 // kernels of setup.cu and class_*.cu on the caller's stream.
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -13,6 +14,7 @@
 #include "class_ag.cuh"
 #include "cross.cuh"
 #include "class_dev.cuh"
+#include "footprint.h"
 #include "kernels.cuh"
 #include "linalg.cuh"
 #include "ozaki.cuh"
@@ -81,8 +83,10 @@ struct caspt2_ctx {
   // precision form: split BF16 tensor-core GEMMs, class-H pair integrals kept for the densities
   OzWork oz{};
   double *hK = nullptr, *hKK = nullptr, *hpack = nullptr;
-  double* hsl = nullptr;              // plain form: K chunk of launch_classH_sliced
-  long hslcap = 0;                    // its doubles, 0: the fused kernel serves
+  // plain form: K chunk of launch_classH_sliced and its doubles, 0: the fused kernel serves.
+  // With hw.guard and oz the workspace that a solve can do without (drop_sliced).
+  double* hsl = nullptr;
+  long hslcap = 0;
   // one-body couplings between classes: dbar2 off-diagonal blocks (opt.dens_offdiag)
   bool x_alloc = false;
   CrossWork xw{};
@@ -116,15 +120,68 @@ struct caspt2_ctx {
   KernelTimer tri{};
   GemmTimer* gemm = nullptr;          // FP64 GEMM launches of a solve (device time, flops)
 
+  // Counting only (context_bytes): alloc adds to `bytes` and hands out no memory.
+  bool dry = false;
+  size_t bytes = 0;
+
+  // Bytes that an allocation takes of the device: blocks of 2 MB, small ones side by side.
+  static size_t granular(size_t b) {
+    const size_t g = b >= (1u << 20) ? (2u << 20) : 512;
+    return (b + g - 1) / g * g;
+  }
+
+  // Without memory for it the sliced workspace is given up first.
   template <class T>
   int alloc(T** p, size_t count) {
     *p = nullptr;
     if (count == 0) count = 1;
+    bytes += granular(count * sizeof(T));
+    if (dry) {
+      *p = reinterpret_cast<T*>(512);
+      return CASPT2_OK;
+    }
     void* q = nullptr;
-    if (cudaMalloc(&q, count * sizeof(T)) != cudaSuccess) return CASPT2_ENOMEM;
+    cudaError_t e = cudaMalloc(&q, count * sizeof(T));
+    if (e != cudaSuccess && hslcap > 0) {
+      cudaGetLastError();
+      drop_sliced();
+      e = cudaMalloc(&q, count * sizeof(T));
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();              // later launches must not find it
+      return CASPT2_ENOMEM;
+    }
     allocs.push_back(q);
     *p = static_cast<T*>(q);
     return CASPT2_OK;
+  }
+
+  void reserve_sliced() {
+    const long cap = classH_sliced_work(d, opt.scheme);
+    if (cap <= 0) return;
+    const size_t ng = classH_guard_size(d, opt.scheme);
+    if (dry) {
+      bytes += granular(sizeof(double) * cap) + granular(sizeof(double) * ng) +
+               granular(oz_slice_bytes(d.c * d.v, d.X, kOzFp64Slices)) +
+               granular(sizeof(double) * d.c * d.v) + granular(sizeof(int));
+      return;
+    }
+    if (cudaMalloc(&hsl, sizeof(double) * cap) != cudaSuccess ||
+        cudaMalloc(&hw.guard, sizeof(double) * ng) != cudaSuccess ||
+        classH_sliced_reserve(d, oz) != cudaSuccess) {
+      cudaGetLastError();
+      drop_sliced();
+      return;
+    }
+    hslcap = cap;
+  }
+
+  void drop_sliced() {
+    if (hsl) cudaFree(hsl);
+    if (hw.guard) cudaFree(hw.guard);
+    hsl = hw.guard = nullptr;
+    hslcap = 0;
+    if (!oz.on) oz_release(oz);
   }
 };
 
@@ -183,6 +240,7 @@ void caspt2_destroy(caspt2_ctx* ctx) {
   int cur = 0;
   cudaGetDevice(&cur);
   cudaSetDevice(ctx->device);
+  ctx->drop_sliced();
   for (void* p : ctx->allocs) cudaFree(p);
   for (auto& e : ctx->ev)
     if (e) cudaEventDestroy(e);
@@ -204,6 +262,31 @@ void caspt2_destroy(caspt2_ctx* ctx) {
 }
 
 int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_options* opt) {
+  return create_context(out, dims, opt, true);
+}
+
+}  // extern "C"
+
+namespace {
+
+// Contraction plans of a class: built once, read by every context and every footprint.
+struct ClassPlans {
+  std::vector<ActPlan> S, F;
+  std::vector<SrcPlan> V;
+};
+const ClassPlans& class_plans(int k) {
+  static ClassPlans plans[7];
+  static std::once_flag once[7];
+  std::call_once(once[k], [k] {
+    build_act_plans(k, false, plans[k].S);
+    build_act_plans(k, true, plans[k].F);
+    build_src_plans(k, plans[k].V);
+  });
+  return plans[k];
+}
+
+int make_context(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_options* opt, bool sliced,
+                 bool dry) {
   if (!out || !dims) return CASPT2_EINVAL;
   *out = nullptr;
   const caspt2_dims& q = *dims;
@@ -228,7 +311,8 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
   if (!c) return CASPT2_ENOMEM;
   c->d = Dims{q.nclosed, q.nact, q.nvirt, q.naux, q.nstate};
   c->opt = o;
-  cudaGetDevice(&c->device);
+  c->dry = dry;
+  if (!dry) cudaGetDevice(&c->device);
   const Dims& d = c->d;
   const size_t nmo = d.nmo(), n = d.n, a = d.a, X = d.X;
   const size_t a2 = a * a, a4 = a2 * a2;
@@ -283,18 +367,6 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       ALLOC(c->hpack, (size_t)d.X * cv);
     }
   }
-  if (st == CASPT2_OK && o.precision == CASPT2_FP64 && (o.class_mask >> CASPT2_CLASS_H & 1u)) {
-    // without the memory for it the fused kernel serves
-    c->hslcap = classH_sliced_work(d, o.scheme);
-    if (c->hslcap > 0 &&
-        (c->alloc(&c->hsl, (size_t)c->hslcap) != CASPT2_OK ||
-         c->alloc(&c->hw.guard, classH_guard_size(d, o.scheme)) != CASPT2_OK ||
-         classH_sliced_reserve(d, c->oz) != cudaSuccess)) {
-      oz_release(c->oz);
-      cudaGetLastError();
-      c->hslcap = 0;
-    }
-  }
   ALLOC(c->lamNL, (size_t)CASPT2_NCLASS * n);
   ALLOC(c->lamLV, (size_t)CASPT2_NCLASS * n * n);
   // classes A-G: plans, class matrices, sources, sector work space, integral blocks
@@ -308,11 +380,9 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       class_setup(k, d, w);
       if (w.vsize == 0 || a == 0) continue;
       c->cw_on[k] = true;
-      std::vector<ActPlan> S, F;
-      std::vector<SrcPlan> V;
-      build_act_plans(k, false, S);
-      build_act_plans(k, true, F);
-      build_src_plans(k, V);
+      const ClassPlans& plans = class_plans(k);
+      const std::vector<ActPlan>&S = plans.S, &F = plans.F;
+      const std::vector<SrcPlan>& V = plans.V;
       for (auto& t : S) c->kmax = std::max<int>(c->kmax, t.rank);
       for (auto& t : F) c->kmax = std::max<int>(c->kmax, t.rank);
       for (auto& t : V) {
@@ -349,7 +419,7 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
         }
         if (nx > 0) ALLOC(w.dX, nx);
       }
-      if (st == CASPT2_OK && class_upload_plans(w, S, F) != cudaSuccess) st = CASPT2_ECUDA;
+      if (st == CASPT2_OK && !dry && class_upload_plans(w, S, F) != cudaSuccess) st = CASPT2_ECUDA;
       ALLOC(w.Sact, 2 * (size_t)w.m * w.m);
       ALLOC(w.Fact, 2 * (size_t)w.m * w.m);
       vmax = std::max(vmax, w.vsize);   // the sources live only during the class's solve
@@ -402,7 +472,7 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
       ALLOC(sb.mdn, (size_t)nmdn);
       ALLOC(sb.info, 2 * sb.jobs.size());
       ALLOC(sb.dev, sb.jobs.size());
-      if (st == CASPT2_OK && !sb.jobs.empty() &&
+      if (st == CASPT2_OK && !dry && !sb.jobs.empty() &&
           cudaMemcpy(sb.dev, sb.jobs.data(), sizeof(SectorJob) * sb.jobs.size(),
                      cudaMemcpyHostToDevice) != cudaSuccess)
         st = CASPT2_ECUDA;
@@ -455,9 +525,12 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
     }
   }
 #undef ALLOC
+  if (st == CASPT2_OK && sliced && o.precision == CASPT2_FP64 &&
+      (o.class_mask >> CASPT2_CLASS_H & 1u))
+    c->reserve_sliced();
   for (auto& e : c->ev)
-    if (st == CASPT2_OK && cudaEventCreate(&e) != cudaSuccess) st = CASPT2_ECUDA;
-  if (st == CASPT2_OK && (cudaEventCreate(&c->hw.ev_gemm0) != cudaSuccess ||
+    if (st == CASPT2_OK && !dry && cudaEventCreate(&e) != cudaSuccess) st = CASPT2_ECUDA;
+  if (st == CASPT2_OK && !dry && (cudaEventCreate(&c->hw.ev_gemm0) != cudaSuccess ||
                           cudaEventCreate(&c->hw.ev_gemm1) != cudaSuccess ||
                           cudaEventCreate(&c->tri.e0) != cudaSuccess ||
                           cudaEventCreate(&c->tri.e1) != cudaSuccess ||
@@ -481,6 +554,15 @@ int caspt2_create(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_option
   *out = c;
   return CASPT2_OK;
 }
+
+}  // namespace
+
+int caspt2::create_context(caspt2_ctx** out, const caspt2_dims* dims, const caspt2_options* opt,
+                           bool sliced) {
+  return make_context(out, dims, opt, sliced, false);
+}
+
+extern "C" {
 
 int caspt2_set_inputs(caspt2_ctx* c, int mem, const double* fock, const double* dfB,
                       const double* rdm1, const double* rdm2, const double* rdm3,
@@ -994,6 +1076,69 @@ int alloc_densities(caspt2_ctx* c) {
   return st;
 }
 
+// Workspace of the split products that a solve and (dens) caspt2_densities make, from above (every
+// sector keeps all its eigenvectors).
+size_t split_bytes(const caspt2_ctx* c, bool dens) {
+  if (!c->oz.on) return 0;
+  const Dims& d = c->d;
+  const long n = d.n, X = d.X, cv = (long)d.c * d.v;
+  const int dims3[3] = {d.c, d.a, d.v};
+  const bool exact = c->oz.S >= kOzMaxSlices;
+  OzNeed need{};
+  auto prod = [&](long M, long N, long K, bool same) {
+    OzNeed q{};
+    if (!oz_need(M, N, K, same, c->oz.S, q)) return;
+    need.slices = std::max(need.slices, q.slices);
+    need.scales = std::max(need.scales, q.scales);
+    need.part = std::max(need.part, q.part);
+  };
+  const bool h_on = (c->opt.class_mask >> CASPT2_CLASS_H & 1u) && cv > 0;
+  if (h_on) prod(cv, cv, X, true);
+  if (h_on && dens) {
+    prod(X, cv, cv, false);
+    prod(d.v, d.v, cv * d.c, false);
+    prod(d.c, d.c, cv * d.v, false);
+  }
+  if (exact && !c->eri_blk.empty()) prod(d.nmo(), d.nmo(), X * d.c, true);
+  for (auto& kv : c->eri_blk) {
+    const long n01 = (long)dims3[kv.first / 27] * dims3[(kv.first / 9) % 3];
+    const long n23 = (long)dims3[(kv.first / 3) % 3] * dims3[kv.first % 3];
+    prod(n01, n23, X, false);
+    if (!dens) continue;
+    prod(X, n01, n23, false);
+    prod(X, n23, n01, false);
+  }
+  for (int k = 0; k < 7; ++k) {
+    if (!c->cw_on[k]) continue;
+    const ClassWork& w = c->cw[k];
+    const long rows = all_tuples(w);
+    for (const SrcGemmGroup& G : w.hG) {
+      long K = 1;
+      for (int q = 0; q < G.g.ns; ++q) K *= d.a;
+      if (exact) prod(std::min(rows, c->sw.srcXcap / K), w.A * n * n, K, false);
+    }
+    for (const SectorKeep& S : w.keep) {
+      if (S.ntup == 0) continue;
+      const long m = S.msec;
+      if (exact && m > kSectorBlockMax) {
+        prod(m, m, m, false);
+        prod(128, m, m, false);        // panels of the blocked back-transformation
+        prod(m, m, 128, false);
+      }
+      const long chunk = std::max<long>(1, std::min<long>(S.ntup, c->sw.wcap / (m * n)));
+      if (exact) prod(m, chunk * n, m, false);
+      if (dens) prod(m, S.ntup * (S.Lsel < 0 ? n : 1), m, false);
+    }
+    if (!dens) continue;
+    prod(rows * n, w.m, w.m, false);
+    prod(w.m, w.m, rows * n, false);
+    for (int q = 0; q < w.dc.next; ++q)
+      if (w.ed.d[q] > 0) prod(w.ed.d[q], w.ed.d[q], rows / w.ed.d[q] * n * w.m, false);
+  }
+  return caspt2_ctx::granular(need.slices) + caspt2_ctx::granular(need.scales) +
+         caspt2_ctx::granular(need.part) + 512;
+}
+
 // The closed-active, active-virtual and closed-virtual blocks of d2 (dbar2 through the
 // one-body couplings between classes) for the classes of class_mask, added to c->dd2.
 int dens_offdiag(caspt2_ctx* c, unsigned class_mask, cudaStream_t s) {
@@ -1083,6 +1228,16 @@ long block_size(const Dims& d, int key) {
 }
 
 }  // namespace
+
+size_t caspt2::context_bytes(const caspt2_dims& dims, const caspt2_options& opt, bool densities,
+                             bool sliced) {
+  caspt2_ctx* c = nullptr;
+  if (make_context(&c, &dims, &opt, sliced, true) != CASPT2_OK) return 0;
+  if (densities && alloc_densities(c) != CASPT2_OK) c->bytes = 0;
+  const size_t b = c->bytes + split_bytes(c, densities);
+  delete c;
+  return b;
+}
 
 extern "C" {
 

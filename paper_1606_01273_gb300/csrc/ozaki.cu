@@ -606,16 +606,39 @@ cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc) {
   return cudaSuccess;
 }
 
+namespace {
+// Small products run as plain FP64: slicing, scaling and the split GEMM are at least six
+// launches (30 to 90 us for the products of a c5 a3 v70 solve), where the FP64 kernel needs
+// one and is exact to FP64 rounding.  2^25 multiply-adds take it about 60 us, provided its
+// blocks fill the chip (K is split over at most eight).
+bool oz_direct(long M, long N, long K) {
+  const double blocks = (double)((M + 31) / 32) * ((N + 31) / 32) * std::max(1L, std::min(8L, K / 32));
+  const double fmas = (double)M * N * K;
+  return fmas <= kOzDirectFmas && (blocks >= 152 || fmas <= kOzDirectFmas * blocks / 152.0);
+}
+// Parts of K over CTAs when the output has few tiles (about two waves of 152 SMs).
+int oz_nsplit(int M, int N, int Kp, bool same) {
+  const long tiles = oz_tiles((M + kOzM - 1) / kOzM, (N + kOzN - 1) / kOzN, same);
+  const int nchunk = (Kp + kOzKChunk - 1) / kOzKChunk;
+  return (int)std::max<long>(1, std::min<long>(nchunk, (304 + tiles - 1) / tiles));
+}
+}  // namespace
+
+bool oz_need(long M, long N, long K, bool same, int S, OzNeed& need) {
+  need = OzNeed{};
+  if (M <= 0 || N <= 0 || oz_direct(M, N, K)) return false;
+  const int k = (int)std::max(K, 1L);
+  need.slices = oz_slice_bytes((int)M, k, S) + (same ? 0 : oz_slice_bytes((int)N, k, S));
+  need.scales = sizeof(double) * (M + (same ? 0 : N));
+  const int ns = oz_nsplit((int)M, (int)N, oz_kpad(k), same);
+  need.part = ns > 1 ? sizeof(double) * ns * M * N : 0;
+  return true;
+}
+
 cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, int M, int N,
                       int K, double alpha, double beta, double* C, long ldc, cudaStream_t s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  // Small products run as plain FP64: slicing, scaling and the split GEMM are at least six
-  // launches (30 to 90 us for the products of a c5 a3 v70 solve), where the FP64 kernel needs
-  // one and is exact to FP64 rounding.  2^25 multiply-adds take it about 60 us, provided its
-  // blocks fill the chip (K is split over at most eight).
-  const long blocks = (long)((M + 31) / 32) * ((N + 31) / 32) * std::max(1, std::min(8, K / 32));
-  const double fmas = (double)M * N * K;
-  if (fmas <= kOzDirectFmas && (blocks >= 152 || fmas <= kOzDirectFmas * blocks / 152.0))
+  if (oz_direct(M, N, K))
     return dgemm_views(M, N, K, alpha, KView{A.X, A.rs, A.cs, A.kin, A.kout},
                        KView{B.X, B.rs, B.cs, B.kin, B.kout}, beta, C, ldc, s);
   const int Kp = oz_kpad(std::max(K, 1));
@@ -629,10 +652,7 @@ cudaError_t oz_matmul(OzWork& w, const OzView& A, const OzView& B, bool same, in
   double* sb = same ? w.sc : w.sc + M;
   if ((e = oz_split(A, M, K, Kp, w.S, as, sa, s)) != cudaSuccess) return e;
   if (!same && (e = oz_split(B, N, K, Kp, w.S, bs, sb, s)) != cudaSuccess) return e;
-  // split K over CTAs when the output has few tiles (about two waves of 152 SMs)
-  const long tiles = oz_tiles((M + kOzM - 1) / kOzM, (N + kOzN - 1) / kOzN, same);
-  const int nchunk = (Kp + kOzKChunk - 1) / kOzKChunk;
-  int nsplit = (int)std::max<long>(1, std::min<long>(nchunk, (304 + tiles - 1) / tiles));
+  const int nsplit = oz_nsplit(M, N, Kp, same);
   if (nsplit > 1) {
     const size_t need = (size_t)nsplit * M * N;
     if (need > w.part_n) {

@@ -65,6 +65,9 @@ struct OzWork {
   size_t part_n = 0;
 };
 void oz_release(OzWork& w);
+// Bytes of slices, scales and split-K partials of an M x N x K product; false: it runs in FP64.
+struct OzNeed { size_t slices, scales, part; };
+bool oz_need(long M, long N, long K, bool same, int S, OzNeed& need);
 // At least `bytes` of slices and nsc scales (and the error flag).
 cudaError_t oz_reserve(OzWork& w, size_t bytes, size_t nsc);
 

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/caspt2.h"
+#include "footprint.h"
 
 namespace {
 
@@ -31,10 +32,11 @@ double ms_since(Clock::time_point t0, Clock::time_point t1) {
   return std::chrono::duration<double, std::milli>(t1 - t0).count();
 }
 
-// Upper estimate of a request's device bytes: inputs, rotated RDMs, class-H pack, the
-// class matrices, sources, kept sector bases and (when requested) the density work
-// space, with a 25% margin and 64 MiB of fixed overhead.
-size_t estimate_bytes(const caspt2_request& q) {
+// Upper estimate of a request's device bytes and 64 MiB of fixed overhead: the larger of what its
+// context allocates (context_bytes) and of inputs, rotated RDMs, class-H pack, the class
+// matrices, sources, kept sector bases and (when requested) the density work space with a 25%
+// margin.  sliced: with the workspace that the plain form can do without.
+size_t estimate_bytes(const caspt2_request& q, bool sliced) {
   const double c = q.dims.nclosed, a = q.dims.nact, v = q.dims.nvirt, X = q.dims.naux,
                n = q.dims.nstate;
   const double nmo = c + a + v, a2 = a * a, a4 = a2 * a2;
@@ -54,7 +56,9 @@ size_t estimate_bytes(const caspt2_request& q) {
   const double cv = c * v;
   if (q.opt.precision == CASPT2_BF16X) w += 2 * cv * cv + X * cv + 4 * (cv + X) * 1024.0;
   if (q.densities) w += 6 * tall + X * nmo * nmo + 3 * cv * cv + 2 * X * cv;
-  return (size_t)(1.25 * 8.0 * w) + ((size_t)64 << 20);
+  const size_t b = caspt2::context_bytes(
+      q.dims, q.opt, q.densities && q.opt.target_state >= 0, sliced);
+  return std::max((size_t)(1.25 * 8.0 * w), b) + ((size_t)64 << 20);
 }
 
 struct Request {
@@ -62,6 +66,7 @@ struct Request {
   caspt2_request q{};
   std::vector<double> in[6];                  // fock, dfB, rdm1..4 (host copies)
   size_t est = 0;
+  bool sliced = true;
   Clock::time_point t_submit, t_admit, t_done;
   bool done = false;
   int status = CASPT2_OK;
@@ -77,16 +82,16 @@ struct PooledCtx {
   size_t est = 0;
 };
 
-std::vector<long long> shape_key(const caspt2_request& q) {
-  const caspt2_dims& d = q.dims;
-  const caspt2_options& o = q.opt;
+std::vector<long long> shape_key(const Request& r) {
+  const caspt2_dims& d = r.q.dims;
+  const caspt2_options& o = r.q.opt;
   long long sh, ov, en, dg;
   std::memcpy(&sh, &o.shift, 8);
   std::memcpy(&ov, &o.ovl_thresh, 8);
   std::memcpy(&en, &o.enuc, 8);
   std::memcpy(&dg, &o.degen_thresh, 8);
   return {d.nclosed, d.nact, d.nvirt, d.naux, d.nstate, o.xms, o.scheme, sh, ov, en,
-          o.target_state, (long long)o.class_mask, o.precision, o.slices, dg};
+          o.target_state, (long long)o.class_mask, o.precision, o.slices, dg, r.sliced};
 }
 
 }  // namespace
@@ -112,7 +117,7 @@ namespace {
 // here); returns the context for the pool, or nullptr after an error.
 caspt2_ctx* run_request(Request& r, cudaStream_t st, caspt2_ctx* ctx) {
   const caspt2_request& q = r.q;
-  int s = ctx ? CASPT2_OK : caspt2_create(&ctx, &q.dims, &q.opt);
+  int s = ctx ? CASPT2_OK : caspt2::create_context(&ctx, &q.dims, &q.opt, r.sliced);
   if (s == CASPT2_OK) {
     const double* p[6];
     for (int k = 0; k < 6; ++k) p[k] = r.in[k].empty() ? nullptr : r.in[k].data();
@@ -162,7 +167,7 @@ void worker(caspt2_server* srv) {
       auto admit = [&]() -> bool {
         if (srv->queue.empty()) return false;
         const std::shared_ptr<Request>& h = srv->queue.front();
-        const std::vector<long long> key = shape_key(h->q);
+        const std::vector<long long> key = shape_key(*h);
         for (auto it = srv->pool.begin(); it != srv->pool.end(); ++it)
           if (it->key == key) {
             ctx = it->ctx;
@@ -194,7 +199,7 @@ void worker(caspt2_server* srv) {
       std::lock_guard<std::mutex> lk(srv->m);
       if (ctx) {
         // keep the context idle for a later request of the same shape (its claim stays)
-        srv->pool.push_back(PooledCtx{shape_key(r->q), ctx, r->est});
+        srv->pool.push_back(PooledCtx{shape_key(*r), ctx, r->est});
         while (srv->pool.size() > srv->pool_max) {
           caspt2_destroy(srv->pool.front().ctx);
           srv->in_use -= srv->pool.front().est;
@@ -259,7 +264,11 @@ int caspt2_server_submit(caspt2_server* srv, const caspt2_request* q, long* tick
     return CASPT2_EINVAL;
   auto r = std::make_shared<Request>();
   r->q = *q;
-  r->est = estimate_bytes(*q);
+  r->est = estimate_bytes(*q, true);
+  if (r->est > srv->budget) {          // a budget for the context alone is enough
+    r->sliced = false;
+    r->est = estimate_bytes(*q, false);
+  }
   if (r->est > srv->budget) return CASPT2_EINVAL;
   const size_t n = d.nstate, a2 = (size_t)d.nact * d.nact;
   const size_t nmo = (size_t)d.nclosed + d.nact + d.nvirt;
