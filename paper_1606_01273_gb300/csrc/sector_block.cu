@@ -137,6 +137,62 @@ __device__ void tridiagonalise(double* A, int ld, int m, const Vecs& q) {
   __syncthreads();
 }
 
+// C[i * N + j] = sum_k A[i * ai + k * ak] B[k * bk + j * bj], two outputs a thread in flight.
+__device__ void block_mm(int M, int N, int K, const double* A, int ai, int ak, const double* B,
+                         int bk, int bj, double* C) {
+  const int total = M * N;
+  for (int o = threadIdx.x; o < total; o += 2 * kNT) {
+    const int o2 = o + kNT < total ? o + kNT : o;
+    const double *a0 = A + (o / N) * ai, *b0 = B + (o % N) * bj;
+    const double *a1 = A + (o2 / N) * ai, *b1 = B + (o2 % N) * bj;
+    double s0 = 0.0, s1 = 0.0;
+    for (int k = 0; k < K; ++k) {
+      s0 = fma(a0[k * ak], b0[k * bk], s0);
+      s1 = fma(a1[k * ak], b1[k * bk], s1);
+    }
+    C[o] = s0;
+    if (o2 != o) C[o2] = s1;
+  }
+}
+
+// Eigenvectors Z [m][nc] of T to the residual's second order: z_j += sum_i z_i (z_i . r_j) / (w_j -
+// w_i), r_j = T z_j - w_j z_j, as rotations of pairs (orthogonality stays).  The vectors of equal
+// eigenvalues come from independent starts; one that Gram-Schmidt leaves little of carries its
+// rounding that much enlarged, and the vectors orthogonalised against it with it (m = 80 with 32
+// equal eigenvalues: 1.8e-12, where a Jacobi sweep reaches 1e-15).  Pairs closer than 1e7 times the
+// residual stay as they are.  Without such a residual, the usual case, only r is formed.
+// scr: 3 m nc doubles.
+__device__ void polish(int m, int nc, double tn, const double* wk, double* Z, double* scr,
+                       const Vecs& q) {
+  const unsigned long long lim = abits(1e-14 * tn);
+  bool bad = false;
+  for (int t = threadIdx.x; t < m * nc; t += kNT) {
+    const int i = t / nc, j = t % nc;
+    double r = (q.d[i] - wk[j]) * Z[t];
+    if (i > 0) r = fma(q.e[i - 1], Z[t - nc], r);
+    if (i + 1 < m) r = fma(q.e[i], Z[t + nc], r);
+    scr[t] = r;
+    bad = bad || abits(r) > lim;
+  }
+  if (!__syncthreads_or(bad)) return;
+  double *E = scr + (long)m * nc, *dZ = E + (long)m * nc;
+  block_mm(nc, nc, m, Z, 1, nc, scr, nc, 1, E);
+  __syncthreads();
+  for (int t = threadIdx.x; t < nc * nc; t += kNT) {       // the pair (i < j) by one thread
+    const int i = t / nc, j = t % nc;
+    if (i > j) continue;
+    const double g = wk[j] - wk[i], e = 0.5 * (E[i * nc + j] + E[j * nc + i]);
+    const double c = i < j && fabs(e) < 1e-7 * g ? e / g : 0.0;
+    E[i * nc + j] = c;
+    E[j * nc + i] = -c;
+  }
+  __syncthreads();
+  block_mm(m, nc, nc, Z, nc, 1, E, nc, 1, dZ);
+  __syncthreads();
+  for (int t = threadIdx.x; t < m * nc; t += kNT) Z[t] += dZ[t];
+  __syncthreads();
+}
+
 // Eigenpairs of A (destroyed; stride ld): q.w holds all m eigenvalues ascending, Z [m][nc] the
 // vectors of the last nc, of which the last nk have eigenvalues >= wmin (eig_guard).  scr: 4 m
 // nc doubles and m nc bytes.  Returns nk, or -1 when the matrix holds a NaN or an infinity.
@@ -281,6 +337,7 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     }
     __syncthreads();
   }
+  polish(m, nc, tn, wk, Z, scr, q);
   for (int j = threadIdx.x; j < m; j += kNT) q.w[j] *= unscale;
   __syncthreads();
   // back-transformation Z <- H_0 ... H_{m-3} Z: lanes over 32 columns, the block's warps
@@ -318,24 +375,6 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
     __syncthreads();
   }
   return nk;
-}
-
-// C[i * N + j] = sum_k A[i * ai + k * ak] B[k * bk + j * bj], two outputs a thread in flight.
-__device__ void block_mm(int M, int N, int K, const double* A, int ai, int ak, const double* B,
-                         int bk, int bj, double* C) {
-  const int total = M * N;
-  for (int o = threadIdx.x; o < total; o += 2 * kNT) {
-    const int o2 = o + kNT < total ? o + kNT : o;
-    const double *a0 = A + (o / N) * ai, *b0 = B + (o % N) * bj;
-    const double *a1 = A + (o2 / N) * ai, *b1 = B + (o2 % N) * bj;
-    double s0 = 0.0, s1 = 0.0;
-    for (int k = 0; k < K; ++k) {
-      s0 = fma(a0[k * ak], b0[k * bk], s0);
-      s1 = fma(a1[k * ak], b1[k * bk], s1);
-    }
-    C[o] = s0;
-    if (o2 != o) C[o2] = s1;
-  }
 }
 
 // Shared memory of an m-row problem: A [m][m | 1], Z [m][m], the vectors.

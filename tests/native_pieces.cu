@@ -46,13 +46,15 @@ int np_root(const double* x, long n, double* r, double* ir) {
   return CASPT2_OK;
 }
 
-// Eigenvalues w [m] and the vectors V [m][*nk] of those at or above wmin.
-int np_eig_above(const double* A, int m, double wmin, double* w, double* V, int* nk) {
+// Eigenvalues w [m] and the vectors V [m][*nk] of those at or above wmin; block: in the one-block
+// solver, else by the library's choice.
+int np_eig_above(const double* A, int m, double wmin, double* w, double* V, int* nk, int block) {
   const size_t mm = (size_t)m * m;
   Dev dA(mm), dw(m), dV(mm), work(caspt2::sym_eig_work(m));
   if (!dA.p || !dw.p || !dV.p || !work.p) return CASPT2_ENOMEM;
   CASPT2_CUDA_TRY(cudaMemcpy(dA.p, A, mm * sizeof(double), cudaMemcpyHostToDevice));
-  const int st = caspt2::sym_eig_above(dA.p, m, wmin, dw.p, dV.p, nk, work.p, nullptr);
+  const int st = block ? caspt2::sym_eig_block(dA.p, m, dw.p, dV.p, work.p, nullptr, wmin, nk)
+                       : caspt2::sym_eig_above(dA.p, m, wmin, dw.p, dV.p, nk, work.p, nullptr);
   if (st != CASPT2_OK) return st;
   CASPT2_CUDA_TRY(cudaMemcpy(w, dw.p, m * sizeof(double), cudaMemcpyDeviceToHost));
   CASPT2_CUDA_TRY(cudaMemcpy(V, dV.p, (size_t)m * *nk * sizeof(double), cudaMemcpyDeviceToHost));

@@ -29,11 +29,13 @@ def _p(x):
     return x.ctypes.data_as(C.c_void_p)
 
 
-def _eig(native, A, wmin=-1e300):
-    """Status, all eigenvalues, the vectors of those at or above wmin."""
+def _eig(native, A, wmin=-1e300, block=None):
+    """Status, all eigenvalues, the vectors of those at or above wmin; up to 96 rows in the
+    one-block solver unless said otherwise."""
     A, m = np.ascontiguousarray(A), A.shape[0]
     w, V, nk = np.zeros(m), np.zeros(m * m), C.c_int()
-    st = native.np_eig_above(_p(A), m, C.c_double(wmin), _p(w), _p(V), C.byref(nk))
+    st = native.np_eig_above(_p(A), m, C.c_double(wmin), _p(w), _p(V), C.byref(nk),
+                             int(m <= 96 if block is None else block))
     return st, w, V[:m * nk.value].reshape(m, nk.value)
 
 
@@ -81,6 +83,53 @@ def test_small_matrix_scaled_by_a_power_of_two(native, m, power):
     assert a[0] == b[0] == 0
     assert np.array_equal(a[1] * f, b[1])
     assert np.array_equal(a[2], b[2])
+
+
+def _repeated(kind, m, rng):
+    """Eigenvalues with many equal ones: a projector's null space, two values, three clusters of
+    different sizes, and one beside a close pair."""
+    if kind == "rank":
+        w = np.concatenate([np.zeros(m - m * 3 // 5), rng.uniform(0.1, 4.0, m * 3 // 5)])
+    elif kind == "two":
+        w = np.where(np.arange(m) % 2, 1.0, -0.5)
+    elif kind == "three":
+        w = np.repeat([0.3, 0.7, 2.0], [m // 4, m // 4, m - 2 * (m // 4)])
+    else:
+        w = np.concatenate([np.full(m - 3, 1.0), [1.0 + 1e-6, 3.0, 3.5]])
+    Q = np.linalg.qr(rng.standard_normal((m, m)))[0]
+    A = (Q * w) @ Q.T
+    return 0.5 * (A + A.T)
+
+
+@pytest.mark.parametrize("m", [8, 16, 31, 32, 60, 80, 96])
+@pytest.mark.parametrize("kind", ["rank", "two", "three", "close"])
+def test_equal_eigenvalues(native, m, kind):
+    """Residual and orthogonality to 20 m eps of the norm, where the vectors of equal eigenvalues
+    come from independent starts; ten matrices each."""
+    for seed in range(10):
+        A = _repeated(kind, m, np.random.default_rng(seed))
+        st, w, V = _eig(native, A)
+        norm = np.abs(w).max()
+        assert st == 0
+        assert np.abs(V.T @ V - np.eye(m)).max() <= 20 * m * EPS
+        assert np.abs(A @ V - V * w).max() <= 20 * m * EPS * norm, seed
+
+
+@pytest.mark.parametrize("m", [1, 5, 32, 96])
+def test_diagonal_and_decoupled(native, m):
+    """No coupling at all, equal elements among them, and two equal blocks."""
+    rng = np.random.default_rng(m)
+    d = np.round(rng.uniform(-2, 2, m), 1)
+    st, w, V = _eig(native, np.diag(d))
+    assert st == 0
+    assert np.abs(w - np.sort(d)).max() <= 4 * EPS * np.abs(d).max()
+    assert np.abs(np.diag(d) @ V - V * w).max() <= 20 * EPS * np.abs(d).max()
+    if m % 2 == 0:
+        A = np.kron(np.eye(2), _spd(m // 2, 1))
+        st, w, V = _eig(native, A)
+        assert st == 0
+        assert np.abs(V.T @ V - np.eye(m)).max() <= 20 * m * EPS
+        assert np.abs(A @ V - V * w).max() <= 20 * m * EPS * np.abs(w).max()
 
 
 def _arguments():
