@@ -686,9 +686,11 @@ int sliced_chunks(const Dims& d, long kcap) {
 }
 }  // namespace
 
-// Doubles of the K workspace, or 0 where the fused kernel serves: up to 2^26 multiply-adds of
-// the full product it takes less than the dozen launches here (c4 v20 X84: 0.17 ms).  The
-// workspace is one chunk of rows, 128 MB unless a single closed orbital needs more.
+// Doubles of the K workspace, or 0 where the fused kernel serves: up to 2^26 multiply-adds of the
+// full product, where it takes 0.16 (c4 v20 X84), 0.34 (c4 v64 X256) and 0.6 ms (c4 v128 X256) of a
+// pass of 4 ms or more and needs neither workspace nor a bound on its error; slices would take
+// 0.11, 0.13 and 0.14.  Just above the line 0.70 against 0.15 (c6 v90 X300).  The workspace is one
+// chunk of rows, 128 MB unless a single closed orbital needs more.
 long classH_sliced_work(const Dims& d, int scheme) {
   const double cv = (double)d.c * d.v, fmas = cv * cv * d.X;
   if (fmas <= 67108864.0 || d.X > (1 << 17) || cv > 1e9) return 0;
@@ -768,8 +770,8 @@ void launch_guard(int G, const double* K, long ld, long off, const ClassHWork& w
 // its place and the sums.  Where k_guard_decide finds that the slices may cost a returned sum
 // more than FP64 products do, the fused kernel forms the sums instead (its launches return at once
 // otherwise, so the host need not wait for the decision).
-// c30 v300 X990, a pass with inputs: 77.7 ms fused (the FMAs alone take 69), 7.9 here: GEMMs 4.9,
-// sums 1.2, numerators 0.3, guard 0.25, slicing 0.15; the energies' error against 64 bits
+// c30 v300 X990, a pass with inputs: 77.7 ms fused (the FMAs alone take 69), 7.9 here: GEMMs 5.0,
+// sums 1.2, numerators 0.3, guard 0.25, slicing 0.15, inputs 0.3; the energies' error against 64 bits
 // 2.7e-16.
 cudaError_t launch_classH_sliced(const double* f, const double* B, const double* Ftil,
                                  const double* E0, double shift, int scheme, const Dims& d,

@@ -88,8 +88,6 @@ __device__ bool grid_sync_bounded(unsigned* count, volatile unsigned* gen, int* 
 // panel entries are contiguous); p [m]; pr [2][m]; part [grid][2 nb + 1]; sync[0..1] barrier,
 // [2] error.  Dynamic shared memory: v [m].
 constexpr int kLatrdPanel = 64;
-constexpr int kLatrdMin = 1024;     // sizes at which the blocked reduction is used (when
-                                    // the rows do not fit in shared memory)
 __global__ void __launch_bounds__(512, 2)
 k_latrd(double* __restrict__ A, int m, int k0, int b, double* __restrict__ vbuf,
         double* __restrict__ tau, double* __restrict__ d, double* __restrict__ e,
@@ -708,45 +706,9 @@ k_ortho_probe2(const double* __restrict__ Z, int m, int nc, const double* __rest
   }
 }
 
-// Back-transformation V = H_0 ... H_{m-3} Z with each block owning cb consecutive columns
-// (cb = 8 with 32 row groups of 256 threads): for every reflector (in reverse order) the block
-// forms r_c = v . Z[k+1.., c] for its columns over rg = blockDim / cb row groups and
-// applies Z[k+1+i][c] -= tau v_i r_c.  Columns are independent, so no grid-wide
-// synchronisation is needed.
-__global__ void __launch_bounds__(256)
-k_backtransform(const double* __restrict__ vbuf, const double* __restrict__ tau, int m, int nc, int cb,
-                double* __restrict__ Z) {
-  __shared__ double part[256];
-  __shared__ double rc[32];
-  const int rg = blockDim.x / cb;
-  const int cx = threadIdx.x % cb, ry = threadIdx.x / cb;
-  const bool act = ry < rg;
-  const int c = blockIdx.x * cb + cx;
-  for (int k = m - 3; k >= 0; --k) {
-    const int n1 = m - k - 1;
-    const double* v = vbuf + (long)k * m + k + 1;
-    double s = 0.0;
-    if (act && c < nc)
-      for (int i = ry; i < n1; i += rg) s += v[i] * Z[(long)(k + 1 + i) * nc + c];
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x < cb) {
-      double t = 0.0;
-      for (int q = 0; q < rg; ++q) t += part[q * cb + threadIdx.x];
-      rc[threadIdx.x] = t * tau[k];
-    }
-    __syncthreads();
-    if (act && c < nc) {
-      const double r = rc[cx];
-      for (int i = ry; i < n1; i += rg) Z[(long)(k + 1 + i) * nc + c] -= v[i] * r;
-    }
-    __syncthreads();
-  }
-}
-
-// Same back-transformation with the block's cb columns of Z resident in shared memory
-// (column-major, zs[c][i]) for the whole reflector loop and one warp per column: the warp
-// forms v . z_c with a shuffle reduction and updates its column, so the block synchronises
+// Back-transformation V = H_0 ... H_{m-3} Z with each block owning cb consecutive columns of Z,
+// resident in shared memory (column-major, zs[c][i]) for the whole reflector loop, and one warp
+// per column: the warp forms v . z_c with a shuffle reduction and updates its column, so the block synchronises
 // once per reflector, when the next reflector (double-buffered in shared memory by
 // 8-byte cp.async copies) has landed.  Z is read and written once.
 __global__ void __launch_bounds__(512)
@@ -1179,22 +1141,15 @@ int sym_eig_tridiag(double* A, int m, double* w, double* V, double* work, cudaSt
     const int st = backtransform_wy(vbuf, tau, m, nk, V, Z, 7 * mm, s, oz);
     if (st != CASPT2_OK) return st;
   } else if (m >= 3) {
+    // columns resident in shared memory: ceil(m / SMs) per block (one block per SM, the FP64
+    // work spread evenly, one warp per column); below kWyMinSize rows 23 and more of them fit
+    const int cbs = std::min(16, (nk + nsm - 1) / nsm);
+    CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_backtransform_smem,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kBackSmemMax));
     ++launch_counter();
-    // columns resident in shared memory: ceil(m / SMs) per block (one block per SM, the
-    // FP64 work spread evenly, one warp per column), fewer per block when they do not fit
-    const long fit = (long)(kBackSmemMax / (8ull * m)) - 2;      // minus the v buffers
-    const int cbs = (int)std::min<long>(std::min<long>(16, (nk + nsm - 1) / nsm), fit);
-    if (cbs >= 1) {
-      CASPT2_CUDA_TRY(cudaFuncSetAttribute(k_backtransform_smem,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kBackSmemMax));
-      k_backtransform_smem<<<(nk + cbs - 1) / cbs, 32 * cbs,
-                             sizeof(double) * (size_t)m * (cbs + 2), s>>>(vbuf, tau, m, nk, cbs,
-                                                                          V);
-    } else {
-      const int cb = 8;     // 8 columns x 32 row groups per block
-      k_backtransform<<<(nk + cb - 1) / cb, 256, 0, s>>>(vbuf, tau, m, nk, cb, V);
-    }
+    k_backtransform_smem<<<(nk + cbs - 1) / cbs, 32 * cbs,
+                           sizeof(double) * (size_t)m * (cbs + 2), s>>>(vbuf, tau, m, nk, cbs, V);
   }
   CASPT2_CUDA_TRY(cudaGetLastError());
   return CASPT2_OK;

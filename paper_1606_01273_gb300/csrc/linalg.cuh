@@ -74,9 +74,10 @@ int sym_eig_block(const double* A, int m, double* w, double* V, double* work, cu
                   double wmin = -1e300, int* nkept = nullptr);
 
 // Eigenpairs of A (destroyed): w[m] ascending, V[m][m] eigenvectors as columns.  One block for
-// up to kSectorBlockMax rows, where the whole solve is a chain of FP64 latencies and its
-// launches and host round trips would cost more (m = 96: 0.8 ms against 1.9 ms for the
-// stages as launches); the whole GPU above.
+// up to kSectorBlockMax rows, the whole GPU above.  A single matrix takes one block 0.4 ms at 33 rows,
+// 1.0 at 64 and 2.0 at 96, the large path 0.34, 0.64 and 0.86; the line stays at the size of
+// the sectors' solver because that leaves residuals of 1e-14 of the norm for repeated
+// eigenvalues too (polish), the large path up to 1e-9.
 int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
             KernelTimer* tm = nullptr, OzWork* oz = nullptr);
 inline size_t sym_eig_work(int m) {

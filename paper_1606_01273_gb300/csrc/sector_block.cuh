@@ -4,7 +4,10 @@
 
 namespace caspt2 {
 
-// Largest sector of the one-block solver: two m x m matrices in shared memory.
+// Largest sector of the one-block solver.  Two m x m matrices in shared memory would allow 118 rows.
+// An eigenproblem takes one block 1.5 ms at 80 rows, 2.0 at 96 and 2.7 at 112, alone on the large
+// path 0.75, 0.86 and 1.07; but the sectors of a solve (11, under SS-SR 11 n) run side by side
+// here and one after the other there.
 constexpr int kSectorBlockMax = 96;
 
 // One sector: class matrices S, F [2][m][m] (identity and pair-swap parts), the sign of the
