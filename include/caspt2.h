@@ -270,8 +270,9 @@ int caspt2_get_densities(caspt2_ctx* ctx, int mem, double* d1, double* d2, doubl
  *   grad_B[Q][p][q]  = dE_P/dB_Qpq at fixed f;
  * both symmetrised, in the layouts of the inputs, to host or device buffers (mem).  MS
  * only (opt.xms = 0): the XMS rotation response is not formed.  The closed-active,
- * active-virtual and closed-virtual entries of grad_f are left zero: an f with those
- * blocks is refused, and their derivative is d-bar(2) of those blocks (caspt2_densities
+ * active-virtual and closed-virtual entries of grad_f hold d1, the derivative through
+ * h = f - g(B, d_sa) alone: an f with those blocks is refused, and what they would add
+ * through the couplings between classes is d-bar(2) of those blocks (caspt2_densities
  * with opt.dens_offdiag).  Recomputes the densities of all solved classes.
  * Errors: EINVAL (xms, target_state < 0), ESTATE (no solve), ENOMEM, ECUDA. */
 int caspt2_gradient(caspt2_ctx* ctx, int mem, double* grad_f, double* grad_B, void* cuda_stream);

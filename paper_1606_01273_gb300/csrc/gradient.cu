@@ -11,7 +11,7 @@
 //   B      through the (pq|rt) blocks and class H (Gamma), H^ref at fixed h (core energy,
 //          g(d_core) and the active 2-electron term), and h.
 // Hence
-//   dE/df = gamma_P + d1 + d2 on those blocks
+//   dE/df = gamma_P + d1 + d2 on those blocks, d1 (the part through h) on the others
 //   dE/dB_Qpq = Gamma_Qpq + ref_Qpq - [D_pq Gd_Q + dsa_pq GD_Q - (M_Q + M_Q^T)_pq / 2],
 //   D = gamma_P + d1, Gd_Q = sum B_Q dsa, GD_Q = sum B_Q D, M_Q = D B_Q dsa,
 // ref_Qpq the derivative of <P|H|P> at fixed h:
@@ -49,7 +49,7 @@ __global__ void k_target_rdms(const double* __restrict__ rdm1, const double* __r
 }
 
 // D = gamma_P + d1 (full nmo x nmo), dsa (closed 2, active d_act) and
-// grad_f = gamma_P + d1 + d2 on the blocks of f the solve takes.
+// grad_f = gamma_P + d1 + d2 on the blocks of f the solve takes, d1 on the others.
 __global__ void k_grad_f(const double* __restrict__ d1, const double* __restrict__ d2,
                          const double* __restrict__ g1, const double* __restrict__ dact, int c,
                          int a, int nmo, double* __restrict__ D, double* __restrict__ dsa,
