@@ -252,7 +252,18 @@ __device__ __forceinline__ double hash_unit(unsigned a, unsigned b) {
   return (double)(h & 0xFFFFFF) / 16777216.0 + 0.5;   // in [0.5, 1.5)
 }
 
-// Unit eigenvector j of nc for the eigenvalue lam by three inverse iterations from a fixed
+// Shift of the inverse iteration for eigenvalue j of the nc ascending ones: equal eigenvalues are
+// offset by 64 roundings of the norm.  At the eigenvalue itself the factorisation singles out one
+// direction of their space, the same for all of them, and the Gram-Schmidt that follows would be
+// left with rounding; at the offset every direction grows alike and the starts stay independent.
+__device__ __forceinline__ double inverse_shift(const double* __restrict__ w, int nc, int j,
+                                                double tnorm) {
+  const double near = 1e-12 * tnorm, x = w[j];
+  const bool close = (j > 0 && x - w[j - 1] <= near) || (j + 1 < nc && w[j + 1] - x <= near);
+  return close ? x + 64 * 2.2e-16 * tnorm : x;
+}
+
+// Unit eigenvector j of nc for the shift lam by three inverse iterations from a fixed
 // start vector, on the pivoted factorisation T - lam = P L U (U with two superdiagonals; a
 // pivot below eps ||T|| is raised to it).  One thread a vector; scr holds [i][j] arrays (4 m nc
 // doubles and m nc bytes), so that threads access consecutive addresses; Z[i * nc + j].  The

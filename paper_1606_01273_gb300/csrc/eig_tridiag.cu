@@ -528,7 +528,8 @@ __global__ void k_inviter(const double* __restrict__ dg, const double* __restric
   }
   __syncthreads();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < nc) inverse_iteration(sde, sde + m, m, w[j], tnorm, nc, j, scr, Z);
+  if (j < nc)
+    inverse_iteration(sde, sde + m, m, inverse_shift(w, nc, j, tnorm), tnorm, nc, j, scr, Z);
 }
 
 // Orthonormalise each cluster of close eigenvalues (w sorted): the block of the cluster's

@@ -76,8 +76,8 @@ int sym_eig_block(const double* A, int m, double* w, double* V, double* work, cu
 // Eigenpairs of A (destroyed): w[m] ascending, V[m][m] eigenvectors as columns.  One block for
 // up to kSectorBlockMax rows, the whole GPU above.  A single matrix takes one block 0.4 ms at 33 rows,
 // 1.0 at 64 and 2.0 at 96, the large path 0.34, 0.64 and 0.86; the line stays at the size of
-// the sectors' solver because that leaves residuals of 1e-14 of the norm for repeated
-// eigenvalues too (polish), the large path up to 1e-9.
+// the sectors' solver, which leaves residuals of 1e-14 of the norm and vectors orthogonal to
+// 1e-14 for repeated eigenvalues too (polish), the large path up to 1e-12 and 1e-13.
 int sym_eig(double* A, int m, double* w, double* V, double* work, cudaStream_t s,
             KernelTimer* tm = nullptr, OzWork* oz = nullptr);
 inline size_t sym_eig_work(int m) {

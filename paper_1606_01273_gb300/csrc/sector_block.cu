@@ -158,8 +158,8 @@ __device__ void block_mm(int M, int N, int K, const double* A, int ai, int ak, c
 // Eigenvectors Z [m][nc] of T to the residual's second order: z_j += sum_i z_i (z_i . r_j) / (w_j -
 // w_i), r_j = T z_j - w_j z_j, as rotations of pairs (orthogonality stays).  The vectors of equal
 // eigenvalues come from independent starts; one that Gram-Schmidt leaves little of carries its
-// rounding that much enlarged, and the vectors orthogonalised against it with it (m = 80 with 32
-// equal eigenvalues: 1.8e-12, where a Jacobi sweep reaches 1e-15).  Pairs closer than 1e7 times the
+// rounding that much enlarged, and the vectors orthogonalised against it with it (4e-13 at 64 rows
+// with 26 equal eigenvalues, where a Jacobi sweep reaches 1e-15).  Pairs closer than 1e7 times the
 // residual stay as they are.  Without such a residual, the usual case, only r is formed.
 // scr: 3 m nc doubles.
 __device__ void polish(int m, int nc, double tn, const double* wk, double* Z, double* scr,
@@ -282,7 +282,7 @@ __device__ int eig_block(double* A, int ld, int m, double wmin, double* Z, doubl
   }
   const double* wk = q.w + (m - nc);
   for (int j = threadIdx.x; j < nc; j += kNT)
-    inverse_iteration(q.d, q.e, m, wk[j], tn, nc, j, scr, Z);
+    inverse_iteration(q.d, q.e, m, inverse_shift(wk, nc, j, tn), tn, nc, j, scr, Z);
   __syncthreads();
   // Gram-Schmidt against all earlier vectors: twice for an eigenvalue closer than 1e-3 of the
   // norm to its predecessor, once for the others.  Those are orthogonal to rounding over the

@@ -115,6 +115,20 @@ def test_equal_eigenvalues(native, m, kind):
         assert np.abs(A @ V - V * w).max() <= 20 * m * EPS * norm, seed
 
 
+@pytest.mark.parametrize("m", [97, 128, 200, 300])
+@pytest.mark.parametrize("kind", ["rank", "two", "three", "close"])
+def test_equal_eigenvalues_large(native, m, kind):
+    """The same on the large path.  Of a unit start Gram-Schmidt leaves 1 / sqrt(k) in a space of k
+    equal eigenvalues and may leave a tenth of 1 / k of the worst: m eps (the reduction) times 10 k,
+    k up to 150, is 1e-10 of the norm; orthogonality is restored to 1e-13 afterwards."""
+    for seed in range(5):
+        A = _repeated(kind, m, np.random.default_rng(seed))
+        st, w, V = _eig(native, A)
+        assert st == 0
+        assert np.abs(V.T @ V - np.eye(m)).max() <= 1e-12
+        assert np.abs(A @ V - V * w).max() <= 1e-10 * np.abs(w).max(), seed
+
+
 @pytest.mark.parametrize("m", [1, 5, 32, 96])
 def test_diagonal_and_decoupled(native, m):
     """No coupling at all, equal elements among them, and two equal blocks."""
