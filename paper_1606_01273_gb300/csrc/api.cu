@@ -703,6 +703,9 @@ int solve_impl(caspt2_ctx* c, void* stream) {
   CASPT2_CUDA_TRY(cudaEventRecord(c->ev[1], s));
 
   // ---- stage 1: class H (direct)
+  // recorded again around the kernels; an empty closed range launches none
+  CASPT2_CUDA_TRY(cudaEventRecord(c->hw.ev_gemm0, s));
+  CASPT2_CUDA_TRY(cudaEventRecord(c->hw.ev_gemm1, s));
   if ((o.class_mask >> CASPT2_CLASS_H & 1u) && c->oz.on) {
     CASPT2_CUDA_TRY(launch_classH_split(c->f, c->B, c->Ftil, c->E0, o.shift, o.scheme, d, c->hw,
                                         c->status, c->ecls + (long)CASPT2_CLASS_H * n * n,
